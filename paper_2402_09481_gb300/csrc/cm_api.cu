@@ -9,6 +9,7 @@
 #include "cm.h"
 #include "cm_internal.h"
 #include "cm_ctx.h"
+#include "cm_gf2.h"
 #include "ntt25.cuh"
 
 namespace cm {
@@ -672,14 +673,113 @@ cm_status enqueue_blocks(cm_ctx *ctx, const std::vector<Block> &bl, const uint64
     return CM_OK;
 }
 
+// How one call runs: as binary polynomials (cm_gf2.cu) or as the block list of
+// the integer transforms.
+struct Route {
+    bool gf = false;
+    gf::Product prod;
+    gf::Ops ops;             // pointers filled in by enqueue_route
+    int kind;
+    uint64_t n;
+    std::vector<Block> bl;
+    uint64_t need = 0, tmp_off = 0, pre_off = 0;
+};
+
+// The operands of z_i = sum_t a_t b_(t+i) over x and y: a_t is x reversed
+// (Toeplitz) or x in order (zero past its end: the Circulant pad bit), b_k is y
+// from an offset, cyclically.
+static void gf_maps(int kind, uint64_t n, uint64_t m, gf::Ops *q) {
+    const bool t = kind == CM_TOEPLITZ;
+    const uint64_t K = kind == CM_CIRCULANT ? n + 1 : n;
+    q->a0.map = bitmap(nullptr, t ? kReverse : kIdentity, n, n, t ? n - 1 : 0);
+    q->b0.map = bitmap(nullptr, kModForward, K + m - 1, t ? n + m - 1 : K, t ? m : 0);
+}
+
+// A product whose K + m - 1 bits fit 2^25 is one pair of transforms; a longer
+// one is cut into input blocks and output windows of 2^25-bit transforms whose
+// products are summed before the window's inverse: one window with blocks as
+// long as fit beside it, or both in steps of 2^24 so that windows share the
+// seed's blocks.
+static void gf_shape(int kind, uint64_t n, uint64_t m, gf::Product *p, gf::Ops *q) {
+    const uint64_t K = kind == CM_CIRCULANT ? n + 1 : n, N = 1ull << gf::kMaxLg;
+    memset(q, 0, sizeof(*q));
+    q->na = q->nb = q->nz = 1;
+    p->nin = 1;
+    q->astep = K;
+    q->zstep = (m + 63) & ~63ull;
+    if (K + m - 1 <= N) {
+        p->lg = gf::kMinLg;
+        while ((1ull << p->lg) < K + m - 1) ++p->lg;
+    } else {
+        p->lg = gf::kMaxLg;
+        if (m <= N / 2) q->astep = q->bstep = N - m + 1;
+        else if (K <= N / 2) q->zstep = q->bstep = (N - K + 1) & ~63ull;
+        else q->astep = q->bstep = q->zstep = N / 2;
+        p->nin = (uint32_t)((K + q->astep - 1) / q->astep);
+        q->na = p->nin;
+        q->nz = (uint32_t)((m + q->zstep - 1) / q->zstep);
+        q->nb = q->na + q->nz - 1;
+    }
+    q->a0.lim = q->astep;
+    q->z0.m = m;
+}
+
+// Products longer than 2^23 take the binary form in a context with default
+// options (a context that names a field, a transform limit, a sum cap or single
+// transforms keeps the integer ones).  Measured, us a call, binary / integer:
+// 2^23 206 / 153, 2^24 216 / 307, 2^25 245 / 722, 2^26 517 / 2565, 2^28
+// 1812 / 10659: below 2^24 too few tiles to fill the GPU.
+constexpr int kGfMinLg = 24;
+
+static bool gf_applies(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m) {
+    const PlanOptions &o = ctx->popt;
+    if (o.fields != kFieldsAll || o.max_lg != 32 || o.max_sum || o.single) return false;
+    if (n > kMaxBits || m > kMaxBits) return false;
+    const uint64_t K = kind == CM_CIRCULANT ? n + 1 : n;
+    return K + m > (1ull << (kGfMinLg - 1)) + 1 && valid_args(kind, n, m);
+}
+
+static cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t budget, Route *r) {
+    r->kind = kind;
+    r->n = n;
+    if (gf_applies(ctx, kind, n, m)) {
+        gf_shape(kind, n, m, &r->prod, &r->ops);
+        gf_maps(kind, n, m, &r->ops);
+        r->pre_off = gf::product_scratch(r->prod, r->ops);
+        r->need = r->pre_off + kFlagBytes;
+        r->gf = r->need <= budget;
+        if (r->gf) return CM_OK;
+    }
+    if (!make_blocks(kind, n, m, ctx->popt, &r->bl)) return CM_EINVAL;
+    r->need = blocks_scratch(r->bl, &r->tmp_off, &r->pre_off);
+    return r->need > budget ? CM_ENOMEM : CM_OK;
+}
+
+static cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t *y, uint64_t *z, void *scratch,
+                               cudaStream_t st) {
+    uint8_t *sc = static_cast<uint8_t *>(scratch);
+    if (!r.gf) return enqueue_blocks(ctx, r.bl, x, y, z, sc, r.tmp_off, r.pre_off, st);
+    r.ops.a0.map.src = x;
+    r.ops.b0.map.src = y;
+    r.ops.z0.z = z;
+    r.ops.z0.status = ctx->d_status;
+    r.ops.z0.pre = nullptr;
+    if (r.kind == CM_DODIS) {
+        uint32_t *pre = reinterpret_cast<uint32_t *>(sc + r.pre_off);
+        cm_status s = enqueue_precondition(ctx, x, r.n, pre, st);
+        if (s != CM_OK) return s;
+        r.ops.z0.pre = pre;
+    }
+    return cuda_status(gf::launch_product(ctx, r.prod, r.ops, ctx->d_gf, scratch, st));
+}
+
 cm_status run_single(cm_ctx *ctx, int kind, const uint64_t *x, uint64_t n, const uint64_t *y,
                      uint64_t m, uint64_t *z, cudaStream_t st) {
     if (!ctx || !x || !y || !z) return CM_EINVAL;
-    std::vector<Block> bl;
-    if (!make_blocks(kind, n, m, ctx->popt, &bl)) return CM_EINVAL;
-    uint64_t tmp_off = 0, pre_off = 0;
-    const uint64_t need = blocks_scratch(bl, &tmp_off, &pre_off);
-    if (need > ctx->budget) return CM_ENOMEM;
+    Route r;
+    cm_status s = make_route(ctx, kind, n, m, ctx->budget, &r);
+    if (s != CM_OK) return s;
+    const uint64_t need = r.need;
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return CM_EDEVICE;
     void *scratch = nullptr;
@@ -690,7 +790,7 @@ cm_status run_single(cm_ctx *ctx, int kind, const uint64_t *x, uint64_t n, const
             return CM_ENOMEM;
         }
     }
-    cm_status s = enqueue_blocks(ctx, bl, x, y, z, static_cast<uint8_t *>(scratch), tmp_off, pre_off, st);
+    s = enqueue_route(ctx, r, x, y, z, scratch, st);
     if (scratch) {
         e = cudaFreeAsync(scratch, st);
         if (s == CM_OK && e != cudaSuccess) s = CM_EDEVICE;
@@ -887,6 +987,7 @@ extern "C" cm_status cm_create(cm_ctx **out, int device, const cm_options *opt) 
     if (cudaMalloc(&c->d_tables, h.size() * sizeof(uint64_t)) != cudaSuccess ||
         cudaMalloc(&c->d_tables30, h30.size() * sizeof(uint32_t)) != cudaSuccess ||
         cudaMalloc(&c->d_tables25, h25.size() * sizeof(uint32_t)) != cudaSuccess ||
+        cudaMalloc(&c->d_gf, gf::kTables * sizeof(gf::Pass)) != cudaSuccess ||
         cudaMalloc(&c->d_status, 64) != cudaSuccess) {
         cm_destroy(c);
         return CM_ENOMEM;
@@ -907,6 +1008,9 @@ extern "C" cm_status cm_create(cm_ctx **out, int device, const cm_options *opt) 
     c->rt30.big_lo_inv = c->rt30.big_hi_fwd + 32768;
     c->rt30.big_hi_inv = c->rt30.big_lo_inv + 32768;
     c->rt30.bits16 = c->rt30.big_hi_inv + 32768;
+    std::vector<gf::Pass> hg(gf::kTables);
+    gf::build_tables(hg.data());
+    cudaMemcpy(c->d_gf, hg.data(), hg.size() * sizeof(gf::Pass), cudaMemcpyHostToDevice);
     cudaMemset(c->d_status, 0, 64);
     c->rt.small = c->d_tables;
     c->rt.big_lo_fwd = c->d_tables + 8192;
@@ -934,6 +1038,7 @@ extern "C" void cm_destroy(cm_ctx *c) {
     if (c->d_tables) cudaFree(c->d_tables);
     if (c->d_tables30) cudaFree(c->d_tables30);
     if (c->d_tables25) cudaFree(c->d_tables25);
+    if (c->d_gf) cudaFree(c->d_gf);
     if (c->d_status) cudaFree(c->d_status);
     if (c->pool) cudaMemPoolDestroy(c->pool);
     delete c;
@@ -1121,15 +1226,15 @@ extern "C" cm_status cm_profile_read(cm_ctx *ctx, cm_profile_entry *out, uint32_
 extern "C" cm_status cm_extract_host(cm_ctx *ctx, int kind, const uint64_t *xh, uint64_t n,
                                      const uint64_t *yh, uint64_t m, uint64_t *zh, cm_stream stream) {
     if (!ctx || !xh || !yh || !zh) return CM_EINVAL;
-    std::vector<Block> bl;
-    if (!make_blocks(kind, n, m, ctx->popt, &bl)) return CM_EINVAL;
-    uint64_t tmp_off = 0, pre_off = 0;
-    const uint64_t sb = blocks_scratch(bl, &tmp_off, &pre_off);
-    const uint64_t sbr = (sb + 255) & ~255ull;
+    if (!valid_args(kind, n, m)) return CM_EINVAL;
     const uint64_t ybits = kind == CM_TOEPLITZ ? n + m - 1 : (kind == CM_CIRCULANT ? n + 1 : n);
     const uint64_t xw = words_of(n), yw = words_of(ybits), zw = words_of(m);
-    const uint64_t io = 8 * (xw + yw + zw) + 3 * 256;
-    if (sbr + io > ctx->budget) return CM_ENOMEM;
+    const uint64_t io = 8 * (xw + yw + zw) + 3 * 256 + 255;
+    if (io > ctx->budget) return CM_ENOMEM;
+    Route r;
+    cm_status s = make_route(ctx, kind, n, m, ctx->budget - io, &r);
+    if (s != CM_OK) return s;
+    const uint64_t sbr = (r.need + 255) & ~255ull;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return CM_EDEVICE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     void *buf = nullptr;
@@ -1141,16 +1246,15 @@ extern "C" cm_status cm_extract_host(cm_ctx *ctx, int kind, const uint64_t *xh, 
     uint64_t *xd = reinterpret_cast<uint64_t *>(b + sbr);
     uint64_t *yd = reinterpret_cast<uint64_t *>(reinterpret_cast<uint8_t *>(xd) + ((8 * xw + 255) & ~255ull));
     uint64_t *zd = reinterpret_cast<uint64_t *>(reinterpret_cast<uint8_t *>(yd) + ((8 * yw + 255) & ~255ull));
-    cm_status s = CM_OK;
     if (cudaMemcpyAsync(xd, xh, 8 * xw, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(yd, yh, 8 * yw, cudaMemcpyHostToDevice, st) != cudaSuccess)
         s = CM_EDEVICE;
     uint32_t pre_h[2] = {1, 1};
-    if (s == CM_OK) s = enqueue_blocks(ctx, bl, xd, yd, zd, b, tmp_off, pre_off, st);
+    if (s == CM_OK) s = enqueue_route(ctx, r, xd, yd, zd, b, st);
     if (s == CM_OK && cudaMemcpyAsync(zh, zd, 8 * zw, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         s = CM_EDEVICE;
     if (s == CM_OK && kind == CM_DODIS &&
-        cudaMemcpyAsync(pre_h, b + pre_off, sizeof(pre_h), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+        cudaMemcpyAsync(pre_h, b + r.pre_off, sizeof(pre_h), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         s = CM_EDEVICE;
     cudaFreeAsync(buf, st);
     if (cudaStreamSynchronize(st) != cudaSuccess) return CM_EDEVICE;

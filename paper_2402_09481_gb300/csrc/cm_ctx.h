@@ -11,6 +11,7 @@
 
 #include "cm.h"
 #include "cm_internal.h"
+#include "gf2_plan.h"
 #include "ntt_device.cuh"
 
 struct cm_server;  // continuous-batching request loop (cm_server.cu)
@@ -29,6 +30,7 @@ struct cm_ctx {
     cm::RootTables30 rt30{};
     uint32_t *d_tables25 = nullptr;
     cm::RootTables25 rt25{};
+    cm::gf::Pass *d_gf = nullptr;  // level tables of the binary-polynomial transforms
     cm_server *server = nullptr;
     // one-launch cluster kernel per length 2^14 .. 2^17: -1 not yet checked, 0 no, 1 yes
     std::atomic<int> cluster25[4] = {-1, -1, -1, -1};

@@ -1,0 +1,771 @@
+// Middle products as binary polynomials: additive transforms over a cross-
+// section of Frobenius orbits.
+//
+// z_i = sum_t a_t b_(t+i) (mod 2) is the transpose of multiplication by the
+// polynomial A(X) = sum a_t X^t over GF(2).  With E the map from 2^k
+// coefficients to the values at 2^k / w points of GF(2^w) (one point from each
+// Frobenius orbit; the values at the others are their squares, so the w bits
+// of each value are all there is), multiplication is E^-1 (E a . E p), and its
+// transpose E^T ((E a) . (E^-T b)): three transforms over k bits an operand,
+// where a number-theoretic transform carries 32- or 64-bit words for each bit.
+//
+// Points.  beta_i is the Cantor basis (D. Cantor 1989), s_i the polynomial that
+// vanishes on span(beta_0 .. beta_(i-1)); s_i(beta_(i+j)) = beta_j.  In the
+// basis X_j = prod s_i^(bit i of j) (Lin, Chung, Han 2014) level i takes
+// f = f0 + s_i f1 to its values on a coset and the next one: f0 + c f1 and
+// f0 + (c + 1) f1 with c = s_i there.  All points lie in beta_k + span(beta_i,
+// i < k).  Frobenius maps beta_i to beta_i + beta_(i-1), so the orbit of a point
+// meets the points whose beta_(k - 2^j) coordinates are 0 exactly once (the
+// cross-section of Li, Chen, Kuo, Cheng, Yang 2018, for a power-of-two set):
+// the "missing" levels i = k - 2^j keep one value of the two, f0 + c f1 with
+// c = x_j + u, which is an element of the field twice as large with x_j
+// coefficient f1.  The first levels so run on single bits, the last on 16- or
+// 32-bit elements; the data are 2^k bits throughout.
+//
+// Transposition.  Under <u, v> = coefficient of the top basis product in u v,
+// multiplications are self-adjoint, and E^-T on the bit-reversed b turns out to
+// be the same levels with c and c + 1 exchanged and u + 1 for u; E^T is its
+// inverse.  The conversion to the basis X_j is stages of XORs (von zur Gathen,
+// Gerhard 1996: division by s_(2^t) = X^(2^(2^t)) + X), transposed the same way.
+// Point bits run complemented in both operands, so that values meet in place.
+//
+// Passes, for arrays of packed bits in natural order (index bits 0..4 inside a
+// word):
+//   k_gf_rows   (k > 16) input bits -> conversion across rows of 2^16 bits
+//   k_gf_units  conversion of each row down to units of 256 bits
+//   k_gf_cols   (k > 18) levels k-1 .. lo on tiles of 2^13 words, both operands
+//   k_gf_mid    256-bit conversions, levels lo-1 .. 0, product, and back
+// and the inverses of the first three on the product.  Levels are bit-sliced
+// (gf2.cuh): a thread holds whole elements, one component a register, 32 of
+// them a word.
+#include <cuda_runtime.h>
+#include <stdint.h>
+#include <string.h>
+
+#include "cm_ctx.h"
+#include "cm_gf2.h"
+#include "cm_internal.h"
+
+namespace cm {
+namespace gf {
+
+namespace {
+
+// Values of positions k .. k + 31 of a map: two 32-bit loads and a funnel shift
+// when they are a run of source bits, else position by position.
+__device__ __forceinline__ uint32_t map_word(const BitMap &m, uint64_t k) {
+    if (k >= m.len) return 0u;
+    if (k + 32 <= m.len) {
+        uint64_t lo;
+        bool run = true;
+        if (m.mode == kIdentity) {
+            lo = k;
+        } else if (m.mode == kModForward) {
+            lo = k + m.off;
+            if (lo >= m.srclen) lo -= m.srclen;
+            if (lo >= m.srclen) lo -= m.srclen;
+            run = lo + 32 <= m.srclen;
+        } else {
+            lo = m.off - k - 31;
+            run = m.off - k < m.srclen && m.off >= k + 31;
+        }
+        if (run) {
+            const uint32_t *p = reinterpret_cast<const uint32_t *>(m.src) + (lo >> 5);
+            const uint32_t sh = (uint32_t)lo & 31u;
+            const uint32_t r = sh ? __funnelshift_r(__ldg(p), __ldg(p + 1), sh) : __ldg(p);
+            return m.mode == kReverse ? __brev(r) : r;
+        }
+    }
+    return m.get_run<32>(k);
+}
+
+// Word w of an operand block's array of 2^lg bits.
+__device__ __forceinline__ uint32_t in_word(const InOp &o, bool is_b, int lg, uint64_t w) {
+    if (is_b) return __brev(map_word(o.map, o.base + (1ull << lg) - 32 - 32 * w));
+    const uint64_t j = 32 * w;
+    if (j >= o.lim) return 0u;
+    uint32_t v = map_word(o.map, o.base + j);
+    if (o.lim - j < 32) v &= (1u << (uint32_t)(o.lim - j)) - 1u;
+    return v;
+}
+
+__device__ __forceinline__ InOp in_op(const Ops &q, uint32_t o) {
+    if (q.in) return q.in[o];
+    InOp r = o < q.na ? q.a0 : q.b0;
+    r.base += o < q.na ? q.astep * o : q.bstep * (o - q.na);
+    return r;
+}
+
+__device__ __forceinline__ OutOp out_op(const Ops &q, uint32_t o) {
+    if (q.out) return q.out[o];
+    OutOp r = q.z0;
+    const uint64_t done = q.zstep * o;
+    r.z += done >> 6;
+    r.m -= done;
+    if (o + 1 < q.nz && r.m > q.zstep) r.m = q.zstep;
+    return r;
+}
+
+// Word w of the product's array goes, reversed, to its place in z.
+__device__ __forceinline__ void out_word(const OutOp &o, bool bad, int lg, uint64_t w, uint32_t v) {
+    const uint64_t i = (1ull << (lg - 5)) - 1 - w;
+    if (i >= 2 * ((o.m + 63) >> 6)) return;
+    v = bad ? 0u : __brev(v);
+    const uint64_t at = 32 * i;
+    if (at >= o.m) v = 0u;
+    else if (o.m - at < 32) v &= (1u << (uint32_t)(o.m - at)) - 1u;
+    reinterpret_cast<uint32_t *>(o.z)[i] = v;
+}
+
+__device__ __forceinline__ bool constant_input(const OutOp &o, bool tell) {
+    const bool bad = o.pre && (o.pre[0] == 0u || o.pre[1] == 0u);
+    if (bad && tell) atomicOr(o.status, kFlagPrecond);
+    return bad;
+}
+
+// ---------------------------------------------------------------------------
+// Conversion across rows.  The stages "add row 2^j below, 2^j bits higher" of a
+// column stripe need the 2^r - 1 bits to its left, so a warp holds 32 columns
+// (words), lanes 16..31 its stripe and lanes 0..15 the words before it; rows sit
+// in registers, five row bits at a time, and the shifts are shuffles.  Left of
+// column 0 the stages are continued on the row's other end:
+//   kConvA     bits shifted past the row's end (hi) return as hi X to the start
+//              of their row and as hi to the next one;
+//   kConvBInv  the transpose: the words before column 0 are X end + (row above's
+//              end) of the input's end words;
+//   kConvB     its inverse: those words are found from the converted end, and
+//              their own inverse image starts the stripe.
+// A CTA has 512 rows of stripes (2^r rows each); the whole-row stages that
+// follow (kConvBInv: precede) run in shared memory.
+constexpr int kRowsThreads = 512;
+constexpr int kRowsSmem = 4 * 512 * (32 + 16);
+
+// Unit (stripe, row) of register i of warp w in a round over row bits b .. b + 4.
+template <int B>
+__device__ __forceinline__ uint32_t row_unit(uint32_t w, int i) {
+    return (w & ((1u << B) - 1u)) | ((uint32_t)i << B) | ((w >> B) << (B + 5));
+}
+
+// Stages of row bits HI - 1 .. LO (those below r) on registers that hold row
+// bits B .. B + 4.
+template <int B, int HI, int LO>
+__device__ __forceinline__ void row_shift_stages(uint32_t (&x)[32], uint32_t lane, int r) {
+#pragma unroll
+    for (int j = HI - 1; j >= LO; --j) {
+        if (j >= r) continue;
+        const int s = 1 << j, bit = 1 << (j - B);
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (!(i & bit)) {
+                const uint32_t y = x[i | bit];
+                if (s < 32) {
+                    uint32_t p = __shfl_up_sync(0xFFFFFFFFu, y, 1);
+                    if (lane == 0) p = 0;
+                    x[i] ^= __funnelshift_l(p, y, s);
+                } else {
+                    const uint32_t p = __shfl_up_sync(0xFFFFFFFFu, y, s >> 5);
+                    x[i] ^= lane >= (uint32_t)(s >> 5) ? p : 0u;
+                }
+            }
+    }
+}
+
+// All shift stages: x in the layout of the first round on entry, row bits 0..4
+// in registers on return.  xch: 512 x 32 words.  RC = max(r, 5).
+template <int RC>
+__device__ __forceinline__ void row_shifts(uint32_t (&x)[32], uint32_t *xch, uint32_t warp, uint32_t lane, int r) {
+    if constexpr (RC > 5) {
+        row_shift_stages<RC - 5, RC, RC - 5>(x, lane, r);
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) xch[row_unit<RC - 5>(warp, i) * 32 + lane] = x[i];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) x[i] = xch[row_unit<0>(warp, i) * 32 + lane];
+        row_shift_stages<0, RC - 5, 0>(x, lane, r);
+    } else {
+        row_shift_stages<0, 5, 0>(x, lane, r);
+    }
+}
+
+// The words before column 0 from the end words e[row][16].
+__device__ __forceinline__ uint32_t row_before(const uint32_t *e, uint32_t row, uint32_t c, uint32_t ld) {
+    uint32_t v = e[row * ld + c] << 1;
+    if (c) v |= e[row * ld + c - 1] >> 31;
+    if (row) v ^= e[(row - 1) * ld + c];
+    return v;
+}
+
+// Whole-row stages on sm[512][CW].
+template <int KIND, int CW>
+__device__ __forceinline__ void row_whole_stages(uint32_t *sm, const Stages &st) {
+    constexpr int LC = CW == 32 ? 5 : 4;
+    const uint32_t c = threadIdx.x & (CW - 1u), g = threadIdx.x >> LC;
+    constexpr uint32_t NG = kRowsThreads >> LC;
+    for (int n = 0; n < st.n; ++n) {
+        const int q = KIND == kConvBInv ? st.n - 1 - n : n;
+        const uint32_t top = st.top[q], H = 1u << top, s = 1u << st.sh[q];
+        auto bulk = [&]() {
+            __syncthreads();
+#pragma unroll
+            for (uint32_t i = 0; i < 256; i += NG) {
+                const uint32_t u = i + g, v = u & (H - 1u), row = v | ((u ^ v) << 1);
+                if (v >= s) sm[row * CW + c] ^= sm[(row + H - s) * CW + c];
+            }
+        };
+        auto wrapped = [&]() {
+            __syncthreads();
+            for (uint32_t u = g; u < (512u >> (top + 1)) * s; u += NG) {
+                const uint32_t row = ((u >> st.sh[q]) << (top + 1)) + (KIND == kConvA ? H : 0u) + (u & (s - 1u));
+                sm[row * CW + c] ^= sm[(row + H - s) * CW + c];
+            }
+        };
+        if (KIND == kConvBInv) {
+            bulk();
+            wrapped();
+        } else {
+            wrapped();
+            bulk();
+        }
+    }
+    __syncthreads();
+}
+
+template <int RC, bool INV>
+__global__ void __launch_bounds__(kRowsThreads, 2) k_gf_rows(const __grid_constant__ Ops q, int lg,
+                                                          const __grid_constant__ Stages st, uint32_t *__restrict__ data) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    uint32_t *xch = sm, *side = sm + 512 * 32;  // side: 2^r x 16 words about column 0
+    constexpr int B0 = RC - 5;                  // first round's lowest row bit
+    const int r = lg - 16, S = 9 - r;           // 2^S stripes a CTA (128 in all)
+    const uint32_t R = 1u << r, groups = S < 7 ? 128u >> S : 1u;
+    const uint32_t grp = blockIdx.x % groups, op = blockIdx.x / groups;
+    uint32_t *arr = data + ((uint64_t)op << (lg - 5));
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const bool first = grp == 0, is_b = op >= q.na;
+    uint32_t x[32];
+    if (!INV) {
+        const InOp in = in_op(q, op);
+        // phase 0: the row's end (its last words, then zeros a's shifts run into);
+        // phase 1: b's words before column 0; phase 2: the stripes
+        for (int phase = first ? 0 : 2; phase < 3; ++phase) {
+            if (phase == 1 && !is_b) continue;
+            __syncthreads();
+            for (int i = 0; i < 32; ++i) {
+                const uint32_t u = row_unit<B0>(warp, i), row = u & (R - 1u), stripe = (grp << S) + (u >> r);
+                uint32_t v = 0, col = ~0u;
+                if (phase == 2) {
+                    if (16 * stripe + lane >= 16 && stripe < 128) col = 16 * stripe + lane - 16;
+                    else if (is_b && stripe < 128) v = side[row * 16 + lane];
+                } else if (u < R) {
+                    if (phase == 1) v = lane >= 16 ? row_before(side, row, lane - 16, 16) : 0u;
+                    else if (is_b) col = 2016u + lane;
+                    else if (lane < 16) col = 2032u + lane;
+                }
+                if (col < 2048u) v = in_word(in, is_b, lg, (uint64_t)row * 2048u + col);
+                xch[u * 32 + lane] = v;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 32; ++i) x[i] = xch[row_unit<B0>(warp, i) * 32 + lane];
+            row_shifts<RC>(x, xch, warp, lane, r);
+            if (phase == 2) break;
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const uint32_t u = row_unit<0>(warp, i);
+                if (lane >= 16 && u < R) side[u * 16 + lane - 16] = x[i];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (lane >= 16) sm[row_unit<0>(warp, i) * 16 + lane - 16] = x[i];
+        __syncthreads();
+        const uint32_t c = threadIdx.x & 15u;
+        if (first && !is_b)
+            for (uint32_t u = threadIdx.x >> 4; u < R; u += 32) sm[u * 16 + c] ^= row_before(side, u, c, 16);
+        if (is_b) row_whole_stages<kConvB, 16>(sm, st);
+        else row_whole_stages<kConvA, 16>(sm, st);
+        for (uint32_t u = threadIdx.x >> 4; u < 512; u += 32) {
+            const uint32_t row = u & (R - 1u), stripe = (grp << S) + (u >> r);
+            if (stripe < 128) arr[(uint64_t)row * 2048u + stripe * 16u + c] = sm[u * 16 + c];
+        }
+    } else {
+        const OutOp out = out_op(q, op);
+        const bool bad = constant_input(out, first && threadIdx.x == 0);
+#pragma unroll 8
+        for (uint32_t u = warp; u < 512; u += 16) {
+            const uint32_t row = u & (R - 1u), stripe = ((grp << S) + (u >> r)) & 127u;
+            sm[u * 32 + lane] = arr[(uint64_t)row * 2048u + ((16u * stripe + lane - 16u) & 2047u)];
+        }
+        row_whole_stages<kConvBInv, 32>(sm, st);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) x[i] = sm[row_unit<B0>(warp, i) * 32 + lane];
+        if (first && lane < 16) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const uint32_t u = row_unit<B0>(warp, i);
+                if (u < R) x[i] = row_before(sm, u, lane, 32);
+            }
+        }
+        row_shifts<RC>(x, xch, warp, lane, r);
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (lane >= 16) sm[row_unit<0>(warp, i) * 16 + lane - 16] = x[i];
+        __syncthreads();
+        const uint32_t c = threadIdx.x & 15u;
+        for (uint32_t u = threadIdx.x >> 4; u < 512; u += 32) {
+            const uint32_t row = u & (R - 1u), stripe = (grp << S) + (u >> r);
+            if (stripe < 128) out_word(out, bad, lg, (uint64_t)row * 2048u + stripe * 16u + c, sm[u * 16 + c]);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Conversion of rows of 2^rb bits to 256-bit units: one CTA a row, one thread a
+// unit.  In place; for lg <= 16 the row is the whole operand, read from the
+// inputs or written to z.
+template <int KIND>
+__device__ void unit_stages(uint32_t (&x)[8], uint32_t *snap, uint32_t nu, int r, const Stages &st) {
+    const uint32_t t = threadIdx.x;
+    auto publish = [&]() {
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) snap[i * nu + t] = x[i];
+        __syncthreads();
+    };
+    auto whole = [&](int q) {
+        publish();
+        whole_stage<KIND>(t, st.top[q], st.sh[q], [&](uint32_t d) { unit_xor(x, snap, nu, t + d); });
+    };
+    if (KIND != kConvBInv) {
+        for (int j = r - 1; j >= 0; --j) {
+            publish();
+            bit_stage_n<KIND>(j, x, snap, nu, t);
+        }
+        for (int q = 0; q < st.n; ++q) whole(q);
+    } else {
+        for (int q = st.n - 1; q >= 0; --q) whole(q);
+        for (int j = 0; j < r; ++j) {
+            publish();
+            bit_stage_n<KIND>(j, x, snap, nu, t);
+        }
+    }
+}
+
+template <bool INV>
+__global__ void __launch_bounds__(256) k_gf_units(const __grid_constant__ Ops q, int lg,
+                                                  const __grid_constant__ Stages st, uint32_t *__restrict__ data) {
+    __shared__ uint32_t snap[2048];
+    const int rb = lg < 16 ? lg : 16;
+    const uint32_t nu = 1u << (rb - 8);  // blockDim.x
+    const uint64_t w0 = ((uint64_t)blockIdx.x << (rb - 5)) + 8 * threadIdx.x;
+    const uint32_t op = (uint32_t)(((uint64_t)blockIdx.x << rb) >> lg);
+    const bool is_b = op >= q.na;
+    uint32_t x[8];
+    if (!INV && lg <= 16) {
+        const InOp in = in_op(q, op);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = in_word(in, is_b, lg, 8 * threadIdx.x + i);
+    } else {
+        const uint4 u = *reinterpret_cast<const uint4 *>(data + w0), v = *reinterpret_cast<const uint4 *>(data + w0 + 4);
+        x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
+        x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
+    }
+    if (INV) unit_stages<kConvBInv>(x, snap, nu, rb - 8, st);
+    else if (is_b) unit_stages<kConvB>(x, snap, nu, rb - 8, st);
+    else unit_stages<kConvA>(x, snap, nu, rb - 8, st);
+    if (INV && lg <= 16) {
+        const OutOp out = out_op(q, op);
+        const bool bad = constant_input(out, threadIdx.x == 0);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) out_word(out, bad, lg, 8 * threadIdx.x + i, x[i]);
+    } else {
+        *reinterpret_cast<uint4 *>(data + w0) = make_uint4(x[0], x[1], x[2], x[3]);
+        *reinterpret_cast<uint4 *>(data + w0 + 4) = make_uint4(x[4], x[5], x[6], x[7]);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Level passes.
+
+__device__ __forceinline__ void load_pass(Pass *P, const Pass *__restrict__ g) {
+    uint32_t *d = reinterpret_cast<uint32_t *>(P);
+    const uint32_t *s = reinterpret_cast<const uint32_t *>(g);
+    for (uint32_t i = threadIdx.x; i < sizeof(Pass) / 4; i += blockDim.x) d[i] = __ldg(s + i);
+}
+
+// Levels lg - 1 .. lo: fields up to GF(2^16), twiddles that depend on the tile's
+// own bits only.  In place; grid: tiles of every array.
+constexpr int kColsThreads = 256;
+
+template <bool INV>
+__global__ void __launch_bounds__(kColsThreads) k_gf_cols(int lg, uint32_t na, const Pass *__restrict__ table,
+                                                          uint32_t *__restrict__ data) {
+    __shared__ __align__(16) uint32_t sm[8192];
+    __shared__ Pass P;
+    const uint32_t tile = blockIdx.x & ((1u << (lg - 18)) - 1u), op = blockIdx.x >> (lg - 18);
+    load_pass(&P, table);
+    __syncthreads();
+    uint32_t *arr = data + ((uint64_t)op << (lg - 5)) + tile_base(P, tile);
+    const uint32_t which = INV || op >= na;
+    for (uint32_t e = 4 * threadIdx.x; e < 8192; e += 4 * kColsThreads) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(arr + lut3(P.glut, e));
+        sm[phys(lut3(P.alut, e))] = v.x;
+        sm[phys(lut3(P.alut, e + 1))] = v.y;
+        sm[phys(lut3(P.alut, e + 2))] = v.z;
+        sm[phys(lut3(P.alut, e + 3))] = v.w;
+    }
+    __syncthreads();
+    for (uint32_t l = 0; l < P.nlev; ++l) {
+        const Lev &v = P.lev[INV ? P.nlev - 1 - l : l];
+        level<13, 9, 4, INV>(sm, v, v.base[which], false, threadIdx.x, kColsThreads);
+        __syncthreads();
+    }
+    for (uint32_t e = 4 * threadIdx.x; e < 8192; e += 4 * kColsThreads) {
+        uint4 v;
+        v.x = sm[phys(lut3(P.alut, e))];
+        v.y = sm[phys(lut3(P.alut, e + 1))];
+        v.z = sm[phys(lut3(P.alut, e + 2))];
+        v.w = sm[phys(lut3(P.alut, e + 3))];
+        *reinterpret_cast<uint4 *>(arr + lut3(P.glut, e)) = v;
+    }
+}
+
+// The word bits change places with five point bits: a warp transposes 32 x 32
+// bit blocks by shuffles (word l of a block in lane l), three instructions a
+// step: exchange, rotate to the other half, merge (bytes: permute).
+template <int NB>
+__device__ void transpose_bits(uint32_t *sm, const Pass &P, uint32_t warp, uint32_t nwarp) {
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t keep[3], rot[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const uint32_t m = b == 0 ? 0x55555555u : b == 1 ? 0x33333333u : 0x0F0F0F0Fu;
+        const bool up = (lane >> b) & 1u;
+        keep[b] = up ? ~m : m;
+        rot[b] = up ? 32u - (1u << b) : 1u << b;
+    }
+    const uint32_t sel3 = (lane & 8u) ? 0x3715u : 0x6240u, sel4 = (lane & 16u) ? 0x3276u : 0x5410u;
+    const uint32_t la = xpose_addr(P, 0, lane);
+#pragma unroll 4
+    for (uint32_t u = warp; u < (1u << (NB - 5)); u += nwarp) {
+        uint32_t *at = sm + phys(la | P.xlut[0][u & 15u] | P.xlut[1][u >> 4]);
+        uint32_t v = *at;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, v, 1 << b);
+            v = (v & keep[b]) | (__funnelshift_l(y, y, rot[b]) & ~keep[b]);
+        }
+        v = __byte_perm(v, __shfl_xor_sync(0xFFFFFFFFu, v, 8), sel3);
+        v = __byte_perm(v, __shfl_xor_sync(0xFFFFFFFFu, v, 16), sel4);
+        *at = v;
+    }
+}
+
+template <int NB, int KIND>
+__device__ void load_tile(uint32_t *sm, const Pass &P, const uint32_t *__restrict__ arr, uint32_t tid, uint32_t nt) {
+    for (uint32_t e = 8 * tid; e < (1u << NB); e += 8 * nt) {
+        const uint32_t *g = arr + lut3(P.glut, e);
+        const uint4 u = *reinterpret_cast<const uint4 *>(g), v = *reinterpret_cast<const uint4 *>(g + 4);
+        uint32_t x[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+        conv8<KIND>(x);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) sm[phys(lut3(P.alut, e + i))] = x[i];
+    }
+}
+
+template <int NB>
+__device__ void store_tile(const uint32_t *sm, const Pass &P, uint32_t *__restrict__ arr, uint32_t tid, uint32_t nt) {
+    for (uint32_t e = 8 * tid; e < (1u << NB); e += 8 * nt) {
+        uint32_t x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = sm[phys(lut3(P.alut, e + i))];
+        conv8<kConvBInv>(x);
+        uint32_t *g = arr + lut3(P.glut, e);
+        *reinterpret_cast<uint4 *>(g) = make_uint4(x[0], x[1], x[2], x[3]);
+        *reinterpret_cast<uint4 *>(g + 4) = make_uint4(x[4], x[5], x[6], x[7]);
+    }
+}
+
+template <int NB, int FMAX>
+struct MidShape {
+    static constexpr int NFREE = NB - FMAX;
+    // one thread a unit of the longest elements in each operand's tile
+    static constexpr int HALF = 1 << (NB - 1 - FMAX);
+    static constexpr int SMEM1 = 4 << NB;
+};
+
+template <int NB, int FMAX>
+__device__ void inverse_levels(uint32_t *sm, const Pass &P, const uint32_t *base, int nt) {
+    for (int l = (int)P.nlev - 1; l >= 0; --l) {
+        level<NB, NB - FMAX, FMAX, true>(sm, P.lev[l], base[l], l >= (int)P.npre, threadIdx.x, (uint32_t)nt);
+        __syncthreads();
+        if (l == (int)P.npre) {
+            transpose_bits<NB>(sm, P, threadIdx.x >> 5, (uint32_t)nt >> 5);
+            __syncthreads();
+        }
+    }
+}
+
+// One pair of tiles: both forward transforms (half the threads each), the
+// product, the inverse transform in place of b's tile.  The ALU pipe bounds it;
+// a thread holds one unit of 2 x 32 words.
+template <int NB, int FMAX>
+__global__ void __launch_bounds__(2 * MidShape<NB, FMAX>::HALF) k_gf_mid(int lg, const Pass *__restrict__ table,
+                                                                         const uint32_t *__restrict__ A,
+                                                                         uint32_t *__restrict__ B) {
+    using S = MidShape<NB, FMAX>;
+    constexpr int NT = 2 * S::HALF, W = 1 << FMAX;
+    extern __shared__ __align__(16) uint32_t sm[];
+    __shared__ Pass P;
+    __shared__ uint32_t base[2][kMaxLev];
+    const int lgt = lg - 5 - NB;
+    const uint32_t tile = blockIdx.x & ((1u << lgt) - 1u), pair = blockIdx.x >> lgt;
+    load_pass(&P, table);
+    __syncthreads();
+    const uint64_t off = ((uint64_t)pair << (lg - 5)) + tile_base(P, tile);
+    if (threadIdx.x < 2 * kMaxLev) {
+        const uint32_t l = threadIdx.x >> 1, o = threadIdx.x & 1u;
+        if (l < P.nlev) base[o][l] = ext_twiddle(P.lev[l], P.lev[l].base[o], tile);
+    }
+    const uint32_t op = threadIdx.x >= S::HALF, tid = threadIdx.x - op * S::HALF;
+    uint32_t *mine = sm + op * (1u << NB);
+    if (op) load_tile<NB, kConvB>(mine, P, B + off, tid, S::HALF);
+    else load_tile<NB, kConvA>(mine, P, A + off, tid, S::HALF);
+    __syncthreads();
+    for (uint32_t l = 0; l < P.nlev; ++l) {
+        if (l == P.npre) {
+            transpose_bits<NB>(sm, P, threadIdx.x >> 5, NT >> 5);
+            transpose_bits<NB>(sm + (1u << NB), P, threadIdx.x >> 5, NT >> 5);
+            __syncthreads();
+        }
+        level<NB, S::NFREE, FMAX, false>(mine, P.lev[l], base[op][l], l >= P.npre, tid, S::HALF);
+        __syncthreads();
+    }
+    uint32_t *sb = sm + (1u << NB);
+    for (uint32_t u = threadIdx.x; u < (1u << S::NFREE); u += NT) {
+        uint32_t a[W], b[W], o[W];
+        const uint32_t at = phys(u);
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            a[j] = sm[at + (j << S::NFREE)];
+            b[j] = sb[at + (j << S::NFREE)];
+        }
+        mul<FMAX>(a, b, o);
+#pragma unroll
+        for (int j = 0; j < W; ++j) sb[at + (j << S::NFREE)] = o[j];
+    }
+    __syncthreads();
+    inverse_levels<NB, FMAX>(sb, P, base[1], NT);
+    store_tile<NB>(sb, P, B + off, threadIdx.x, NT);
+}
+
+// Several blocks: the forward half alone, tile words to H in tile order ...
+__global__ void __launch_bounds__(128) k_gf_fwd(int lg, uint32_t na, const Pass *__restrict__ table,
+                                                const uint32_t *__restrict__ data, uint32_t *__restrict__ hat) {
+    __shared__ __align__(16) uint32_t sm[8192];
+    __shared__ Pass P;
+    __shared__ uint32_t base[kMaxLev];
+    const uint32_t tile = blockIdx.x & ((1u << (lg - 18)) - 1u), op = blockIdx.x >> (lg - 18);
+    const bool is_b = op >= na;
+    load_pass(&P, table);
+    __syncthreads();
+    if (threadIdx.x < P.nlev)
+        base[threadIdx.x] = ext_twiddle(P.lev[threadIdx.x], P.lev[threadIdx.x].base[is_b], tile);
+    const uint32_t *arr = data + ((uint64_t)op << (lg - 5)) + tile_base(P, tile);
+    if (is_b) load_tile<13, kConvB>(sm, P, arr, threadIdx.x, 128);
+    else load_tile<13, kConvA>(sm, P, arr, threadIdx.x, 128);
+    __syncthreads();
+    for (uint32_t l = 0; l < P.nlev; ++l) {
+        if (l == P.npre) {
+            transpose_bits<13>(sm, P, threadIdx.x >> 5, 4);
+            __syncthreads();
+        }
+        level<13, 8, 5, false>(sm, P.lev[l], base[l], l >= P.npre, threadIdx.x, 128);
+        __syncthreads();
+    }
+    uint4 *o = reinterpret_cast<uint4 *>(hat + ((uint64_t)op << (lg - 5)) + ((uint64_t)tile << 13));
+    for (uint32_t i = threadIdx.x; i < 2048; i += 128) o[i] = reinterpret_cast<const uint4 *>(sm)[i];
+}
+
+// ... and a window's sum of products with the inverse: window w adds a's block
+// i times b's block i + w over i < nin.  One thread a point word (32 elements).
+__global__ void __launch_bounds__(256) k_gf_sum(int lg, uint32_t na, uint32_t nin, const Pass *__restrict__ table,
+                                                const uint32_t *__restrict__ hat, uint32_t *__restrict__ out) {
+    __shared__ __align__(16) uint32_t sm[8192];
+    __shared__ Pass P;
+    __shared__ uint32_t base[kMaxLev];
+    const uint32_t tile = blockIdx.x & ((1u << (lg - 18)) - 1u), win = blockIdx.x >> (lg - 18);
+    load_pass(&P, table);
+    __syncthreads();
+    if (threadIdx.x < P.nlev)
+        base[threadIdx.x] = ext_twiddle(P.lev[threadIdx.x], P.lev[threadIdx.x].base[1], tile);
+    const uint32_t at = phys(threadIdx.x);
+    const uint32_t *ha = hat + ((uint64_t)tile << 13) + at;
+    const uint32_t *hb = ha + ((uint64_t)(na + win) << (lg - 5));
+    uint32_t acc[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) acc[j] = 0;
+    for (uint32_t i = 0; i < nin; ++i) {
+        uint32_t a[32], b[32], o[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            a[j] = __ldg(ha + (j << 8));
+            b[j] = __ldg(hb + (j << 8));
+        }
+        mul<5>(a, b, o);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) acc[j] ^= o[j];
+        ha += 1ull << (lg - 5);
+        hb += 1ull << (lg - 5);
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j) sm[at + (j << 8)] = acc[j];
+    __syncthreads();
+    inverse_levels<13, 5>(sm, P, base, 256);
+    store_tile<13>(sm, P, out + ((uint64_t)win << (lg - 5)) + tile_base(P, tile), threadIdx.x, 256);
+}
+
+void conv_stages(int base, int k, Stages *s) {
+    if (k <= 1) return;
+    int t = 0;
+    while ((2 << t) < k) ++t;  // the largest t with 2^t < k
+    const int q = 1 << t, r = k - q;
+    for (int j = r - 1; j >= 0; --j) {
+        s->top[s->n] = (uint8_t)(base + q + j);
+        s->sh[s->n++] = (uint8_t)(base + j);
+    }
+    conv_stages(base + q, r, s);
+    conv_stages(base, q, s);
+}
+
+Stages stages_of(int bits) {
+    Stages s;
+    memset(&s, 0, sizeof(s));
+    conv_stages(0, bits, &s);
+    return s;
+}
+
+struct Scope {  // tracing, when there is a context
+    alignas(ProfScope) unsigned char mem[sizeof(ProfScope)];
+    ProfScope *p = nullptr;
+    Scope(cm_ctx *c, const char *name, cudaStream_t st) {
+        if (c) p = new (mem) ProfScope(c, name, st);
+    }
+    ~Scope() {
+        if (p) p->~ProfScope();
+    }
+};
+
+template <int RC>
+cudaError_t rows_launch_r(bool inv, const Ops &q, int lg, uint32_t ops, uint32_t *data, cudaStream_t st) {
+    cudaError_t e = inv ? smem_attr_once<k_gf_rows<RC, true>>(kRowsSmem) : smem_attr_once<k_gf_rows<RC, false>>(kRowsSmem);
+    if (e != cudaSuccess) return e;
+    const int r = lg - 16;
+    const Stages s = stages_of(r);
+    const uint32_t grid = ops * (r > 2 ? 128u >> (9 - r) : 1u);
+    if (inv) k_gf_rows<RC, true><<<grid, kRowsThreads, kRowsSmem, st>>>(q, lg, s, data);
+    else k_gf_rows<RC, false><<<grid, kRowsThreads, kRowsSmem, st>>>(q, lg, s, data);
+    return cudaGetLastError();
+}
+
+cudaError_t rows_launch(cm_ctx *c, bool inv, const Ops &q, int lg, uint32_t ops, uint32_t *data, cudaStream_t st) {
+    Scope ps(c, inv ? "k_gf_rows_inv" : "k_gf_rows", st);
+    switch (lg - 16) {
+        case 6: return rows_launch_r<6>(inv, q, lg, ops, data, st);
+        case 7: return rows_launch_r<7>(inv, q, lg, ops, data, st);
+        case 8: return rows_launch_r<8>(inv, q, lg, ops, data, st);
+        case 9: return rows_launch_r<9>(inv, q, lg, ops, data, st);
+        default: return rows_launch_r<5>(inv, q, lg, ops, data, st);
+    }
+}
+
+cudaError_t units_launch(cm_ctx *c, bool inv, const Ops &q, int lg, uint32_t ops, uint32_t *data, cudaStream_t st) {
+    const int rb = lg < 16 ? lg : 16;
+    const Stages s = stages_of(rb - 8);
+    const uint32_t grid = ops << (lg - rb), nt = 1u << (rb - 8);
+    Scope ps(c, inv ? "k_gf_units_inv" : "k_gf_units", st);
+    if (inv) k_gf_units<true><<<grid, nt, 0, st>>>(q, lg, s, data);
+    else k_gf_units<false><<<grid, nt, 0, st>>>(q, lg, s, data);
+    return cudaGetLastError();
+}
+
+template <int NB, int FMAX>
+cudaError_t mid_launch(int lg, uint32_t pairs, const Pass *table, const uint32_t *A, uint32_t *B, cudaStream_t st) {
+    using S = MidShape<NB, FMAX>;
+    cudaError_t e = smem_attr_once<k_gf_mid<NB, FMAX>>(2 * S::SMEM1);
+    if (e != cudaSuccess) return e;
+    k_gf_mid<NB, FMAX><<<pairs << (lg - 5 - NB), 2 * S::HALF, 2 * S::SMEM1, st>>>(lg, table, A, B);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+void build_tables(Pass *t) {
+    for (int lg = kMinLg; lg <= kMaxLg; ++lg) {
+        Pass *p = t + 2 * (lg - kMinLg);
+        memset(p, 0, 2 * sizeof(Pass));
+        build_passes(lg, p, p + 1);
+    }
+}
+
+static bool summed(const Product &p, const Ops &q) { return p.nin > 1 || (!q.in && q.nz > 1); }
+
+uint64_t product_scratch(const Product &p, const Ops &q) {
+    const uint64_t arr = 1ull << (p.lg - 3);
+    return (q.na + q.nb) * arr * (summed(p, q) ? 2 : 1);
+}
+
+cudaError_t launch_product(cm_ctx *c, const Product &p, const Ops &q, const Pass *tables, void *scratch,
+                           cudaStream_t st) {
+    const Shape s = shape_of(p.lg);
+    const Pass *mid = tables + 2 * (p.lg - kMinLg), *col = mid + 1;
+    const bool sum = summed(p, q);
+    const uint32_t ops = q.na + q.nb;
+    uint32_t *data = static_cast<uint32_t *>(scratch);
+    uint32_t *B = data + ((uint64_t)q.na << (p.lg - 5));
+    cudaError_t e = cudaSuccess;
+    if (s.colr && (e = rows_launch(c, false, q, p.lg, ops, data, st)) != cudaSuccess) return e;
+    if ((e = units_launch(c, false, q, p.lg, ops, data, st)) != cudaSuccess) return e;
+    if (s.two) {
+        Scope ps(c, "k_gf_cols", st);
+        k_gf_cols<false><<<ops << (p.lg - 18), kColsThreads, 0, st>>>(p.lg, q.na, col, data);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    uint32_t *out = B;
+    if (sum) {
+        uint32_t *hat = data + ((uint64_t)ops << (p.lg - 5));
+        {
+            Scope ps(c, "k_gf_fwd", st);
+            k_gf_fwd<<<ops << (p.lg - 18), 128, 0, st>>>(p.lg, q.na, mid, data, hat);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+        out = data;  // the operands' arrays are free again: na + nb >= nz of them
+        Scope ps(c, "k_gf_sum", st);
+        k_gf_sum<<<q.nz << (p.lg - 18), 256, 0, st>>>(p.lg, q.na, p.nin, mid, hat, out);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    } else {
+        Scope ps(c, "k_gf_mid", st);
+        switch (s.nb) {
+            case 10: e = mid_launch<10, 4>(p.lg, q.na, mid, data, B, st); break;
+            case 11: e = mid_launch<11, 5>(p.lg, q.na, mid, data, B, st); break;
+            case 12: e = mid_launch<12, 5>(p.lg, q.na, mid, data, B, st); break;
+            default: e = mid_launch<13, 5>(p.lg, q.na, mid, data, B, st);
+        }
+        if (e != cudaSuccess) return e;
+    }
+    if (s.two) {
+        Scope ps(c, "k_gf_cols_inv", st);
+        k_gf_cols<true><<<q.nz << (p.lg - 18), kColsThreads, 0, st>>>(p.lg, 0, col, out);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if ((e = units_launch(c, true, q, p.lg, q.nz, out, st)) != cudaSuccess) return e;
+    if (s.colr) e = rows_launch(c, true, q, p.lg, q.nz, out, st);
+    return e;
+}
+
+}  // namespace gf
+}  // namespace cm

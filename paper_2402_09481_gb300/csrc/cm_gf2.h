@@ -1,0 +1,63 @@
+// Launch interface of the binary-polynomial product (cm_gf2.cu).
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "cm.h"
+#include "gf2_plan.h"
+#include "ntt_device.cuh"
+
+struct cm_ctx;
+
+namespace cm {
+namespace gf {
+
+// One operand block: bit j of its array is map(base + j) for j < lim (a), or
+// map(base + 2^lg - 1 - j) (b, reversed; lim unused).
+struct InOp {
+    BitMap map;
+    uint64_t base, lim;
+};
+
+// One output window: m bits to z (words past m written 0); zero, with the
+// status flag set, when the Dodis et al. flags at pre (if any) report a
+// constant input.
+struct OutOp {
+    uint64_t *z;
+    uint64_t m;
+    const uint32_t *pre;
+    uint32_t *status;
+};
+
+// The operand blocks and windows of one launch sequence.  Blocks 0 .. na - 1
+// are a's, then nb of b.  A single extraction generates them from one pair of
+// maps and fixed steps; a batch lists them in device memory (in / out).
+struct Ops {
+    const InOp *in;
+    const OutOp *out;
+    InOp a0, b0;
+    OutOp z0;
+    uint64_t astep, bstep, zstep;  // zstep a multiple of 64
+    uint32_t na, nb, nz;
+};
+
+// A transform length and the blocks over it.  nin > 1 or nz > 1 (generated ops
+// only): window w sums the products of a's block i with b's block i + w.
+struct Product {
+    int lg;
+    uint32_t nin;  // products summed per window (1: pair i gives window i)
+};
+
+// Scratch bytes of a product over `ops`.
+uint64_t product_scratch(const Product &p, const Ops &ops);
+// Enqueue it; scratch holds product_scratch bytes.  tables: device Pass tables
+// (2 per length from kMinLg on: mid, col).  c: context for tracing (may be null).
+cudaError_t launch_product(cm_ctx *c, const Product &p, const Ops &ops, const Pass *tables, void *scratch,
+                           cudaStream_t st);
+
+// Host image of the device tables.
+constexpr int kTables = 2 * (kMaxLg - kMinLg + 1);
+void build_tables(Pass *t);  // kTables entries
+
+}  // namespace gf
+}  // namespace cm

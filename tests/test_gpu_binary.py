@@ -1,0 +1,105 @@
+"""The binary-polynomial form of the products (additive transforms over packed
+bits, products longer than 2^23 in a context with default options) against the
+integer transforms of another context, every bit, and the oracle on sampled
+rows: each transform length at its edges, ragged lengths, every kind, one
+window of several blocks, several windows of one block, and both."""
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from oracle import extractors as ex
+from paper_2402_09481_gb300 import inputs, native
+from conftest import from_dev, to_dev
+
+pytestmark = pytest.mark.gpu
+T, C, D = native.TOEPLITZ, native.CIRCULANT, native.DODIS
+
+
+@pytest.fixture(scope="module")
+def q30():
+    from paper_2402_09481_gb300 import build
+    build.build()
+    c = native.Context(0, field=native.FIELD_Q30)
+    yield c
+    c.close()
+
+
+def ybits(kind, n, m):
+    return n + m - 1 if kind == T else (n + 1 if kind == C else n)
+
+
+def run(ctx, kind, n, m, x, y):
+    z = torch.full((native.words(m),), -1, dtype=torch.int64, device="cuda")
+    if kind == T:
+        return ctx.toeplitz(x, n, y, m, z)
+    if kind == C:
+        return ctx.circulant(x, n, y, m, z)
+    return ctx.dodis(x, y, n, m, z)
+
+
+def resolve(kind, n, m):
+    if kind == C:
+        n = oracle.next_na(n + 1) - 1
+    elif kind == D:
+        n = oracle.next_na(n)
+    return n, m if kind == T else min(m, n)
+
+
+CASES = [(T, 2 ** lg - m + 1 + d, m) for lg in (24, 25) for m, d in ((2 ** (lg - 2) + 17, 0), (77, 0), (2 ** (lg - 1) + 1, 1))
+         if not (lg == 25 and d)]
+CASES += [
+    (T, 2 ** 23, 2), (T, 1, 2 ** 24), (T, 2 ** 24 + 1, 2 ** 24),
+    (C, 12_000_000, 4_000_000), (C, 16777258, 8388629), (D, 9_000_000, 1), (D, 9_000_000, 8_999_999),
+    # one window, several input blocks; one block, several windows; both
+    (T, 40_000_000, 3), (T, 70_000_001, 5_000_011), (T, 5, 40_000_000), (T, 3_000_001, 70_000_003),
+    (T, 40_000_003, 40_000_001), (C, 50_000_000, 20_000_003), (D, 60_000_000, 50_000_000),
+]
+
+
+@pytest.mark.parametrize("kind,n,m", CASES)
+def test_binary_form_matches(cm_ctx, q30, kind, n, m):
+    n, m = resolve(kind, n, m)
+    xw = inputs.bernoulli_half(31 + n % 83, n)
+    if kind == D:
+        xw[0] = (xw[0] | np.uint64(1)) & ~np.uint64(2)
+    yw = inputs.bernoulli_half(32 + m % 79, ybits(kind, n, m))
+    x, y = to_dev(xw), to_dev(yw)
+    cm_ctx.profile_enable(True)
+    cm_ctx.profile_read(reset=True)
+    z = run(cm_ctx, kind, n, m, x, y)
+    prof = cm_ctx.profile_read(reset=True)
+    cm_ctx.profile_enable(False)
+    assert any(k.startswith("k_gf") for k in prof), prof
+    assert torch.equal(z, run(q30, kind, n, m, x, y))
+    zw = from_dev(z)
+    rows = np.unique(np.concatenate([np.arange(min(m, 8)), np.arange(max(0, m - 8), m),
+                                     np.random.default_rng(m).integers(0, m, 8)]))
+    got = ((zw[rows >> 6] >> (rows & 63).astype(np.uint64)) & np.uint64(1)).astype(np.uint8)
+    fn = {T: lambda: oracle.toeplitz_rows(xw, n, yw, m, rows), C: lambda: oracle.circulant_rows(xw, n, yw, m, rows),
+          D: lambda: oracle.dodis_rows(xw, yw, n, m, rows)}[kind]
+    assert (got == fn()).all()
+
+
+@pytest.mark.parametrize("P,m", [(9_000_000, 70001), (40_000_000, 20_000_000)])
+def test_binary_form_precondition(cm_ctx, P, m):
+    # a constant Dodis et al. input: zero output, reported, flag cleared after
+    P = oracle.next_na(P)
+    y = to_dev(inputs.bernoulli_half(6, P))
+    for fill in (0, 1):
+        z = run(cm_ctx, D, P, m, to_dev(ex.pack_bits(np.full(P, fill, dtype=np.uint8))), y)
+        assert cm_ctx.device_status()[0] == native.CM_EPRECOND
+        assert not from_dev(z).any()
+    assert cm_ctx.device_status() == (native.CM_OK, 0)
+
+
+def test_binary_form_budget_falls_back(q30):
+    # a scratch budget below the binary form's: the integer planner's blocks, same bits
+    n, m = 9_000_000, 1_000_000
+    ctx = native.Context(0, hbm_budget_bytes=4_000_000)
+    try:
+        x, y = to_dev(inputs.bernoulli_half(8, n)), to_dev(inputs.bernoulli_half(9, n + m - 1))
+        assert torch.equal(run(ctx, T, n, m, x, y), run(q30, T, n, m, x, y))
+    finally:
+        ctx.close()

@@ -10,7 +10,9 @@
  * product's length) is exact: q = 5 * 2^25 + 1 with lazy reduction for
  * transforms up to 2^25, the paper's own q = 3 * 2^30 + 1 (Section
  * "Performance") up to 2^30, and Goldilocks p = 2^64 - 2^32 + 1 up to 2^32.
- * The choice changes speed, never a result bit.
+ * Long single calls and batches of a context with default options work on the
+ * bits themselves instead: the same product over GF(2), by additive transforms
+ * of binary polynomials.  The choice changes speed, never a result bit.
  *
  * Conventions shared by every entry point
  * ---------------------------------------
@@ -77,8 +79,11 @@ typedef struct {
      * up to 2^30 and Goldilocks above (the planner may prefer blocks over the
      * smaller fields to one longer transform); CM_FIELD_Q30 skips the field of
      * 5 * 2^25 + 1; CM_FIELD_GOLDILOCKS takes Goldilocks throughout.  Results
-     * are identical.  Batches and the server run their work-list instances
-     * over 3 * 2^30 + 1 (Goldilocks in a CM_FIELD_GOLDILOCKS context). */
+     * are identical.  Under CM_FIELD_AUTO, with max_transform_lg,
+     * max_sum_blocks and plan_mode at their defaults too, single calls with
+     * K + m - 1 > 2^23 and batch instances with K + m - 1 > 2^14 run as binary
+     * polynomials (when that form's scratch fits the budget).  The work list of
+     * batches and the server runs over 5 * 2^25 + 1. */
     uint32_t field;
     /* Most input blocks whose transform-domain products are summed before one
      * inverse transform; 0 = as many as keep every count below the field's
@@ -270,12 +275,15 @@ typedef struct {
 /*
  * Plan a batch of `count` extractions of any mix of kinds (the paper has no
  * batched form; each instance computes exactly what its single call computes).
- * All instances with transform length L <= 2^25 run in ONE persistent kernel
+ * Instances with 2^14 < L <= 2^25 run as binary polynomials, the instances of
+ * one length together in each launch, when the context's options leave the
+ * form to the library (cm_options.field).  Shorter ones (all up to 2^21 in
+ * other contexts and under CM_BATCH_TEST_STALL) run in ONE persistent kernel
  * launch that walks a work list: an instance with L <= 2^13 is one item, a
  * larger one is split into forward column-pass tiles, fused middle rows,
  * inverse tiles with parity, and pack chunks, each item starting once the
  * items it depends on are done (bounded waits; CM_FLAG_TIMEOUT if one runs
- * out).  Instances with L > 2^25 run through the single-call kernels after it.
+ * out).  Longer instances run the single calls' kernels after it.
  * Scratch for every instance is allocated here (cudaMalloc, held until
  * cm_batch_destroy); CM_ENOMEM if it exceeds the context budget.  With
  * CM_BATCH_AUTOTUNE the candidate column-pass tiles (2^14 and 2^13 elements)
@@ -473,8 +481,11 @@ uint64_t cm_next_na_prime(uint64_t n);
 /* Largest member of N_A <= n (0 if n < 3). */
 uint64_t cm_prev_na_prime(uint64_t n);
 
-/* How a single call of (kind, n, m) runs under the given options (the
- * planner of cm_toeplitz). */
+/* How the integer transforms run (kind, n, m) under the given options (the
+ * planner described at cm_toeplitz).  The server plans every request this way;
+ * single calls and batches do where they do not take the binary form (see
+ * cm_options.field), whose scratch is smaller: a quarter byte per transform
+ * bit, half a byte where blocks are summed. */
 typedef struct {
     uint64_t transform_length; /* the longest product's transform length L */
     uint64_t products;         /* middle products: input blocks x output windows */

@@ -10,6 +10,7 @@
 #include "cm_internal.h"
 #include "cm_ctx.h"
 #include "cm_gf2.h"
+#include "cm_route.h"
 #include "ntt25.cuh"
 
 namespace cm {
@@ -673,22 +674,10 @@ cm_status enqueue_blocks(cm_ctx *ctx, const std::vector<Block> &bl, const uint64
     return CM_OK;
 }
 
-// How one call runs: as binary polynomials (cm_gf2.cu) or as the block list of
-// the integer transforms.
-struct Route {
-    bool gf = false;
-    gf::Product prod;
-    gf::Ops ops;             // pointers filled in by enqueue_route
-    int kind;
-    uint64_t n;
-    std::vector<Block> bl;
-    uint64_t need = 0, tmp_off = 0, pre_off = 0;
-};
-
 // The operands of z_i = sum_t a_t b_(t+i) over x and y: a_t is x reversed
 // (Toeplitz) or x in order (zero past its end: the Circulant pad bit), b_k is y
 // from an offset, cyclically.
-static void gf_maps(int kind, uint64_t n, uint64_t m, gf::Ops *q) {
+void gf_maps(int kind, uint64_t n, uint64_t m, gf::Ops *q) {
     const bool t = kind == CM_TOEPLITZ;
     const uint64_t K = kind == CM_CIRCULANT ? n + 1 : n;
     q->a0.map = bitmap(nullptr, t ? kReverse : kIdentity, n, n, t ? n - 1 : 0);
@@ -700,7 +689,7 @@ static void gf_maps(int kind, uint64_t n, uint64_t m, gf::Ops *q) {
 // products are summed before the window's inverse: one window with blocks as
 // long as fit beside it, or both in steps of 2^24 so that windows share the
 // seed's blocks.
-static void gf_shape(int kind, uint64_t n, uint64_t m, gf::Product *p, gf::Ops *q) {
+void gf_shape(int kind, uint64_t n, uint64_t m, gf::Product *p, gf::Ops *q) {
     const uint64_t K = kind == CM_CIRCULANT ? n + 1 : n, N = 1ull << gf::kMaxLg;
     memset(q, 0, sizeof(*q));
     q->na = q->nb = q->nz = 1;
@@ -731,15 +720,19 @@ static void gf_shape(int kind, uint64_t n, uint64_t m, gf::Product *p, gf::Ops *
 // 1812 / 10659: below 2^24 too few tiles to fill the GPU.
 constexpr int kGfMinLg = 24;
 
-static bool gf_applies(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m) {
+bool gf_allowed(const cm_ctx *ctx) {
     const PlanOptions &o = ctx->popt;
-    if (o.fields != kFieldsAll || o.max_lg != 32 || o.max_sum || o.single) return false;
+    return o.fields == kFieldsAll && o.max_lg == 32 && !o.max_sum && !o.single;
+}
+
+static bool gf_applies(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m) {
+    if (!gf_allowed(ctx)) return false;
     if (n > kMaxBits || m > kMaxBits) return false;
     const uint64_t K = kind == CM_CIRCULANT ? n + 1 : n;
     return K + m > (1ull << (kGfMinLg - 1)) + 1 && valid_args(kind, n, m);
 }
 
-static cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t budget, Route *r) {
+cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t budget, Route *r) {
     r->kind = kind;
     r->n = n;
     if (gf_applies(ctx, kind, n, m)) {
@@ -755,7 +748,7 @@ static cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m,
     return r->need > budget ? CM_ENOMEM : CM_OK;
 }
 
-static cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t *y, uint64_t *z, void *scratch,
+cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t *y, uint64_t *z, void *scratch,
                                cudaStream_t st) {
     uint8_t *sc = static_cast<uint8_t *>(scratch);
     if (!r.gf) return enqueue_blocks(ctx, r.bl, x, y, z, sc, r.tmp_off, r.pre_off, st);
@@ -770,7 +763,7 @@ static cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const u
         if (s != CM_OK) return s;
         r.ops.z0.pre = pre;
     }
-    return cuda_status(gf::launch_product(ctx, r.prod, r.ops, ctx->d_gf, scratch, st));
+    return cuda_status(gf::launch_product(ctx, ctx->nsm, r.prod, r.ops, ctx->d_gf, scratch, st));
 }
 
 cm_status run_single(cm_ctx *ctx, int kind, const uint64_t *x, uint64_t n, const uint64_t *y,

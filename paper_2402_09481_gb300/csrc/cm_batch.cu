@@ -27,6 +27,7 @@
 #include "cm_ctx.h"
 #include "cm_internal.h"
 #include "cm_batch_internal.h"
+#include "cm_route.h"
 #include "ntt_generic.cuh"
 
 namespace cm {
@@ -364,12 +365,28 @@ void build_worklist(const cm_desc *descs, const Plan *plans, const uint32_t *idx
 
 using namespace cm;
 
+// The instances of one transform length: both operands' arrays (na + nb of
+// them) at `off` in the batch's scratch.
+struct GfGroup {
+    int lg;
+    std::vector<uint32_t> idx;
+    size_t off;
+    gf::Ops ops;
+};
+
 struct cm_batch {
     cm_ctx *ctx = nullptr;
     std::vector<cm_desc> descs;
     std::vector<Plan> plans;
     std::vector<uint32_t> wl;       // instances on the work list
-    std::vector<uint32_t> solo;     // instances with L > 2^21 (single-call kernels)
+    std::vector<uint32_t> solo;     // instances that run the single-call kernels one by one
+    std::vector<Route> routes;      // theirs, where that is not their plan (same order as solo)
+    std::vector<GfGroup> groups;    // binary-polynomial products, one group a transform length
+    std::vector<gf::SameOp> same;   // their Dodis et al. inputs
+    void *d_gfops = nullptr;        // operand, window and input lists of the groups
+    gf::SameOp *d_same = nullptr;
+    uint32_t *d_gfpre = nullptr;    // two words per entry of same
+    uint32_t long_instances = 0;    // L > 2^21
     std::vector<size_t> off_scratch;
     void *scratch = nullptr;
     size_t scratch_bytes = 0;
@@ -425,12 +442,91 @@ static cm_status batch_enqueue(cm_batch *b, cudaStream_t st) {
         b->kernel_launches += 1;
     }
     uint8_t *sc = static_cast<uint8_t *>(b->scratch);
-    for (uint32_t di : b->solo) {
+    if (!b->same.empty()) {
+        if (cudaMemsetAsync(b->d_gfpre, 0, 8 * b->same.size(), st) != cudaSuccess) return CM_EDEVICE;
+        ProfScope ps(ctx, "k_gf_same", st);
+        if (gf::launch_same(b->d_same, (uint32_t)b->same.size(), st) != cudaSuccess) return CM_EDEVICE;
+        b->kernel_launches += 1;
+    }
+    for (const GfGroup &g : b->groups) {
+        const gf::Product p{g.lg, 1};
+        if (gf::launch_product(ctx, ctx->nsm, p, g.ops, ctx->d_gf, sc + g.off, st) != cudaSuccess) return CM_EDEVICE;
+        b->kernel_launches += gf::product_launches(p, g.ops);
+    }
+    for (size_t i = 0; i < b->solo.size(); ++i) {
+        const uint32_t di = b->solo[i];
         const cm_desc &d = b->descs[di];
+        if (!b->routes.empty()) {
+            Route &r = b->routes[i];
+            cm_status s = enqueue_route(ctx, r, d.x, d.y, d.z, sc + b->off_scratch[di], st);
+            if (s != CM_OK) return s;
+            b->kernel_launches += r.gf ? gf::product_launches(r.prod, r.ops) + (d.kind == CM_DODIS)
+                                       : b->plans[di].launches;
+            continue;
+        }
         cm_status s = enqueue_extract(ctx, b->plans[di], d.x, d.y, d.z, sc + b->off_scratch[di], st);
         if (s != CM_OK) return s;
         b->kernel_launches += b->plans[di].launches;
     }
+    return CM_OK;
+}
+
+// Device lists of the groups' operands, windows and Dodis et al. inputs.
+static cm_status gf_lists(cm_batch *b) {
+    size_t nin = 0, nout = 0;
+    for (const GfGroup &g : b->groups) {
+        nin += 2 * g.idx.size();
+        nout += g.idx.size();
+    }
+    if (!nin) return CM_OK;
+    for (const GfGroup &g : b->groups)
+        for (uint32_t di : g.idx)
+            if (b->descs[di].kind == CM_DODIS) b->same.push_back({b->descs[di].x, b->descs[di].n, nullptr});
+    const size_t out_off = round256(nin * sizeof(gf::InOp)), same_off = round256(out_off + nout * sizeof(gf::OutOp)),
+                 pre_off = round256(same_off + b->same.size() * sizeof(gf::SameOp));
+    const size_t bytes = pre_off + 8 * b->same.size() + 8;
+    if (cudaMalloc(&b->d_gfops, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return CM_ENOMEM;
+    }
+    uint8_t *base = static_cast<uint8_t *>(b->d_gfops);
+    gf::InOp *din = reinterpret_cast<gf::InOp *>(base);
+    gf::OutOp *dout = reinterpret_cast<gf::OutOp *>(base + out_off);
+    b->d_same = reinterpret_cast<gf::SameOp *>(base + same_off);
+    b->d_gfpre = reinterpret_cast<uint32_t *>(base + pre_off);
+    std::vector<gf::InOp> in;
+    std::vector<gf::OutOp> out;
+    size_t ns = 0;
+    for (GfGroup &g : b->groups) {
+        const uint32_t cnt = (uint32_t)g.idx.size();
+        std::vector<gf::InOp> second;
+        memset(&g.ops, 0, sizeof(g.ops));
+        g.ops.in = din + in.size();
+        g.ops.out = dout + out.size();
+        g.ops.na = g.ops.nb = g.ops.nz = cnt;
+        for (uint32_t di : g.idx) {
+            const cm_desc &d = b->descs[di];
+            gf::Ops q;
+            gf::Product p;
+            gf_shape(d.kind, d.n, d.m, &p, &q);
+            gf_maps(d.kind, d.n, d.m, &q);
+            q.a0.map.src = d.x;
+            q.b0.map.src = d.y;
+            in.push_back(q.a0);
+            second.push_back(q.b0);
+            uint32_t *pre = nullptr;
+            if (d.kind == CM_DODIS) {
+                pre = b->d_gfpre + 2 * ns;
+                b->same[ns++].flags = pre;
+            }
+            out.push_back({d.z, d.m, pre, b->ctx->d_status});
+        }
+        in.insert(in.end(), second.begin(), second.end());
+    }
+    if (cudaMemcpy(din, in.data(), in.size() * sizeof(gf::InOp), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(dout, out.data(), out.size() * sizeof(gf::OutOp), cudaMemcpyHostToDevice) != cudaSuccess ||
+        (ns && cudaMemcpy(b->d_same, b->same.data(), ns * sizeof(gf::SameOp), cudaMemcpyHostToDevice) != cudaSuccess))
+        return CM_EDEVICE;
     return CM_OK;
 }
 
@@ -440,6 +536,7 @@ static void batch_free(cm_batch *b) {
     if (b->d_insts) cudaFree(b->d_insts);
     if (b->d_items) cudaFree(b->d_items);
     if (b->d_ctrl) cudaFree(b->d_ctrl);
+    if (b->d_gfops) cudaFree(b->d_gfops);
     if (b->scratch) cudaFree(b->scratch);
     delete b;
 }
@@ -471,6 +568,11 @@ extern "C" cm_status cm_batch_create(cm_ctx *ctx, const cm_desc *descs, uint32_t
     b->descs.assign(descs, descs + count);
     b->plans.resize(count);
     b->off_scratch.assign(count, 0);
+    // Transforms of 2^15 .. 2^25 run as binary polynomials, every length's
+    // instances together, unless the context's options ask for the integer ones
+    // (the bounded waits that CM_BATCH_TEST_STALL runs out are the work list's).
+    const bool use_gf = gf_allowed(ctx) && !b->test_stall;
+    std::vector<uint32_t> by_lg[gf::kMaxLg + 1];
     size_t total = 0;
     for (uint32_t i = 0; i < count; ++i) {
         const cm_desc &d = descs[i];
@@ -479,16 +581,39 @@ extern "C" cm_status cm_batch_create(cm_ctx *ctx, const cm_desc *descs, uint32_t
             return CM_EINVAL;
         }
         b->off_scratch[i] = total;
-        if (on_worklist(b->plans[i])) {
+        if (!on_worklist(b->plans[i])) ++b->long_instances;
+        if (use_gf && b->plans[i].lg >= gf::kMinLg && b->plans[i].lg <= gf::kMaxLg) {
+            by_lg[b->plans[i].lg].push_back(i);
+        } else if (on_worklist(b->plans[i])) {
             b->wl.push_back(i);
             total += worklist_scratch_bytes(b->plans[i]);
         } else {
             // the single-call kernels, over the context's field set
             make_plan(d.kind, d.n, d.m, &b->plans[i], ctx->popt.fields, ctx->popt.tune);
             b->solo.push_back(i);
-            total += round256(b->plans[i].scratch_bytes);
+            if (use_gf) {  // past 2^25
+                Route r;
+                const cm_status rs = make_route(ctx, d.kind, d.n, d.m, ctx->budget, &r);
+                if (rs != CM_OK) {
+                    delete b;
+                    return rs;
+                }
+                total += round256(r.need);
+                b->routes.push_back(r);
+            } else {
+                total += round256(b->plans[i].scratch_bytes);
+            }
         }
     }
+    for (int lg = gf::kMaxLg; lg >= gf::kMinLg; --lg)
+        if (!by_lg[lg].empty()) {
+            GfGroup g;
+            g.lg = lg;
+            g.idx = by_lg[lg];
+            g.off = total;
+            total += round256(2 * g.idx.size() << (lg - 3));
+            b->groups.push_back(g);
+        }
     if (total > ctx->budget) {
         delete b;
         return CM_ENOMEM;
@@ -508,6 +633,7 @@ extern "C" cm_status cm_batch_create(cm_ctx *ctx, const cm_desc *descs, uint32_t
         return CM_EDEVICE;
     }
     cm_status s = batch_build(b);
+    if (s == CM_OK) s = gf_lists(b);
     if (s != CM_OK) {
         batch_free(b);
         return s;
@@ -583,7 +709,9 @@ extern "C" cm_status cm_batch_info(const cm_batch *b, cm_batch_stats *st) {
     memset(st, 0, sizeof(*st));
     st->instances = (uint32_t)b->descs.size();
     st->work_items = b->nitems;
-    st->solo_instances = (uint32_t)b->solo.size();
+    for (const GfGroup &g : b->groups)  // tiles of the last pass
+        st->work_items += (uint32_t)g.idx.size() * (uint32_t)gf::shape_of(g.lg).tiles;
+    st->solo_instances = b->long_instances;
     st->tile_lg = (uint32_t)b->tile_lg;
     st->grid = (uint32_t)b->grid;
     st->scratch_bytes = b->scratch_bytes;

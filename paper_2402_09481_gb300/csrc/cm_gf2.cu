@@ -51,42 +51,91 @@ namespace gf {
 
 namespace {
 
-// Values of positions k .. k + 31 of a map: two 32-bit loads and a funnel shift
-// when they are a run of source bits, else position by position.
-__device__ __forceinline__ uint32_t map_word(const BitMap &m, uint64_t k) {
-    if (k >= m.len) return 0u;
-    if (k + 32 <= m.len) {
-        uint64_t lo;
-        bool run = true;
-        if (m.mode == kIdentity) {
-            lo = k;
-        } else if (m.mode == kModForward) {
-            lo = k + m.off;
-            if (lo >= m.srclen) lo -= m.srclen;
-            if (lo >= m.srclen) lo -= m.srclen;
-            run = lo + 32 <= m.srclen;
-        } else {
-            lo = m.off - k - 31;
-            run = m.off - k < m.srclen && m.off >= k + 31;
-        }
-        if (run) {
-            const uint32_t *p = reinterpret_cast<const uint32_t *>(m.src) + (lo >> 5);
-            const uint32_t sh = (uint32_t)lo & 31u;
-            const uint32_t r = sh ? __funnelshift_r(__ldg(p), __ldg(p + 1), sh) : __ldg(p);
-            return m.mode == kReverse ? __brev(r) : r;
+// How an operand block's words lie in the source: word w of the array, inside
+// [w0[i], w0[i] + n[i]), is the 32 bits from bit sh[i] of source word
+// p[i] + dir w (in reversed order when dir < 0).  The two pieces are the bits
+// before and after b's cyclic wrap; words w >= zero (a) or < zero (b) are 0, and
+// the few others (at the pieces' ends) are read bit by bit.
+struct Lin {
+    const uint32_t *p[2];
+    uint32_t sh[2], w0[2], n[2], zero;
+    bool back;
+};
+
+__device__ __forceinline__ Lin lin_of(const InOp &o, bool is_b, int lg) {
+    Lin l;
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(o.map.src);
+    const int64_t N = 1ll << lg, nw = N >> 5;
+    l.w0[0] = l.w0[1] = l.n[0] = l.n[1] = l.sh[0] = l.sh[1] = 0;
+    l.p[0] = l.p[1] = src;
+    l.back = is_b || o.map.mode == kReverse;
+    if (!is_b) {
+        const uint64_t left = o.map.len > o.base ? o.map.len - o.base : 0, bits = left < o.lim ? left : o.lim;
+        l.zero = (uint32_t)(((int64_t)bits + 31 < N ? (int64_t)bits + 31 : N) >> 5);
+        l.n[0] = (uint32_t)((int64_t)bits < N ? (int64_t)bits >> 5 : nw);
+        const int64_t c = l.back ? (int64_t)o.map.off - (int64_t)o.base - 31 : (int64_t)o.base;
+        l.sh[0] = (uint32_t)c & 31u;
+        l.p[0] = src + (c >> 5);
+    } else {
+        const int64_t top = (int64_t)o.base + N;  // word w: positions top - 32 - 32 w ..
+        const int64_t z = top - (int64_t)o.map.len, cut = top + (int64_t)o.map.off - (int64_t)o.map.srclen;
+        l.zero = z > 0 ? (uint32_t)(z >> 5) : 0u;               // words wholly past the end
+        const int64_t full = z > 0 ? (z + 31) >> 5 : 0;         // first word wholly inside
+        const int64_t e1 = cut > 0 ? cut >> 5 : 0;              // words [full, e1) lie past the wrap
+        const int64_t b0 = cut > 0 ? (cut + 31) >> 5 : 0;       // words [b0, nw) before it
+        for (int i = 0; i < 2; ++i) {
+            int64_t w0 = i ? full : (full > b0 ? full : b0), w1 = i ? (e1 < nw ? e1 : nw) : nw;
+            l.w0[i] = (uint32_t)(w0 < nw ? w0 : nw);
+            l.n[i] = w1 > w0 ? (uint32_t)(w1 - w0) : 0u;
+            const int64_t c = top - 32 + (int64_t)o.map.off - (i ? (int64_t)o.map.srclen : 0);
+            l.sh[i] = (uint32_t)c & 31u;
+            l.p[i] = src + (c >> 5);
         }
     }
-    return m.get_run<32>(k);
+    return l;
 }
 
-// Word w of an operand block's array of 2^lg bits.
-__device__ __forceinline__ uint32_t in_word(const InOp &o, bool is_b, int lg, uint64_t w) {
-    if (is_b) return __brev(map_word(o.map, o.base + (1ull << lg) - 32 - 32 * w));
-    const uint64_t j = 32 * w;
-    if (j >= o.lim) return 0u;
-    uint32_t v = map_word(o.map, o.base + j);
-    if (o.lim - j < 32) v &= (1u << (uint32_t)(o.lim - j)) - 1u;
-    return v;
+// Words at(0) .. at(N - 1) (~0: none) of an operand block's array of 2^lg bits:
+// all the loads first, so that they are in flight together.
+template <int N, class F>
+__device__ __forceinline__ void in_words(const InOp &o, const Lin &l, bool is_b, int lg, F at, uint32_t (&v)[N]) {
+    uint32_t lo[N], hi[N], sh[N];
+    bool slow = false;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const uint32_t w = at(i);
+        const bool in0 = w - l.w0[0] < l.n[0], in1 = w - l.w0[1] < l.n[1];
+        const uint32_t *p = (in1 ? l.p[1] : l.p[0]) + (l.back ? -(int64_t)w : (int64_t)w);
+        sh[i] = in1 ? l.sh[1] : l.sh[0];
+        lo[i] = hi[i] = 0;
+        if (in0 || in1) {
+            lo[i] = __ldg(p);
+            if (sh[i]) hi[i] = __ldg(p + 1);
+        } else {
+            slow |= w != ~0u && (is_b ? w >= l.zero : w < l.zero);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        v[i] = __funnelshift_r(lo[i], hi[i], sh[i]);
+        if (l.back) v[i] = __brev(v[i]);
+    }
+    if (slow) {
+#pragma unroll 1
+        for (int i = 0; i < N; ++i) {
+            const uint32_t w = at(i);
+            if (w == ~0u || w - l.w0[0] < l.n[0] || w - l.w0[1] < l.n[1] || !(is_b ? w >= l.zero : w < l.zero)) continue;
+            uint32_t r = 0;
+            for (uint32_t b = 0; b < 32; ++b) {
+                const uint64_t j = 32ull * w + b;
+                const uint64_t k = is_b ? o.base + (1ull << lg) - 1 - j : o.base + j;
+                if (is_b || j < o.lim) r |= (uint32_t)o.map.get(k) << b;
+            }
+#pragma unroll
+            for (int t = 0; t < N; ++t)
+                if (t == i) v[t] = r;
+        }
+    }
 }
 
 __device__ __forceinline__ InOp in_op(const Ops &q, uint32_t o) {
@@ -196,36 +245,72 @@ __device__ __forceinline__ uint32_t row_before(const uint32_t *e, uint32_t row, 
     return v;
 }
 
-// Whole-row stages on sm[512][CW].
+// One whole-row stage (top, sh) on sm[512][CW].
 template <int KIND, int CW>
-__device__ __forceinline__ void row_whole_stages(uint32_t *sm, const Stages &st) {
+__device__ __forceinline__ void row_whole_stage(uint32_t *sm, uint32_t top, uint32_t sh) {
     constexpr int LC = CW == 32 ? 5 : 4;
-    const uint32_t c = threadIdx.x & (CW - 1u), g = threadIdx.x >> LC;
     constexpr uint32_t NG = kRowsThreads >> LC;
-    for (int n = 0; n < st.n; ++n) {
-        const int q = KIND == kConvBInv ? st.n - 1 - n : n;
-        const uint32_t top = st.top[q], H = 1u << top, s = 1u << st.sh[q];
-        auto bulk = [&]() {
-            __syncthreads();
+    const uint32_t c = threadIdx.x & (CW - 1u), g = threadIdx.x >> LC;
+    const uint32_t H = 1u << top, s = 1u << sh;
+    auto bulk = [&]() {
+        __syncthreads();
 #pragma unroll
-            for (uint32_t i = 0; i < 256; i += NG) {
-                const uint32_t u = i + g, v = u & (H - 1u), row = v | ((u ^ v) << 1);
-                if (v >= s) sm[row * CW + c] ^= sm[(row + H - s) * CW + c];
-            }
-        };
-        auto wrapped = [&]() {
-            __syncthreads();
-            for (uint32_t u = g; u < (512u >> (top + 1)) * s; u += NG) {
-                const uint32_t row = ((u >> st.sh[q]) << (top + 1)) + (KIND == kConvA ? H : 0u) + (u & (s - 1u));
-                sm[row * CW + c] ^= sm[(row + H - s) * CW + c];
-            }
-        };
-        if (KIND == kConvBInv) {
-            bulk();
-            wrapped();
-        } else {
-            wrapped();
-            bulk();
+        for (uint32_t i = 0; i < 256; i += NG) {
+            const uint32_t u = i + g, v = u & (H - 1u), row = v | ((u ^ v) << 1);
+            if (v >= s) sm[row * CW + c] ^= sm[(row + H - s) * CW + c];
+        }
+    };
+    auto wrapped = [&]() {
+        __syncthreads();
+        for (uint32_t u = g; u < (512u >> (top + 1)) * s; u += NG) {
+            const uint32_t row = ((u >> sh) << (top + 1)) + (KIND == kConvA ? H : 0u) + (u & (s - 1u));
+            sm[row * CW + c] ^= sm[(row + H - s) * CW + c];
+        }
+    };
+    if (KIND == kConvBInv) {
+        bulk();
+        wrapped();
+    } else {
+        wrapped();
+        bulk();
+    }
+}
+
+// The stages that convert k index bits from `base` on, in kConvA's order: the
+// shifts of the top k - q of them (q the largest power of two below k), then
+// those bits and the lower q among themselves.
+constexpr void conv_list(int base, int k, Stages *s) {
+    if (k <= 1) return;
+    int t = 0;
+    while ((2 << t) < k) ++t;
+    const int q = 1 << t, r = k - q;
+    for (int j = r - 1; j >= 0; --j) {
+        s->top[s->n] = (uint8_t)(base + q + j);
+        s->sh[s->n++] = (uint8_t)(base + j);
+    }
+    conv_list(base + q, r, s);
+    conv_list(base, q, s);
+}
+template <int BITS>
+struct StageList {
+    Stages s;
+    constexpr StageList() : s{} { conv_list(0, BITS, &s); }
+};
+
+// All whole-row stages: RC > 5 rows' list is known at compile time.
+template <int KIND, int CW, int RC>
+__device__ __forceinline__ void row_whole_stages(uint32_t *sm, const Stages &st) {
+    if constexpr (RC > 5) {
+        constexpr StageList<RC> L{};
+#pragma unroll
+        for (int n = 0; n < L.s.n; ++n) {
+            const int q = KIND == kConvBInv ? L.s.n - 1 - n : n;
+            row_whole_stage<KIND, CW>(sm, L.s.top[q], L.s.sh[q]);
+        }
+    } else {
+        for (int n = 0; n < st.n; ++n) {
+            const int q = KIND == kConvBInv ? st.n - 1 - n : n;
+            row_whole_stage<KIND, CW>(sm, st.top[q], st.sh[q]);
         }
     }
     __syncthreads();
@@ -246,24 +331,32 @@ __global__ void __launch_bounds__(kRowsThreads, 2) k_gf_rows(const __grid_consta
     uint32_t x[32];
     if (!INV) {
         const InOp in = in_op(q, op);
+        const Lin lin = lin_of(in, is_b, lg);
         // phase 0: the row's end (its last words, then zeros a's shifts run into);
         // phase 1: b's words before column 0; phase 2: the stripes
         for (int phase = first ? 0 : 2; phase < 3; ++phase) {
             if (phase == 1 && !is_b) continue;
             __syncthreads();
-            for (int i = 0; i < 32; ++i) {
-                const uint32_t u = row_unit<B0>(warp, i), row = u & (R - 1u), stripe = (grp << S) + (u >> r);
-                uint32_t v = 0, col = ~0u;
-                if (phase == 2) {
-                    if (16 * stripe + lane >= 16 && stripe < 128) col = 16 * stripe + lane - 16;
-                    else if (is_b && stripe < 128) v = side[row * 16 + lane];
-                } else if (u < R) {
-                    if (phase == 1) v = lane >= 16 ? row_before(side, row, lane - 16, 16) : 0u;
-                    else if (is_b) col = 2016u + lane;
-                    else if (lane < 16) col = 2032u + lane;
+            for (int i0 = 0; i0 < 32; i0 += 8) {
+                uint32_t v[8];
+                if (phase != 1)
+                    in_words<8>(in, lin, is_b, lg, [&](int i) -> uint32_t {
+                        const uint32_t u = row_unit<B0>(warp, i0 + i), row = u & (R - 1u), stripe = (grp << S) + (u >> r);
+                        uint32_t col = ~0u;
+                        if (phase == 2) {
+                            if (16 * stripe + lane >= 16 && stripe < 128) col = 16 * stripe + lane - 16;
+                        } else if (u < R && (is_b || lane < 16)) {
+                            col = (is_b ? 2016u : 2032u) + lane;
+                        }
+                        return col == ~0u ? col : row * 2048u + col;
+                    }, v);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint32_t u = row_unit<B0>(warp, i0 + i), row = u & (R - 1u);
+                    if (phase == 1) v[i] = u < R && lane >= 16 ? row_before(side, row, lane - 16, 16) : 0u;
+                    if (phase == 2 && is_b && first && u < R && lane < 16) v[i] = side[row * 16 + lane];
+                    xch[u * 32 + lane] = v[i];
                 }
-                if (col < 2048u) v = in_word(in, is_b, lg, (uint64_t)row * 2048u + col);
-                xch[u * 32 + lane] = v;
             }
             __syncwarp();
 #pragma unroll
@@ -285,8 +378,8 @@ __global__ void __launch_bounds__(kRowsThreads, 2) k_gf_rows(const __grid_consta
         const uint32_t c = threadIdx.x & 15u;
         if (first && !is_b)
             for (uint32_t u = threadIdx.x >> 4; u < R; u += 32) sm[u * 16 + c] ^= row_before(side, u, c, 16);
-        if (is_b) row_whole_stages<kConvB, 16>(sm, st);
-        else row_whole_stages<kConvA, 16>(sm, st);
+        if (is_b) row_whole_stages<kConvB, 16, RC>(sm, st);
+        else row_whole_stages<kConvA, 16, RC>(sm, st);
         for (uint32_t u = threadIdx.x >> 4; u < 512; u += 32) {
             const uint32_t row = u & (R - 1u), stripe = (grp << S) + (u >> r);
             if (stripe < 128) arr[(uint64_t)row * 2048u + stripe * 16u + c] = sm[u * 16 + c];
@@ -299,7 +392,7 @@ __global__ void __launch_bounds__(kRowsThreads, 2) k_gf_rows(const __grid_consta
             const uint32_t row = u & (R - 1u), stripe = ((grp << S) + (u >> r)) & 127u;
             sm[u * 32 + lane] = arr[(uint64_t)row * 2048u + ((16u * stripe + lane - 16u) & 2047u)];
         }
-        row_whole_stages<kConvBInv, 32>(sm, st);
+        row_whole_stages<kConvBInv, 32, RC>(sm, st);
 #pragma unroll
         for (int i = 0; i < 32; ++i) x[i] = sm[row_unit<B0>(warp, i) * 32 + lane];
         if (first && lane < 16) {
@@ -367,8 +460,7 @@ __global__ void __launch_bounds__(256) k_gf_units(const __grid_constant__ Ops q,
     uint32_t x[8];
     if (!INV && lg <= 16) {
         const InOp in = in_op(q, op);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = in_word(in, is_b, lg, 8 * threadIdx.x + i);
+        in_words<8>(in, lin_of(in, is_b, lg), is_b, lg, [&](int i) -> uint32_t { return 8 * threadIdx.x + i; }, x);
     } else {
         const uint4 u = *reinterpret_cast<const uint4 *>(data + w0), v = *reinterpret_cast<const uint4 *>(data + w0 + 4);
         x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
@@ -392,9 +484,10 @@ __global__ void __launch_bounds__(256) k_gf_units(const __grid_constant__ Ops q,
 // Level passes.
 
 __device__ __forceinline__ void load_pass(Pass *P, const Pass *__restrict__ g) {
-    uint32_t *d = reinterpret_cast<uint32_t *>(P);
-    const uint32_t *s = reinterpret_cast<const uint32_t *>(g);
-    for (uint32_t i = threadIdx.x; i < sizeof(Pass) / 4; i += blockDim.x) d[i] = __ldg(s + i);
+    uint4 *d = reinterpret_cast<uint4 *>(P);
+    const uint4 *s = reinterpret_cast<const uint4 *>(g);
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x; i < sizeof(Pass) / 16; i += blockDim.x) d[i] = __ldg(s + i);
 }
 
 // Levels lg - 1 .. lo: fields up to GF(2^16), twiddles that depend on the tile's
@@ -411,6 +504,7 @@ __global__ void __launch_bounds__(kColsThreads) k_gf_cols(int lg, uint32_t na, c
     __syncthreads();
     uint32_t *arr = data + ((uint64_t)op << (lg - 5)) + tile_base(P, tile);
     const uint32_t which = INV || op >= na;
+#pragma unroll
     for (uint32_t e = 4 * threadIdx.x; e < 8192; e += 4 * kColsThreads) {
         const uint4 v = *reinterpret_cast<const uint4 *>(arr + lut3(P.glut, e));
         sm[phys(lut3(P.alut, e))] = v.x;
@@ -467,6 +561,7 @@ __device__ void transpose_bits(uint32_t *sm, const Pass &P, uint32_t warp, uint3
 
 template <int NB, int KIND>
 __device__ void load_tile(uint32_t *sm, const Pass &P, const uint32_t *__restrict__ arr, uint32_t tid, uint32_t nt) {
+#pragma unroll 4
     for (uint32_t e = 8 * tid; e < (1u << NB); e += 8 * nt) {
         const uint32_t *g = arr + lut3(P.glut, e);
         const uint4 u = *reinterpret_cast<const uint4 *>(g), v = *reinterpret_cast<const uint4 *>(g + 4);
@@ -510,15 +605,17 @@ __device__ void inverse_levels(uint32_t *sm, const Pass &P, const uint32_t *base
     }
 }
 
-// One pair of tiles: both forward transforms (half the threads each), the
-// product, the inverse transform in place of b's tile.  The ALU pipe bounds it;
-// a thread holds one unit of 2 x 32 words.
-template <int NB, int FMAX>
-__global__ void __launch_bounds__(2 * MidShape<NB, FMAX>::HALF) k_gf_mid(int lg, const Pass *__restrict__ table,
+// One pair of tiles: both forward transforms, the product, the inverse
+// transform in place of b's tile.  The ALU pipe bounds it; a thread holds one
+// unit of 2 x 32 words.  PAR: half the threads on each operand, for few tiles
+// (a tile's own time counts); else one operand after the other on half as many
+// threads, so that three CTAs of an SM fill each other's gaps.
+template <int NB, int FMAX, bool PAR>
+__global__ void __launch_bounds__((PAR ? 2 : 1) * MidShape<NB, FMAX>::HALF) k_gf_mid(int lg, const Pass *__restrict__ table,
                                                                          const uint32_t *__restrict__ A,
                                                                          uint32_t *__restrict__ B) {
     using S = MidShape<NB, FMAX>;
-    constexpr int NT = 2 * S::HALF, W = 1 << FMAX;
+    constexpr int NT = (PAR ? 2 : 1) * S::HALF, W = 1 << FMAX;
     extern __shared__ __align__(16) uint32_t sm[];
     __shared__ Pass P;
     __shared__ uint32_t base[2][kMaxLev];
@@ -527,22 +624,25 @@ __global__ void __launch_bounds__(2 * MidShape<NB, FMAX>::HALF) k_gf_mid(int lg,
     load_pass(&P, table);
     __syncthreads();
     const uint64_t off = ((uint64_t)pair << (lg - 5)) + tile_base(P, tile);
-    if (threadIdx.x < 2 * kMaxLev) {
-        const uint32_t l = threadIdx.x >> 1, o = threadIdx.x & 1u;
-        if (l < P.nlev) base[o][l] = ext_twiddle(P.lev[l], P.lev[l].base[o], tile);
+    for (uint32_t i = threadIdx.x; i < 2 * P.nlev; i += NT) {
+        const uint32_t l = i >> 1, o = i & 1u;
+        base[o][l] = ext_twiddle(P.lev[l], P.lev[l].base[o], tile);
     }
-    const uint32_t op = threadIdx.x >= S::HALF, tid = threadIdx.x - op * S::HALF;
+    const uint32_t op = PAR ? threadIdx.x >= S::HALF : 0u, tid = threadIdx.x - op * S::HALF;
     uint32_t *mine = sm + op * (1u << NB);
-    if (op) load_tile<NB, kConvB>(mine, P, B + off, tid, S::HALF);
+    if (PAR ? op : false) load_tile<NB, kConvB>(mine, P, B + off, tid, S::HALF);
     else load_tile<NB, kConvA>(mine, P, A + off, tid, S::HALF);
+    if (!PAR) load_tile<NB, kConvB>(sm + (1u << NB), P, B + off, tid, S::HALF);
     __syncthreads();
-    for (uint32_t l = 0; l < P.nlev; ++l) {
+    for (uint32_t k = 0; k < (PAR ? 1u : 2u) * P.nlev; ++k) {
+        const uint32_t o = PAR ? op : k >= P.nlev, l = k - (PAR ? 0u : o * P.nlev);
+        uint32_t *t = sm + o * (1u << NB);
         if (l == P.npre) {
-            transpose_bits<NB>(sm, P, threadIdx.x >> 5, NT >> 5);
-            transpose_bits<NB>(sm + (1u << NB), P, threadIdx.x >> 5, NT >> 5);
+            transpose_bits<NB>(PAR ? sm : t, P, threadIdx.x >> 5, NT >> 5);
+            if (PAR) transpose_bits<NB>(sm + (1u << NB), P, threadIdx.x >> 5, NT >> 5);
             __syncthreads();
         }
-        level<NB, S::NFREE, FMAX, false>(mine, P.lev[l], base[op][l], l >= P.npre, tid, S::HALF);
+        level<NB, S::NFREE, FMAX, false>(t, P.lev[l], base[o][l], l >= P.npre, tid, S::HALF);
         __syncthreads();
     }
     uint32_t *sb = sm + (1u << NB);
@@ -629,23 +729,27 @@ __global__ void __launch_bounds__(256) k_gf_sum(int lg, uint32_t na, uint32_t ni
     store_tile<13>(sm, P, out + ((uint64_t)win << (lg - 5)) + tile_base(P, tile), threadIdx.x, 256);
 }
 
-void conv_stages(int base, int k, Stages *s) {
-    if (k <= 1) return;
-    int t = 0;
-    while ((2 << t) < k) ++t;  // the largest t with 2^t < k
-    const int q = 1 << t, r = k - q;
-    for (int j = r - 1; j >= 0; --j) {
-        s->top[s->n] = (uint8_t)(base + q + j);
-        s->sh[s->n++] = (uint8_t)(base + j);
+__global__ void __launch_bounds__(256) k_gf_same(const SameOp *__restrict__ ops) {
+    const SameOp o = ops[blockIdx.x];
+    const uint64_t words = (o.n + 63) >> 6;
+    bool any1 = false, any0 = false;
+    for (uint64_t w = (uint64_t)blockIdx.y * 256 + threadIdx.x; w < words; w += (uint64_t)gridDim.y * 256) {
+        const uint64_t mask = o.n - 64 * w < 64 ? (1ull << (o.n - 64 * w)) - 1 : ~0ull, v = __ldg(o.x + w) & mask;
+        any1 |= v != 0;
+        any0 |= v != mask;
     }
-    conv_stages(base + q, r, s);
-    conv_stages(base, q, s);
+    any1 = __syncthreads_or(any1);
+    any0 = __syncthreads_or(any0);
+    if (threadIdx.x == 0) {
+        if (any1) atomicOr(o.flags, 1u);
+        if (any0) atomicOr(o.flags + 1, 1u);
+    }
 }
 
 Stages stages_of(int bits) {
     Stages s;
     memset(&s, 0, sizeof(s));
-    conv_stages(0, bits, &s);
+    conv_list(0, bits, &s);
     return s;
 }
 
@@ -694,11 +798,18 @@ cudaError_t units_launch(cm_ctx *c, bool inv, const Ops &q, int lg, uint32_t ops
 }
 
 template <int NB, int FMAX>
-cudaError_t mid_launch(int lg, uint32_t pairs, const Pass *table, const uint32_t *A, uint32_t *B, cudaStream_t st) {
+cudaError_t mid_launch(int nsm, int lg, uint32_t pairs, const Pass *table, const uint32_t *A, uint32_t *B,
+                       cudaStream_t st) {
     using S = MidShape<NB, FMAX>;
-    cudaError_t e = smem_attr_once<k_gf_mid<NB, FMAX>>(2 * S::SMEM1);
-    if (e != cudaSuccess) return e;
-    k_gf_mid<NB, FMAX><<<pairs << (lg - 5 - NB), 2 * S::HALF, 2 * S::SMEM1, st>>>(lg, table, A, B);
+    const uint32_t grid = pairs << (lg - 5 - NB);
+    cudaError_t e;
+    if (grid <= (uint32_t)nsm) {
+        if ((e = smem_attr_once<k_gf_mid<NB, FMAX, true>>(2 * S::SMEM1)) != cudaSuccess) return e;
+        k_gf_mid<NB, FMAX, true><<<grid, 2 * S::HALF, 2 * S::SMEM1, st>>>(lg, table, A, B);
+    } else {
+        if ((e = smem_attr_once<k_gf_mid<NB, FMAX, false>>(2 * S::SMEM1)) != cudaSuccess) return e;
+        k_gf_mid<NB, FMAX, false><<<grid, S::HALF, 2 * S::SMEM1, st>>>(lg, table, A, B);
+    }
     return cudaGetLastError();
 }
 
@@ -719,7 +830,17 @@ uint64_t product_scratch(const Product &p, const Ops &q) {
     return (q.na + q.nb) * arr * (summed(p, q) ? 2 : 1);
 }
 
-cudaError_t launch_product(cm_ctx *c, const Product &p, const Ops &q, const Pass *tables, void *scratch,
+uint32_t product_launches(const Product &p, const Ops &q) {
+    const Shape s = shape_of(p.lg);
+    return 2 + (s.colr ? 2 : 0) + (s.two ? 2 : 0) + (summed(p, q) ? 2 : 1);
+}
+
+cudaError_t launch_same(const SameOp *ops, uint32_t count, cudaStream_t st) {
+    k_gf_same<<<dim3(count, 8), 256, 0, st>>>(ops);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_product(cm_ctx *c, int nsm, const Product &p, const Ops &q, const Pass *tables, void *scratch,
                            cudaStream_t st) {
     const Shape s = shape_of(p.lg);
     const Pass *mid = tables + 2 * (p.lg - kMinLg), *col = mid + 1;
@@ -750,10 +871,10 @@ cudaError_t launch_product(cm_ctx *c, const Product &p, const Ops &q, const Pass
     } else {
         Scope ps(c, "k_gf_mid", st);
         switch (s.nb) {
-            case 10: e = mid_launch<10, 4>(p.lg, q.na, mid, data, B, st); break;
-            case 11: e = mid_launch<11, 5>(p.lg, q.na, mid, data, B, st); break;
-            case 12: e = mid_launch<12, 5>(p.lg, q.na, mid, data, B, st); break;
-            default: e = mid_launch<13, 5>(p.lg, q.na, mid, data, B, st);
+            case 10: e = mid_launch<10, 4>(nsm, p.lg, q.na, mid, data, B, st); break;
+            case 11: e = mid_launch<11, 5>(nsm, p.lg, q.na, mid, data, B, st); break;
+            case 12: e = mid_launch<12, 5>(nsm, p.lg, q.na, mid, data, B, st); break;
+            default: e = mid_launch<13, 5>(nsm, p.lg, q.na, mid, data, B, st);
         }
         if (e != cudaSuccess) return e;
     }

@@ -52,8 +52,19 @@ struct Product {
 uint64_t product_scratch(const Product &p, const Ops &ops);
 // Enqueue it; scratch holds product_scratch bytes.  tables: device Pass tables
 // (2 per length from kMinLg on: mid, col).  c: context for tracing (may be null).
-cudaError_t launch_product(cm_ctx *c, const Product &p, const Ops &ops, const Pass *tables, void *scratch,
+cudaError_t launch_product(cm_ctx *c, int nsm, const Product &p, const Ops &ops, const Pass *tables, void *scratch,
                            cudaStream_t st);
+
+// Dodis et al. flags of `count` listed inputs (x bits, pairs of zeroed words):
+// flags[0] set by a 1 bit, flags[1] by a 0 bit.
+struct SameOp {
+    const uint64_t *x;
+    uint64_t n;
+    uint32_t *flags;
+};
+cudaError_t launch_same(const SameOp *ops, uint32_t count, cudaStream_t st);
+// Kernel launches of a product.
+uint32_t product_launches(const Product &p, const Ops &ops);
 
 // Host image of the device tables.
 constexpr int kTables = 2 * (kMaxLg - kMinLg + 1);

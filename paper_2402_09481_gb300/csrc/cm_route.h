@@ -1,0 +1,33 @@
+// How one extraction runs: as binary polynomials (cm_gf2.cu) or as the block
+// list of the integer transforms (cm_api.cu).
+#pragma once
+#include <vector>
+
+#include "cm_ctx.h"
+#include "cm_gf2.h"
+#include "cm_internal.h"
+
+namespace cm {
+
+struct Route {
+    bool gf = false;
+    gf::Product prod;
+    gf::Ops ops;  // pointers filled in by enqueue_route
+    int kind;
+    uint64_t n;
+    std::vector<Block> bl;
+    uint64_t need = 0, tmp_off = 0, pre_off = 0;  // scratch bytes; offsets in it
+};
+
+// The context's options leave the choice of transform to the library.
+bool gf_allowed(const cm_ctx *ctx);
+// The operands' maps and the transform length(s) of (kind, n, m), valid arguments.
+void gf_maps(int kind, uint64_t n, uint64_t m, gf::Ops *q);
+void gf_shape(int kind, uint64_t n, uint64_t m, gf::Product *p, gf::Ops *q);
+
+// CM_EINVAL for invalid arguments, CM_ENOMEM when no form fits `budget`.
+cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t budget, Route *r);
+cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t *y, uint64_t *z, void *scratch,
+                        cudaStream_t st);
+
+}  // namespace cm

@@ -27,7 +27,7 @@ struct Lev {
     uint32_t lanes[32];   // of the point bits inside a word: component j's lane pattern
 };
 
-struct Pass {
+struct alignas(16) Pass {
     uint32_t nlev, npre;      // levels; those before the word bits change places with point bits
     uint32_t next;            // bits of the tile number
     uint32_t xp[5];           // address bit that changes places with word bit b

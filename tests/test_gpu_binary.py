@@ -103,3 +103,40 @@ def test_binary_form_budget_falls_back(q30):
         assert torch.equal(run(ctx, T, n, m, x, y), run(q30, T, n, m, x, y))
     finally:
         ctx.close()
+
+
+def test_batch_every_length_matches(cm_ctx, q30):
+    # the batch's groups, 2^15 .. 2^25 and past them, every kind, K + m - 1 at
+    # the edges of each length, and constant Dodis et al. inputs zeroed alone
+    specs = []
+    for lg in range(15, 26):
+        L = 2 ** lg
+        specs += [(T, L - L // 3, L // 3 + 1), (T, L // 2, 2), (T, 5, L - 4),
+                  (C, oracle.next_na(L // 2 + 7) - 1, L // 4 + 3), (D, oracle.next_na(L * 5 // 9), L // 3)]
+    specs += [(T, 2 ** 25, 2 ** 24), (T, 100, 50), (T, 9000, 7000)]
+    items, bad = [], []
+    for j, (kind, n, m) in enumerate(specs):
+        xw, yw = inputs.bernoulli_half(500 + 2 * j, n), inputs.bernoulli_half(501 + 2 * j, ybits(kind, n, m))
+        if kind == D:
+            xw[0] = (xw[0] | np.uint64(1)) & ~np.uint64(2)
+            if j % 3 == 1:
+                xw = ex.pack_bits(np.full(n, j & 1, dtype=np.uint8))
+                bad.append(j)
+        items.append((kind, n, m, to_dev(xw), to_dev(yw),
+                      torch.full((native.words(m),), -1, dtype=torch.int64, device="cuda")))
+    want = [run(q30, k, n, m, x, y) for k, n, m, x, y, _ in items]
+    assert q30.device_status()[0] == native.CM_EPRECOND and bad
+    for graph in (True, False):
+        b = cm_ctx.batch(items, graph=graph)
+        b.launch()
+        assert cm_ctx.device_status()[0] == native.CM_EPRECOND
+        for j, it in enumerate(items):
+            assert torch.equal(it[5], want[j]), (graph, specs[j])
+            it[5].fill_(-1)
+        b.launch()  # a replay writes the same bits
+        torch.cuda.synchronize()
+        for j, it in enumerate(items):
+            assert torch.equal(it[5], want[j]), (graph, specs[j])
+            it[5].fill_(-1)
+        b.close()
+    cm_ctx.device_status()

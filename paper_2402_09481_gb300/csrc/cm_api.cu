@@ -718,6 +718,7 @@ void gf_shape(int kind, uint64_t n, uint64_t m, gf::Product *p, gf::Ops *q) {
 // transforms keeps the integer ones).  Measured, us a call, binary / integer:
 // 2^23 206 / 153, 2^24 216 / 307, 2^25 245 / 722, 2^26 517 / 2565, 2^28
 // 1812 / 10659: below 2^24 too few tiles to fill the GPU.
+// Products of up to 2^13 terms run densely in one launch (cm_gf2_dense.cu).
 constexpr int kGfMinLg = 24;
 
 bool gf_allowed(const cm_ctx *ctx) {
@@ -725,17 +726,18 @@ bool gf_allowed(const cm_ctx *ctx) {
     return o.fields == kFieldsAll && o.max_lg == 32 && !o.max_sum && !o.single;
 }
 
-static bool gf_applies(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m) {
-    if (!gf_allowed(ctx)) return false;
-    if (n > kMaxBits || m > kMaxBits) return false;
-    const uint64_t K = kind == CM_CIRCULANT ? n + 1 : n;
-    return K + m > (1ull << (kGfMinLg - 1)) + 1 && valid_args(kind, n, m);
-}
-
 cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t budget, Route *r) {
     r->kind = kind;
     r->n = n;
-    if (gf_applies(ctx, kind, n, m)) {
+    r->m = m;
+    const uint64_t terms = (kind == CM_CIRCULANT ? n + 1 : n) + m - 1;
+    if (gf_allowed(ctx) && n - 1 < kMaxBits && m - 1 < kMaxBits &&
+        (terms <= 1ull << gf::kDenseMaxLg || terms > 1ull << (kGfMinLg - 1)) && valid_args(kind, n, m)) {
+        if (terms <= 1ull << gf::kDenseMaxLg) {
+            gf_maps(kind, n, m, &r->ops);
+            r->dense = true;
+            return CM_OK;
+        }
         gf_shape(kind, n, m, &r->prod, &r->ops);
         gf_maps(kind, n, m, &r->ops);
         r->pre_off = gf::product_scratch(r->prod, r->ops);
@@ -751,6 +753,14 @@ cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64
 cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t *y, uint64_t *z, void *scratch,
                                cudaStream_t st) {
     uint8_t *sc = static_cast<uint8_t *>(scratch);
+    if (r.dense) {
+        r.ops.a0.map.src = x;
+        r.ops.b0.map.src = y;
+        ProfScope ps(ctx, "k_gf_dense", st);
+        return cuda_status(gf::launch_dense(r.ops.a0.map, r.ops.b0.map, (uint32_t)(r.kind == CM_CIRCULANT ? r.n + 1 : r.n),
+                                            (uint32_t)r.m, r.kind == CM_DODIS, z, ctx->d_status,
+                                            sc ? reinterpret_cast<uint32_t *>(sc + r.pre_off) : nullptr, st));
+    }
     if (!r.gf) return enqueue_blocks(ctx, r.bl, x, y, z, sc, r.tmp_off, r.pre_off, st);
     r.ops.a0.map.src = x;
     r.ops.b0.map.src = y;
@@ -1222,11 +1232,12 @@ extern "C" cm_status cm_extract_host(cm_ctx *ctx, int kind, const uint64_t *xh, 
     if (!valid_args(kind, n, m)) return CM_EINVAL;
     const uint64_t ybits = kind == CM_TOEPLITZ ? n + m - 1 : (kind == CM_CIRCULANT ? n + 1 : n);
     const uint64_t xw = words_of(n), yw = words_of(ybits), zw = words_of(m);
-    const uint64_t io = 8 * (xw + yw + zw) + 3 * 256 + 255;
+    const uint64_t io = 8 * (xw + yw + zw) + 4 * 256 + 255;
     if (io > ctx->budget) return CM_ENOMEM;
     Route r;
     cm_status s = make_route(ctx, kind, n, m, ctx->budget - io, &r);
     if (s != CM_OK) return s;
+    if (r.dense) r.need = kFlagBytes;  // Dodis et al. flags, read back below
     const uint64_t sbr = (r.need + 255) & ~255ull;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return CM_EDEVICE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -66,6 +66,13 @@ cudaError_t launch_same(const SameOp *ops, uint32_t count, cudaStream_t st);
 // Kernel launches of a product.
 uint32_t product_launches(const Product &p, const Ops &ops);
 
+// z = the m outputs of K terms, K + m - 1 <= 2^13, in one launch (cm_gf2_dense.cu);
+// check: a is a Dodis et al. input, all of it; pre (may be null): its flags,
+// pre[0] == 0 without a 1 bit, pre[1] == 0 without a 0 bit.
+constexpr int kDenseMaxLg = 13;
+cudaError_t launch_dense(const BitMap &a, const BitMap &b, uint32_t K, uint32_t m, bool check, uint64_t *z,
+                         uint32_t *status, uint32_t *pre, cudaStream_t st);
+
 // Host image of the device tables.
 constexpr int kTables = 2 * (kMaxLg - kMinLg + 1);
 void build_tables(Pass *t);  // kTables entries

@@ -10,11 +10,11 @@
 namespace cm {
 
 struct Route {
-    bool gf = false;
+    bool gf = false, dense = false;
     gf::Product prod;
     gf::Ops ops;  // pointers filled in by enqueue_route
     int kind;
-    uint64_t n;
+    uint64_t n, m;
     std::vector<Block> bl;
     uint64_t need = 0, tmp_off = 0, pre_off = 0;  // scratch bytes; offsets in it
 };

@@ -140,3 +140,36 @@ def test_batch_every_length_matches(cm_ctx, q30):
             it[5].fill_(-1)
         b.close()
     cm_ctx.device_status()
+
+
+DENSE = [(T, 1, 1), (T, 33, 31), (T, 1, 8192), (T, 8192, 1), (T, 4096, 2048), (T, 4095, 4098), (T, 1025, 63),
+         (C, 1000, 500), (C, 5000, 3100), (D, 30, 29), (D, 4093, 4093), (D, 8000, 65)]
+
+
+@pytest.mark.parametrize("kind,n,m", DENSE)
+def test_dense_form_matches(cm_ctx, q30, kind, n, m):
+    # products of up to 2^13 terms: one launch, every output against the oracle
+    n, m = resolve(kind, n, m)
+    xw, yw = inputs.bernoulli_half(41 + n, n), inputs.bernoulli_half(42 + m, ybits(kind, n, m))
+    if kind == D:
+        xw[0] = (xw[0] | np.uint64(1)) & ~np.uint64(2)
+    x, y = to_dev(xw), to_dev(yw)
+    cm_ctx.profile_enable(True)
+    cm_ctx.profile_read(reset=True)
+    z = run(cm_ctx, kind, n, m, x, y)
+    prof = cm_ctx.profile_read(reset=True)
+    cm_ctx.profile_enable(False)
+    assert prof["k_gf_dense"][0] == 1 and len(prof) == 1
+    want = {T: lambda: oracle.toeplitz_packed(xw, n, yw, m), C: lambda: oracle.circulant_packed(xw, n, yw, m),
+            D: lambda: oracle.dodis_packed(xw, yw, n, m)}[kind]()
+    assert (from_dev(z) == want).all()
+    zh = torch.zeros(native.words(m), dtype=torch.int64)
+    assert cm_ctx.extract_host(kind, x.cpu(), n, y.cpu(), m, zh) == native.CM_OK
+    assert (zh.numpy().view(np.uint64) == want).all()
+    if kind == D:
+        for fill in (0, 1):
+            c = ex.pack_bits(np.full(n, fill, dtype=np.uint8))
+            assert not from_dev(run(cm_ctx, D, n, m, to_dev(c), y)).any()
+            assert cm_ctx.device_status()[0] == native.CM_EPRECOND
+            assert cm_ctx.extract_host(D, torch.from_numpy(c.view(np.int64)), n, y.cpu(), m, zh) == native.CM_EPRECOND
+            cm_ctx.device_status()

@@ -822,7 +822,7 @@ def run_batched_b(args, world, rank, local):
     prof = ctx.profile_read(reset=True)
     ctx.profile_enable(False)
     kname = {native.ENGINE_GF2: "k_ss_gf2", native.ENGINE_BMMA: "k_ss_bmma",
-             native.ENGINE_F8: "k_ss_f8"}.get(engine, "k_ss_imma")
+             native.ENGINE_F4: "k_ss_f4"}.get(engine, "k_ss_imma")
     c_, t_ = prof[kname]
     per_launch = t_ / c_
     clocks = sampler.summary(tw0, tw1)
@@ -845,10 +845,10 @@ def run_batched_b(args, world, rank, local):
                 "traffic": ncu_traffic(kname, "batched_b"),
                 "b1_tensor_ops": {"value": count * m * n / (per_launch * 1e-3) / 1e12, "unit": "T bit-AND-POPC/s",
                                   "note": "no measured or nominal peak for b1 MMA on this GPU"}}
-    elif engine == native.ENGINE_F8:
-        ops = 2 * count * m * n               # e4m3 multiply-adds of the counts
-        roof = {"bound": "tensor", "kernel": kname, "achieved": ops / (per_launch * 1e-3) / 1e12, "peak": 4500.0,
-                "unit": "TFLOP/s", "frac": ops / (per_launch * 1e-3) / 4.5e15, "peak_source": "nominal dense fp8",
+    elif engine == native.ENGINE_F4:
+        ops = 2 * count * m * n               # e2m1 multiply-adds of the counts
+        roof = {"bound": "tensor", "kernel": kname, "achieved": ops / (per_launch * 1e-3) / 1e12, "peak": 13500.0,
+                "unit": "TFLOP/s", "frac": ops / (per_launch * 1e-3) / 13.5e15, "peak_source": "nominal dense fp4",
                 "traffic": ncu_traffic(kname, "batched_b"), "avg_launch_ms": per_launch}
     else:
         ops = 2 * count * m * n
@@ -889,10 +889,10 @@ def run_batched_b(args, world, rank, local):
             "metric": "extracted output Gbit/s", "value": value, "unit": "Gbit/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_per_step,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": {native.ENGINE_GF2: "u32 (GF(2) words)",
-                                                                 native.ENGINE_BMMA: "b1", native.ENGINE_F8: "e4m3 (exact 0/1 counts in f32)"}.get(engine, "s8"),
+                                                                 native.ENGINE_BMMA: "b1", native.ENGINE_F4: "e2m1 (exact 0/1 counts in f32)"}.get(engine, "s8"),
             "data": "synthetic",
             "config": {"workload": f"Shared Toeplitz seed: {count} inputs of n = 4096 bits, m = 2048, "
-                                   "Bernoulli(1/2)", "engine": {1: "imma", 2: "gf2", 3: "bmma", 4: "f8"}.get(engine),
+                                   "Bernoulli(1/2)", "engine": {1: "imma", 2: "gf2", 3: "bmma", 4: "f4"}.get(engine),
                        "l2": "inputs (%d MB) larger than L2" % (8 * X.size >> 20),
                        "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
             "compare": others, "latency_ms": {"p50": statistics.median(step_ms), "p99": max(step_ms)},

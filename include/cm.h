@@ -317,11 +317,11 @@ cm_status cm_batch_toeplitz(cm_ctx *ctx, const cm_desc *descs, uint32_t count, c
 
 /* ----- many inputs under one shared Toeplitz seed ------------------------- */
 
-#define CM_ENGINE_AUTO 0 /* long calls: CM_ENGINE_F8; else the fastest of 1 .. 3, timed on the first call of an (n, m) */
+#define CM_ENGINE_AUTO 0 /* long calls: CM_ENGINE_F4; else the fastest of 1 .. 3, timed on the first call of an (n, m) */
 #define CM_ENGINE_IMMA 1 /* INT8 tensor cores (mma.sync s8 x s8 -> s32), mod-2 epilogue */
 #define CM_ENGINE_GF2 2  /* CUDA cores: XOR of AND over packed words, parity epilogue */
 #define CM_ENGINE_BMMA 3 /* binary tensor cores (mma.sync b1 x b1 -> s32, AND-POPC), mod-2 epilogue */
-#define CM_ENGINE_F8 4   /* tcgen05 e4m3 product of 0 / 1 operands, exact float counts, parity epilogue; n <= 2^14 */
+#define CM_ENGINE_F4 4   /* tcgen05 e2m1 product of 0 / 1 operands, exact float counts, parity epilogue; n <= 2^14 */
 
 /*
  * Z_c = toep(y) X_c over GF(2) for c < count: the Toeplitz extractor of Eq.
@@ -335,11 +335,11 @@ cm_status cm_batch_toeplitz(cm_ctx *ctx, const cm_desc *descs, uint32_t count, c
  * its seeded extractor with the seed reused, which Section "Useful theorems
  * and results" permits for strong extractors.
  * Requires 1 <= n, m <= 2^24, n * m <= 2^34, 1 <= count <= 2^31, engine one
- * of CM_ENGINE_*, n <= 2^14 for CM_ENGINE_F8; CM_EINVAL otherwise.
- * CM_ENGINE_AUTO takes CM_ENGINE_F8 for n <= 2^14 and n * m * count >= 2^30
+ * of CM_ENGINE_*, n <= 2^14 for CM_ENGINE_F4; CM_EINVAL otherwise.
+ * CM_ENGINE_AUTO takes CM_ENGINE_F4 for n <= 2^14 and n * m * count >= 2^30
  * where its matrix fits the budget.  Scratch: the expanded matrix from the
- * context pool, ceil(m/64)*64 * ceil(n/1024)*1024 / 8 bytes, for CM_ENGINE_F8
- * ceil(m/256)*256 * ceil(n/128)*128 bytes.
+ * context pool, ceil(m/64)*64 * ceil(n/1024)*1024 / 8 bytes, for CM_ENGINE_F4
+ * ceil(m/224)*224 * ceil(n/256)*128 bytes.
  */
 cm_status cm_batch_toeplitz_shared_seed(cm_ctx *ctx, const uint64_t *y, uint64_t n, uint64_t m,
                                         const uint64_t *X, uint64_t count, uint64_t *Z, int engine,

@@ -33,7 +33,7 @@
 #include "cm.h"
 #include "cm_ctx.h"
 #include "cm_internal.h"
-#include "cm_ss_f8.h"
+#include "cm_ss_f4.h"
 
 namespace cm {
 namespace {
@@ -345,9 +345,9 @@ k_ss_bmma(const uint32_t *__restrict__ T, uint32_t rows_pad, uint32_t words_pad,
 
 // CM_ENGINE_AUTO takes the tcgen05 engine for this many bit products or more.
 // Measured, us a call, CUDA cores / tcgen05 (n x m x count): 4096 x 2048 x 65536
-// 1309 / 369, 8000 x 6000 x 300 169 / 76, 4096 x 2048 x 300 58 / 38, 1000 x 300 x
-// 4096 (2^30.2) 22.3 / 19.6; below, either is launch latency.
-constexpr double kSsF8Min = 1073741824.0;
+// 1309 / 232, 8000 x 6000 x 300 169 / 44, 4096 x 2048 x 300 59 / 28, 1000 x 300 x
+// 4096 (2^30.2) 22.3 / 16.6; below, either is launch latency.
+constexpr double kSsF4Min = 1073741824.0;
 
 std::mutex g_engine_mu;
 // (n, m, engine asked for) -> the variant the first call of that shape timed fastest
@@ -359,9 +359,9 @@ std::map<std::pair<uint64_t, uint64_t>, int> g_engine_wide;
 // Engine variants the autotuner times: the INT8 engine, the GF(2) engine
 // with 4 or 2 instances per thread, and the binary engine with 64- or 128-row
 // tiles.
-constexpr int kVarImma = 0, kVarGf2x4 = 1, kVarGf2x2 = 2, kVarBmma64 = 3, kVarBmma128 = 4, kVarF8 = 5;
+constexpr int kVarImma = 0, kVarGf2x4 = 1, kVarGf2x2 = 2, kVarBmma64 = 3, kVarBmma128 = 4, kVarF4 = 5;
 inline int engine_of(int var) {
-    if (var == kVarF8) return CM_ENGINE_F8;
+    if (var == kVarF4) return CM_ENGINE_F4;
     return var == kVarImma ? CM_ENGINE_IMMA : (var >= kVarBmma64 ? CM_ENGINE_BMMA : CM_ENGINE_GF2);
 }
 
@@ -402,38 +402,38 @@ extern "C" cm_status cm_batch_toeplitz_shared_seed(cm_ctx *ctx, const uint64_t *
                                                    int engine, cm_stream stream) {
     if (!ctx || !y || !X || !Z || n == 0 || m == 0 || count == 0) return CM_EINVAL;
     if (engine != CM_ENGINE_AUTO && engine != CM_ENGINE_IMMA && engine != CM_ENGINE_GF2 && engine != CM_ENGINE_BMMA &&
-        engine != CM_ENGINE_F8)
+        engine != CM_ENGINE_F4)
         return CM_EINVAL;
     if (n > (1ull << 24) || m > (1ull << 24) || (n * m) > (1ull << 34) || count > (1ull << 31))
         return CM_EINVAL;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return CM_EDEVICE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (engine == CM_ENGINE_F8 && n > kSsF8MaxN) return CM_EINVAL;
-    if (engine == CM_ENGINE_F8 ||
-        (engine == CM_ENGINE_AUTO && n <= kSsF8MaxN && ss_f8_bytes(n, m) <= ctx->budget &&
-         (double)n * (double)m * (double)count >= kSsF8Min)) {
-        const uint64_t tb = ss_f8_bytes(n, m);
+    if (engine == CM_ENGINE_F4 && n > kSsF4MaxN) return CM_EINVAL;
+    if (engine == CM_ENGINE_F4 ||
+        (engine == CM_ENGINE_AUTO && n <= kSsF4MaxN && ss_f4_bytes(n, m) <= ctx->budget &&
+         (double)n * (double)m * (double)count >= kSsF4Min)) {
+        const uint64_t tb = ss_f4_bytes(n, m);
         if (tb > ctx->budget) return CM_ENOMEM;
         void *Tf = nullptr;
         if (cudaMallocFromPoolAsync(&Tf, tb, ctx->pool, st) == cudaSuccess) {
             cudaError_t e;
             {
-                ProfScope ps(ctx, "k_ss_f8_rows", st);
-                e = launch_ss_f8_rows(y, n, m, Tf, ctx->nsm, st);
+                ProfScope ps(ctx, "k_ss_f4_rows", st);
+                e = launch_ss_f4_rows(y, n, m, Tf, ctx->nsm, st);
             }
             if (e == cudaSuccess) {
-                ProfScope ps(ctx, "k_ss_f8", st);
-                e = launch_ss_f8(Tf, n, m, X, count, Z, ctx->d_status, ctx->nsm, st);
+                ProfScope ps(ctx, "k_ss_f4", st);
+                e = launch_ss_f4(Tf, n, m, X, count, Z, ctx->d_status, ctx->nsm, st);
             }
             cudaFreeAsync(Tf, st);
             if (engine == CM_ENGINE_AUTO) {
                 std::lock_guard<std::mutex> lock(g_engine_mu);
-                g_engine_wide[{n, m}] = kVarF8;
+                g_engine_wide[{n, m}] = kVarF4;
             }
             return e == cudaSuccess ? CM_OK : CM_EDEVICE;
         }
         cudaGetLastError();
-        if (engine == CM_ENGINE_F8) return CM_ENOMEM;
+        if (engine == CM_ENGINE_F4) return CM_ENOMEM;
     }
     const uint32_t rows_pad = (uint32_t)((m + kSsRows - 1) / kSsRows * kSsRows);
     const uint32_t words_pad = (uint32_t)((n + 32 * kSsKw - 1) / (32 * kSsKw) * kSsKw);
@@ -506,7 +506,7 @@ extern "C" cm_status cm_batch_toeplitz_shared_seed(cm_ctx *ctx, const uint64_t *
 
 extern "C" int cm_shared_seed_engine(uint64_t n, uint64_t m) {
     std::lock_guard<std::mutex> lock(g_engine_mu);
-    if (g_engine_wide.count({n, m})) return CM_ENGINE_F8;
+    if (g_engine_wide.count({n, m})) return CM_ENGINE_F4;
     auto it = g_engine_choice.find(std::make_tuple(n, m, (int)CM_ENGINE_AUTO));
     if (it == g_engine_choice.end()) return CM_ENGINE_AUTO;
     return engine_of(it->second);

@@ -1,25 +1,27 @@
 // Many inputs under one Toeplitz seed on the 5th-generation tensor cores:
-// Z = toep(y) X as an e4m3 product with 0 / 1 operands (tcgen05.mma
-// kind::f8f6f4, float accumulators in tensor memory), parities in the epilogue.
+// Z = toep(y) X as an e2m1 product with 0 / 1 operands (tcgen05.mma kind::mxf4,
+// every block scale 1, float accumulators in tensor memory), parities in the
+// epilogue.
 //
-// sm_103a has no integer tcgen05 kind, but counts are exact in float: an input
-// bit is 2^-6 (byte 0x08, so that a shift and a mask make four elements), a
-// matrix bit 1.0 (0x38), and the epilogue adds 2^17, whose unit in the last
-// place is 2^-6: bit 0 of the word is the count's parity.
+// sm_103a has no integer tcgen05 kind, but counts are exact in float: a bit is
+// 0.5 (nibble 1, so that a shift and a mask make eight elements), products are
+// 0.25, and the epilogue adds 2^21, whose unit in the last place is 0.25: bit 0
+// of the word is the count's parity.
 //
-// A CTA makes 256 inputs x 256 outputs: two accumulators of 128 x 256 (all 512
-// columns of tensor memory), 128 columns of K a stage, three stages.
-//   warps 4..11  one input row a thread: 128 bits -> 128 bytes, swizzled to
-//                shared memory (16 shift/mask pairs per 32 bits)
+// A CTA makes 256 inputs x 224 outputs: two accumulators of 128 x 224 and 64
+// columns of scales fill tensor memory; 256 columns of K a stage, three stages.
+//   warps 4..11  input bits -> nibbles, swizzled to shared memory (a shift and a
+//                mask per eight elements)
 //   warp 12      bulk copies of the matrix, expanded once per call into the
-//                swizzled order of its shared-memory tiles (32 KB a stage)
-//   warp 13      issues the MMAs (2 x 4 of 128 x 256 x 32 a stage)
-//   warps 0..3   accumulators -> parity words, 32 bytes a row
-// Elements lie along K in the order the cheap expansion gives (bit q + 8 b of a
-// 32-bit word at byte 4 q + b) in both operands.  Shared-memory traffic bounds
-// it (operands in, operands out for two MMAs: about 40 KB per 284 cycles of
-// MMA at the e4m3 rate).  65536 inputs of 4096 bits, m = 2048: 369 us, 3.0 PFLOP/s
-// (the CUDA-core engine, AND / XOR on words: 1309 us).
+//                swizzled order of its shared-memory tiles (28 KB a stage)
+//   warp 13      issues the MMAs (2 x 4 of 128 x 224 x 64 a stage)
+//   warps 0..3   accumulators -> parity words, 28 bytes a row
+// Elements lie along K in the order the cheap expansion gives (bit q + 4 b of a
+// 32-bit word at nibble b of word q) in both operands.  Shared-memory traffic
+// bounds it (operands in and, for two MMAs, out again: 37 KB per step of K = 64).
+// 65536 inputs of 4096 bits, m = 2048: 232 us, 4.7 PFLOP/s (the CUDA-core engine,
+// AND / XOR on words: 1309 us; an e4m3 form of this kernel: 369 us; input loads a
+// row a lane instead of eight rows a warp: 305 us).
 //
 // Every wait has a limit, after which the kernel records CM_FLAG_TIMEOUT and
 // ends.
@@ -27,16 +29,19 @@
 #include <stdint.h>
 
 #include "cm_internal.h"
-#include "cm_ss_f8.h"
+#include "cm_ss_f4.h"
 
 namespace cm {
 
 namespace {
 
-constexpr int kStages = 3, kChunk = 128;
-constexpr int kTileBytes = 256 * kChunk;                 // one operand's stage
-constexpr int kSmem = kStages * 2 * kTileBytes + 1024;   // 1 KB to align
-constexpr int kF8Threads = 14 * 32;
+constexpr int kStages = 3, kChunk = 256;              // K elements a stage: rows of 128 bytes
+constexpr int kRows = 224;                            // outputs a CTA
+constexpr int kInBytes = 256 * 128, kTileBytes = kRows * 128;
+constexpr int kStageBytes = kInBytes + kTileBytes;
+constexpr int kSmem = kStages * kStageBytes + 1024;   // 1 KB to align
+constexpr uint32_t kScaleCol = 2 * kRows;             // tensor memory columns of scales
+constexpr int kF4Threads = 14 * 32;
 constexpr uint64_t kWaitNs = 2000000000ull;
 
 __device__ __forceinline__ uint32_t saddr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -81,14 +86,14 @@ __device__ __forceinline__ uint64_t operand(uint32_t addr) {
     return (uint64_t)((addr & 0x3FFFFu) >> 4) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
 }
 
-// e4m3 x e4m3 -> f32, M = 128, N = 256, both operands K-major.
-constexpr uint32_t kInstr = (1u << 4) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
+// e2m1 x e2m1 -> f32, ue8m0 scales, M = 128, N = 224, both operands K-major.
+constexpr uint32_t kInstr = (1u << 7) | (1u << 10) | ((uint32_t)(kRows >> 3) << 17) | (1u << 23) | ((128u >> 4) << 24);
 
-__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, bool add) {
+__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t scale, bool add) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-        "l"(a), "l"(b), "r"(kInstr), "r"((uint32_t)add)
+        " tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%5], [%5], p;\n}" ::"r"(d),
+        "l"(a), "l"(b), "r"(kInstr), "r"((uint32_t)add), "r"(scale)
         : "memory");
 }
 
@@ -96,9 +101,9 @@ __device__ __forceinline__ void commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-__global__ void __launch_bounds__(kF8Threads, 1) k_ss_f8(const uint8_t *__restrict__ T, uint32_t chunks, uint32_t pblocks,
+__global__ void __launch_bounds__(kF4Threads, 1) k_ss_f4(const uint8_t *__restrict__ T, uint32_t chunks, uint32_t pblocks,
                                                        const uint64_t *__restrict__ X, uint64_t n, uint64_t wx,
-                                                       uint64_t count, uint64_t *__restrict__ Z, uint64_t m,
+                                                       uint64_t count, uint64_t *__restrict__ Z,
                                                        uint64_t wz, uint64_t units, uint32_t *status) {
     extern __shared__ uint8_t raw[];
     __shared__ __align__(8) uint64_t bars[2 * kStages + 2];
@@ -127,41 +132,55 @@ __global__ void __launch_bounds__(kF8Threads, 1) k_ss_f8(const uint8_t *__restri
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_at;
+    if (warp < 4) {  // every scale 1.0 (127), whatever row and block it is read for
+#pragma unroll 1
+        for (uint32_t c = 0; c < 64; c += 8)
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(
+                             tmem + ((warp * 32u) << 16) + kScaleCol + c),
+                         "r"(0x7F7F7F7Fu)
+                         : "memory");
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
     if (warp >= 4 && warp < 12) {
-        const uint32_t r = threadIdx.x - 128;  // input row of the CTA's 256
+        // rows 8 i + lane / 4 of the warp's 32, 64-bit word lane % 4 of a stage's
+        // four: a load touches 8 rows' sectors, a store 8 distinct 16-byte pieces
+        const uint32_t r0 = (warp - 4) * 32 + (lane >> 2), q = lane & 3u;
         uint32_t it = 0;
         bool ok = true;
         for (uint64_t u = blockIdx.x; u < units && ok; u += gridDim.x) {
-            const uint64_t c = u / pblocks * 256 + r;
-            const uint64_t *row = X + c * wx;
-            auto load = [&](uint32_t k, uint64_t (&w)[2]) {
+            const uint64_t c0 = u / pblocks * 256 + r0;
+            const uint64_t *row = X + c0 * wx + q;
+            auto load = [&](uint32_t k, uint64_t (&w)[4]) {
+                const uint64_t j = 4ull * k + q;
+                const uint64_t keep = j + 1 < wx ? ~0ull : j < wx ? ((n & 63) ? (1ull << (n & 63)) - 1 : ~0ull) : 0ull;
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const uint64_t j = 2ull * k + i;
-                    w[i] = c < count && j < wx ? __ldg(row + j) : 0ull;
-                    if (j < wx && n - 64 * j < 64) w[i] &= (1ull << (n - 64 * j)) - 1;
-                }
+                for (int i = 0; i < 4; ++i)
+                    w[i] = keep && c0 + 8 * i < count ? __ldg(row + 8 * i * wx + 4ull * k) & keep : 0ull;
             };
-            uint64_t w[2], nx[2];
+            uint64_t w[4], nx[4];
             load(0, w);
             for (uint32_t k = 0; k < chunks; ++k, ++it) {
                 if (k + 1 < chunks) load(k + 1, nx);
                 const uint32_t s = it % kStages, ph = (it / kStages) & 1u;
                 if (!(ok = wait(empty + 8 * s, ph ^ 1u, &dead))) break;
-                uint8_t *dst = base + s * 2 * kTileBytes + r * 128;
+                uint8_t *dst = base + s * kStageBytes + r0 * 128;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const uint32_t b = (uint32_t)(w[j >> 2] >> (32 * ((j >> 1) & 1)));
-                    uint4 v;
-                    if (j & 1) v = make_uint4((b >> 1) & 0x08080808u, (b >> 2) & 0x08080808u, (b >> 3) & 0x08080808u, (b >> 4) & 0x08080808u);
-                    else v = make_uint4((b << 3) & 0x08080808u, (b << 2) & 0x08080808u, (b << 1) & 0x08080808u, b & 0x08080808u);
-                    *reinterpret_cast<uint4 *>(dst + ((j ^ (r & 7u)) << 4)) = v;
-                }
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t b = (uint32_t)(w[i] >> (32 * h));
+                        *reinterpret_cast<uint4 *>(dst + i * 1024 + (((2 * q + h) ^ (r0 & 7u)) << 4)) =
+                            make_uint4(b & 0x11111111u, (b >> 1) & 0x11111111u, (b >> 2) & 0x11111111u,
+                                       (b >> 3) & 0x11111111u);
+                    }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 arrive(full + 8 * s);
-                w[0] = nx[0];
-                w[1] = nx[1];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) w[i] = nx[i];
             }
         }
     } else if (warp == 12 && lane == 0) {
@@ -175,7 +194,7 @@ __global__ void __launch_bounds__(kF8Threads, 1) k_ss_f8(const uint8_t *__restri
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full + 8 * s), "r"(kTileBytes) : "memory");
                 asm volatile(
                     "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                        saddr(base + (s * 2 + 1) * kTileBytes)),
+                        saddr(base + s * kStageBytes + kInBytes)),
                     "l"(src + (uint64_t)k * kTileBytes), "r"(kTileBytes), "r"(full + 8 * s)
                     : "memory");
             }
@@ -190,12 +209,12 @@ __global__ void __launch_bounds__(kF8Threads, 1) k_ss_f8(const uint8_t *__restri
                 const uint32_t s = it % kStages, ph = (it / kStages) & 1u;
                 if (!(ok = wait(full + 8 * s, ph, &dead))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint64_t a = operand(saddr(base + s * 2 * kTileBytes)), a2 = operand(saddr(base + s * 2 * kTileBytes + kTileBytes / 2)),
-                               b = operand(saddr(base + (s * 2 + 1) * kTileBytes));
+                const uint32_t at = saddr(base + s * kStageBytes);
+                const uint64_t a = operand(at), a2 = operand(at + kInBytes / 2), b = operand(at + kInBytes);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {  // 32 bytes of K: 2 units of the descriptor's address
-                    mma(tmem, a + 2 * q, b + 2 * q, k || q);
-                    mma(tmem + 256, a2 + 2 * q, b + 2 * q, k || q);
+                    mma(tmem, a + 2 * q, b + 2 * q, tmem + kScaleCol, k || q);
+                    mma(tmem + kRows, a2 + 2 * q, b + 2 * q, tmem + kScaleCol, k || q);
                 }
                 commit(empty + 8 * s);
             }
@@ -210,11 +229,11 @@ __global__ void __launch_bounds__(kF8Threads, 1) k_ss_f8(const uint8_t *__restri
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {
                 const uint64_t c = u / pblocks * 256 + h * 128 + threadIdx.x;
-                uint32_t word[8];
+                uint32_t word[7];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
+                for (int q = 0; q < 7; ++q) {
                     uint32_t v[32];
-                    const uint32_t at = tmem + ((warp * 32u) << 16) + 256 * h + 32 * q;
+                    const uint32_t at = tmem + ((warp * 32u) << 16) + kRows * h + 32 * q;
                     asm volatile(
                         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
                         "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
@@ -227,19 +246,15 @@ __global__ void __launch_bounds__(kF8Threads, 1) k_ss_f8(const uint8_t *__restri
                     uint32_t o = 0;
 #pragma unroll
                     for (int j = 0; j < 32; ++j)
-                        o = __funnelshift_r(o, __float_as_uint(__uint_as_float(v[j]) + 131072.0f), 1);
+                        o = __funnelshift_r(o, __float_as_uint(__uint_as_float(v[j]) + 2097152.0f), 1);
                     word[q] = o;
                 }
                 if (c < count) {
+                    uint32_t *row = reinterpret_cast<uint32_t *>(Z + c * wz);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const uint64_t w = 4 * pb + q;
-                        uint64_t v = (uint64_t)word[2 * q + 1] << 32 | word[2 * q];
-                        if (w < wz) {
-                            if (m - 64 * w < 64) v &= (1ull << (m - 64 * w)) - 1;
-                            Z[c * wz + w] = v;
-                        }
-                    }
+                    for (int q = 0; q < 7; ++q)
+                        if (7 * pb + q < 2 * wz) row[7 * pb + q] = word[q];  // rows past m are 0 in the matrix
+                    if (7 * pb + 7 < 2 * wz && pb + 1 == pblocks) row[7 * pb + 7] = 0;
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -257,16 +272,17 @@ __global__ void __launch_bounds__(kF8Threads, 1) k_ss_f8(const uint8_t *__restri
     }
 }
 
-// The matrix in tile order: block (p, k) holds rows 256 p .. of the Toeplitz
-// matrix, columns 128 k .. as bytes, rows of 128 with their 16-byte pieces
+// The matrix in tile order: block (p, k) holds rows 224 p .. of the Toeplitz
+// matrix, columns 256 k .. as nibbles, rows of 128 bytes with their 16-byte pieces
 // exchanged by row mod 8.  One thread a row's 32 columns.
-__global__ void __launch_bounds__(256) k_ss_f8_rows(const uint32_t *__restrict__ y, uint64_t n, uint64_t m, uint32_t chunks,
+__global__ void __launch_bounds__(256) k_ss_f4_rows(const uint32_t *__restrict__ y, uint64_t n, uint64_t m, uint32_t chunks,
                                                     uint8_t *__restrict__ T, uint64_t total) {
     const uint64_t N = n + m - 1;
     for (uint64_t t = (uint64_t)blockIdx.x * 256 + threadIdx.x; t < total; t += (uint64_t)gridDim.x * 256) {
-        const uint32_t g = (uint32_t)(t & 3u), r = (uint32_t)(t >> 2) & 255u;
-        const uint64_t blk = t >> 10, p = blk / chunks, k = blk - p * chunks;
-        const uint64_t i = 256 * p + r, j0 = 128 * k + 32 * g;
+        const uint32_t g = (uint32_t)(t & 7u);
+        const uint64_t rr = t >> 3, blk = rr / kRows, p = blk / chunks, k = blk - p * chunks;
+        const uint32_t r = (uint32_t)(rr - blk * kRows);
+        const uint64_t i = kRows * p + r, j0 = (uint64_t)kChunk * k + 32 * g;
         uint32_t w = 0;  // bit t: y[(i - j0 - t) mod N]
         if (i < m && j0 < n) {
             const uint32_t cnt = n - j0 < 32 ? (uint32_t)(n - j0) : 32u;
@@ -288,40 +304,33 @@ __global__ void __launch_bounds__(256) k_ss_f8_rows(const uint32_t *__restrict__
             if (cnt < 32) w &= (1u << cnt) - 1u;
         }
         uint8_t *row = T + blk * kTileBytes + r * 128;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            uint4 v;
-            v.x = ((w >> (4 * h)) & 0x01010101u) * 0x38u;
-            v.y = ((w >> (4 * h + 1)) & 0x01010101u) * 0x38u;
-            v.z = ((w >> (4 * h + 2)) & 0x01010101u) * 0x38u;
-            v.w = ((w >> (4 * h + 3)) & 0x01010101u) * 0x38u;
-            *reinterpret_cast<uint4 *>(row + (((2 * g + h) ^ (r & 7u)) << 4)) = v;
-        }
+        *reinterpret_cast<uint4 *>(row + ((g ^ (r & 7u)) << 4)) =
+            make_uint4(w & 0x11111111u, (w >> 1) & 0x11111111u, (w >> 2) & 0x11111111u, (w >> 3) & 0x11111111u);
     }
 }
 
 }  // namespace
 
-uint64_t ss_f8_bytes(uint64_t n, uint64_t m) {
-    return (m + 255) / 256 * ((n + kChunk - 1) / kChunk) * kTileBytes;
+uint64_t ss_f4_bytes(uint64_t n, uint64_t m) {
+    return (m + kRows - 1) / kRows * ((n + kChunk - 1) / kChunk) * kTileBytes;
 }
 
-cudaError_t launch_ss_f8_rows(const uint64_t *y, uint64_t n, uint64_t m, void *T, int nsm, cudaStream_t st) {
-    const uint64_t total = ss_f8_bytes(n, m) / 32;
+cudaError_t launch_ss_f4_rows(const uint64_t *y, uint64_t n, uint64_t m, void *T, int nsm, cudaStream_t st) {
+    const uint64_t total = ss_f4_bytes(n, m) / 16;
     const uint64_t blocks = (total + 255) / 256, cap = (uint64_t)nsm * 16;
-    k_ss_f8_rows<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, st>>>(
+    k_ss_f4_rows<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, st>>>(
         reinterpret_cast<const uint32_t *>(y), n, m, (uint32_t)((n + kChunk - 1) / kChunk), static_cast<uint8_t *>(T), total);
     return cudaGetLastError();
 }
 
-cudaError_t launch_ss_f8(const void *T, uint64_t n, uint64_t m, const uint64_t *X, uint64_t count, uint64_t *Z,
+cudaError_t launch_ss_f4(const void *T, uint64_t n, uint64_t m, const uint64_t *X, uint64_t count, uint64_t *Z,
                          uint32_t *status, int nsm, cudaStream_t st) {
-    cudaError_t e = smem_attr_once<k_ss_f8>(kSmem);
+    cudaError_t e = smem_attr_once<k_ss_f4>(kSmem);
     if (e != cudaSuccess) return e;
-    const uint64_t pblocks = (m + 255) / 256, units = (count + 255) / 256 * pblocks;
-    k_ss_f8<<<(unsigned)(units < (uint64_t)nsm ? units : nsm), kF8Threads, kSmem, st>>>(
+    const uint64_t pblocks = (m + kRows - 1) / kRows, units = (count + 255) / 256 * pblocks;
+    k_ss_f4<<<(unsigned)(units < (uint64_t)nsm ? units : nsm), kF4Threads, kSmem, st>>>(
         static_cast<const uint8_t *>(T), (uint32_t)((n + kChunk - 1) / kChunk), (uint32_t)pblocks, X, n, (n + 63) / 64, count,
-        Z, m, (m + 63) / 64, units, status);
+        Z, (m + 63) / 64, units, status);
     return cudaGetLastError();
 }
 

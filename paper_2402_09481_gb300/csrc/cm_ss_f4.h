@@ -1,0 +1,17 @@
+// The shared-seed product on tcgen05 (cm_ss_f4.cu).
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace cm {
+
+// Longest input: its counts, all ones included, are checked exact in the
+// accumulator.
+constexpr uint64_t kSsF4MaxN = 1ull << 14;
+// Bytes of the expanded matrix.
+uint64_t ss_f4_bytes(uint64_t n, uint64_t m);
+cudaError_t launch_ss_f4_rows(const uint64_t *y, uint64_t n, uint64_t m, void *T, int nsm, cudaStream_t st);
+cudaError_t launch_ss_f4(const void *T, uint64_t n, uint64_t m, const uint64_t *X, uint64_t count, uint64_t *Z,
+                         uint32_t *status, int nsm, cudaStream_t st);
+
+}  // namespace cm

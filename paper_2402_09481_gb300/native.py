@@ -172,7 +172,7 @@ class ServerStats(ctypes.Structure):
 
 
 BATCH_AUTOTUNE, BATCH_NO_GRAPH, BATCH_TEST_STALL = 0x1, 0x2, 0x4
-ENGINE_AUTO, ENGINE_IMMA, ENGINE_GF2, ENGINE_BMMA, ENGINE_F8 = 0, 1, 2, 3, 4
+ENGINE_AUTO, ENGINE_IMMA, ENGINE_GF2, ENGINE_BMMA, ENGINE_F4 = 0, 1, 2, 3, 4
 
 
 class CMError(RuntimeError):

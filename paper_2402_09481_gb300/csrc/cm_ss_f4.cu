@@ -309,6 +309,19 @@ __global__ void __launch_bounds__(256) k_ss_f4_rows(const uint32_t *__restrict__
     }
 }
 
+__global__ void __launch_bounds__(256) k_ss_f4_pack(const uint32_t *__restrict__ G, uint64_t gw, uint64_t m, uint32_t chunks,
+                                                    uint8_t *__restrict__ T, uint64_t total) {
+    for (uint64_t t = (uint64_t)blockIdx.x * 256 + threadIdx.x; t < total; t += (uint64_t)gridDim.x * 256) {
+        const uint32_t g = (uint32_t)(t & 7u);
+        const uint64_t rr = t >> 3, blk = rr / kRows, p = blk / chunks, k = blk - p * chunks;
+        const uint32_t r = (uint32_t)(rr - blk * kRows);
+        const uint64_t i = kRows * p + r, j = 8 * k + g;
+        const uint32_t w = i < m && j < gw ? __ldg(G + i * gw + j) : 0u;
+        *reinterpret_cast<uint4 *>(T + blk * kTileBytes + r * 128 + ((g ^ (r & 7u)) << 4)) =
+            make_uint4(w & 0x11111111u, (w >> 1) & 0x11111111u, (w >> 2) & 0x11111111u, (w >> 3) & 0x11111111u);
+    }
+}
+
 }  // namespace
 
 uint64_t ss_f4_bytes(uint64_t n, uint64_t m) {
@@ -320,6 +333,13 @@ cudaError_t launch_ss_f4_rows(const uint64_t *y, uint64_t n, uint64_t m, void *T
     const uint64_t blocks = (total + 255) / 256, cap = (uint64_t)nsm * 16;
     k_ss_f4_rows<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, st>>>(
         reinterpret_cast<const uint32_t *>(y), n, m, (uint32_t)((n + kChunk - 1) / kChunk), static_cast<uint8_t *>(T), total);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_ss_f4_pack(const uint32_t *G, uint64_t gw, uint64_t n, uint64_t m, void *T, int nsm, cudaStream_t st) {
+    const uint64_t total = ss_f4_bytes(n, m) / 16, blocks = (total + 255) / 256, cap = (uint64_t)nsm * 16;
+    k_ss_f4_pack<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, st>>>(
+        G, gw, m, (uint32_t)((n + kChunk - 1) / kChunk), static_cast<uint8_t *>(T), total);
     return cudaGetLastError();
 }
 

@@ -16,6 +16,15 @@
 //     since every tap of the moduli up to l = 256 is at most (l + 1) / 2;
 //   - an XOR of the next chunk (pre-aligned by k_rsh_chunks).
 // The output bit is the parity of alpha2' AND p' (both aligned alike).
+//
+// Many outputs at once share the chunks, and multiplying by a chunk is a matrix
+// over GF(2): with s chunks in J groups of B, p = sum_j alpha1^(B j) r_j and
+// r_j = sum_i x_(jB+i) alpha1^i.  The r_j of all outputs are one product of a
+// (J l) x (B l) bit matrix of the chunks with the bits of alpha1^0 .. alpha1^(B-1)
+// (s l^2 bit products an output either way), which runs on the tensor cores as
+// the shared-seed product does (cm_ss_f4.cu); each output then takes B - 1
+// products for its powers and J for Horner's rule over the groups, where the
+// plain form takes s - 1.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -26,6 +35,7 @@
 
 #include "cm_ctx.h"
 #include "cm_internal.h"
+#include "cm_ss_f4.h"
 #include "cm_trevisan.h"
 
 namespace cm {
@@ -457,6 +467,175 @@ static cudaError_t launch_rsh_kernel(const uint64_t *X, uint64_t s, const uint64
     return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------
+// The grouped form.
+
+// Bits of alpha1^0 .. alpha1^(B-1) of each output, l each, back to back in rows
+// of wx words.
+template <int W, bool WIDE>
+__global__ void __launch_bounds__(kRshThreads)
+k_rsh_powers(const uint64_t *__restrict__ seeds, uint32_t l, uint64_t m, uint32_t t1, uint32_t t2, uint32_t t3,
+             int ntaps, uint32_t B, uint64_t wx, uint64_t *__restrict__ V) {
+    constexpr int WT = WIDE ? W + 1 : W;
+    extern __shared__ __align__(16) uint64_t T[];
+    const int tid = threadIdx.x;
+    const RshField F{t1, t2, t3, ntaps, l >> 6, l & 63, 64 * W - (int)l};
+    const uint64_t out = (uint64_t)blockIdx.x * kRshThreads + tid;
+    if (out >= m) return;
+    uint64_t a1[W], al[WT], p[W];
+    aligned_element<W>(seeds, 2ull * l * m, 2ull * l * out, l, a1);
+    to_plain<W, WT>(a1, F.delta, al);
+    build_table<WT>(T, tid, al);
+#pragma unroll
+    for (int q = 0; q < W; ++q) p[q] = q ? 0ull : 1ull << F.delta;
+    uint64_t *row = V + out * wx;
+    uint64_t acc = 0, w = 0;
+    uint32_t have = 0;
+    for (uint32_t i = 0; i < B; ++i) {
+        uint64_t e[W], r[W];
+        to_plain<W, W>(p, F.delta, e);
+#pragma unroll
+        for (int q = 0; q < W; ++q) {
+            const uint32_t c = l - 64u * q < 64u ? l - 64u * q : 64u;
+            acc |= e[q] << have;
+            if (have + c >= 64) {
+                row[w++] = acc;
+                acc = have ? e[q] >> (64 - have) : 0ull;
+                have = have + c - 64;
+            } else {
+                have += c;
+            }
+        }
+        if (i + 1 < B) {
+            mul_table<W, WT>(T, tid, F, p, r);
+#pragma unroll
+            for (int q = 0; q < W; ++q) p[q] = r[q];
+        }
+    }
+    if (have) row[w] = acc;
+}
+
+// Horner's rule over the groups: R holds r_0 .. r_(J-1) of each output, l bits
+// each, back to back in rows of wz words.
+template <int W, bool WIDE>
+__global__ void __launch_bounds__(kRshThreads)
+k_rsh_join(const uint64_t *__restrict__ R, uint64_t wz, const uint64_t *__restrict__ seeds, uint32_t l, uint64_t m,
+           uint32_t t1, uint32_t t2, uint32_t t3, int ntaps, uint32_t B, uint32_t J, uint32_t *__restrict__ z32) {
+    constexpr int WT = WIDE ? W + 1 : W;
+    extern __shared__ __align__(16) uint64_t T[];
+    const int tid = threadIdx.x;
+    const RshField F{t1, t2, t3, ntaps, l >> 6, l & 63, 64 * W - (int)l};
+    const uint64_t out = (uint64_t)blockIdx.x * kRshThreads + tid;
+    uint32_t par = 0;
+    if (out < m) {
+        uint64_t a1[W], a2[W], al[WT], beta[W], pa[W];
+        aligned_element<W>(seeds, 2ull * l * m, 2ull * l * out, l, a1);
+        aligned_element<W>(seeds, 2ull * l * m, 2ull * l * out + l, l, a2);
+        to_plain<W, WT>(a1, F.delta, al);
+        pow_aligned<W, WT>(T, tid, F, al, B, beta);
+        to_plain<W, WT>(beta, F.delta, al);
+        build_table<WT>(T, tid, al);
+        const uint64_t *row = R + out * wz;
+#pragma unroll
+        for (int q = 0; q < W; ++q) pa[q] = 0;
+        for (uint32_t j = J; j-- > 0;) {
+            uint64_t e[W], r[W];
+            if (j + 1 < J) mul_table<W, WT>(T, tid, F, pa, r);
+            else {
+#pragma unroll
+                for (int q = 0; q < W; ++q) r[q] = 0;
+            }
+#pragma unroll
+            for (int q = 0; q < W; ++q) {  // bits j l .. of the row, aligned
+                const uint32_t lo = 64u * q;
+                e[q] = bits64(row, (uint64_t)(j + 1) * l, (uint64_t)j * l + lo);
+            }
+#pragma unroll
+            for (int q = 0; q < W; ++q)
+                pa[q] = r[q] ^ (F.delta ? (e[q] << F.delta) | (q ? e[q - 1] >> (64 - F.delta) : 0ull) : e[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < W; ++q) par ^= __popcll(a2[q] & pa[q]) & 1u;
+    }
+    const uint32_t word = __ballot_sync(0xffffffffu, par);
+    if ((tid & 31) == 0 && out < (m + 63) / 64 * 64) z32[out >> 5] = word;
+}
+
+// Rows of the chunks' matrix: block (j, i) of l x l bits is multiplication by
+// chunk s - 1 - (j B + i) (zero past the chunks).  A warp makes one block, 32
+// columns (x z^b, one a lane) at a time, and exchanges them into rows.
+__global__ void __launch_bounds__(128) k_rsh_matrix(const uint64_t *__restrict__ X, int W, uint64_t s, uint32_t l,
+                                                    uint32_t t1, uint32_t t2, uint32_t t3, int ntaps, uint32_t B,
+                                                    uint32_t J, uint64_t gw, uint32_t *__restrict__ G) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint64_t blk = (uint64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (blk >= (uint64_t)B * J || blk >= s) return;  // the zero blocks stay as cleared
+    const uint32_t j = (uint32_t)(blk / B), i = (uint32_t)(blk - (uint64_t)j * B);
+    const int delta = 64 * W - (int)l;
+    uint64_t e[4] = {0, 0, 0, 0};
+    const uint64_t *src = X + (s - 1 - blk) * W;
+    for (int q = 0; q < W; ++q) {  // plain
+        uint64_t v = src[q] >> delta;
+        if (delta && q + 1 < W) v |= src[q + 1] << (64 - delta);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (k == q) e[k] = v;
+    }
+    const uint32_t lw = l >> 6, lb = l & 63;
+    auto step = [&](uint64_t (&p)[4]) {  // p <- p z mod f
+        const uint64_t c3 = p[2] >> 63, c2 = p[1] >> 63, c1 = p[0] >> 63, c4 = p[3] >> 63;
+        p[3] = p[3] << 1 | c3;
+        p[2] = p[2] << 1 | c2;
+        p[1] = p[1] << 1 | c1;
+        p[0] <<= 1;
+        uint64_t top = c4;  // l = 256: the bit shifted out
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (lw == (uint32_t)k) {
+                top = (p[k] >> lb) & 1ull;
+                p[k] &= ~(1ull << lb);
+            }
+        if (top) {
+            p[0] ^= 1ull;
+#pragma unroll
+            for (int n = 0; n < 3; ++n) {
+                const uint32_t t = n == 0 ? t1 : n == 1 ? t2 : t3;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (n < ntaps && (t >> 6) == (uint32_t)k) p[k] ^= 1ull << (t & 63);
+            }
+        }
+    };
+    for (uint32_t b0 = 0; b0 < l; b0 += 32) {
+        uint64_t p[4] = {e[0], e[1], e[2], e[3]};
+        for (uint32_t k = 0; k < 31; ++k)
+            if (k < lane) step(p);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            if (32u * q >= l) break;
+            uint32_t v = b0 + lane < l ? (uint32_t)(p[q >> 1] >> (32 * (q & 1))) : 0u;
+#pragma unroll
+            for (int b = 0; b < 5; ++b) {  // lane r ends with row 32 q + r of these columns
+                const uint32_t mk = b == 0 ? 0x55555555u : b == 1 ? 0x33333333u : b == 2 ? 0x0F0F0F0Fu : b == 3 ? 0x00FF00FFu : 0x0000FFFFu;
+                const int sh = 1 << b;
+                const uint32_t y = __shfl_xor_sync(0xffffffffu, v, sh);
+                v = (lane & sh) ? (v & ~mk) | ((y & ~mk) >> sh) : (v & mk) | ((y & mk) << sh);
+            }
+            const uint32_t r = 32u * q + lane;
+            if (r < l && v) {
+                const uint64_t at = (uint64_t)i * l + b0;
+                uint32_t *row = G + ((uint64_t)j * l + r) * gw + (at >> 5);
+                const uint32_t o = (uint32_t)at & 31u;
+                atomicOr(row, v << o);
+                if (o && (v >> (32 - o))) atomicOr(row + 1, v >> (32 - o));
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) e[k] = __shfl_sync(0xffffffffu, p[k], 31);
+        step(e);
+    }
+}
+
 // One-bit seeds from the weak design's sets: bit j < 2l of seed i is
 // y[sets[i * t + j]] (an index at or past d reads 0); seeds (zeroed first)
 // receive 2 l m bits.
@@ -524,10 +703,54 @@ static cudaError_t launch_rsh_w(const uint64_t *x, uint64_t n, uint32_t l, const
     }
 }
 
-static uint64_t rsh_scratch(uint64_t n, uint32_t l) {
+// The grouped form's shape and scratch: chunks, powers, matrix (packed, then in
+// tile order), group sums.
+struct RshGroups {
+    bool on = false;
+    uint32_t B = 0, J = 0;
+    uint64_t K = 0, rows = 0, wx = 0, wz = 0, gw = 0;
+    uint64_t v_off = 0, g_off = 0, t_off = 0, r_off = 0, bytes = 0;
+};
+
+static uint64_t rsh_chunk_bytes(uint64_t n, uint32_t l) {
     const int W = (int)((l + 63) / 64);
     const uint64_t s = (n + l - 1) / l;
     return (8ull * W * s + 255) & ~255ull;
+}
+
+// The grouped form is taken from 2^33 bit products on, for enough outputs that
+// its two field passes (one thread an output) are not its time, where its
+// scratch fits the budget.  Measured, ms, plain / grouped, (n, l, m): (2^20, 121,
+// 2^16) 15.35 / 3.89, of which the product on the tensor cores 3.24; (2^20, 121,
+// 4096) 0.89 / 0.64; (2^17, 100, 2^15) 1.04 / 0.35; (10^5, 200, 8192) 1.10 / 0.32;
+// (2^14, 121, 8192) 0.121 / 0.095; (2^14, 60, 2^14) 0.074 / 0.068.
+static RshGroups rsh_groups(uint64_t n, uint32_t l, uint64_t m, uint64_t budget) {
+    RshGroups g;
+    const uint64_t s = (n + l - 1) / l;
+    if (m < 4096 || s < 64 || (double)s * l * l * (double)m < 8589934592.0 || s > 1ull << 31 || m > 1ull << 31) return g;
+    uint64_t B = 1;
+    while (B * B < s) ++B;
+    if (B * l > kSsF4MaxN) B = kSsF4MaxN / l;
+    g.B = (uint32_t)B;
+    g.J = (uint32_t)((s + B - 1) / B);
+    g.K = B * l;
+    g.rows = (uint64_t)g.J * l;
+    g.wx = (g.K + 63) / 64;
+    g.wz = (g.rows + 63) / 64;
+    g.gw = 2 * g.wx;
+    auto r256 = [](uint64_t v) { return (v + 255) & ~255ull; };
+    g.v_off = rsh_chunk_bytes(n, l);
+    g.g_off = g.v_off + r256(8 * g.wx * m);
+    g.t_off = g.g_off + r256(4 * g.gw * g.rows);
+    g.r_off = g.t_off + r256(ss_f4_bytes(g.K, g.rows));
+    g.bytes = g.r_off + r256(8 * g.wz * m);
+    g.on = g.bytes <= budget;
+    return g;
+}
+
+static uint64_t rsh_scratch(uint64_t n, uint32_t l, uint64_t m, uint64_t budget) {
+    const RshGroups g = rsh_groups(n, l, m, budget);
+    return g.on ? g.bytes : rsh_chunk_bytes(n, l);
 }
 
 static cm_status cuda_st(cudaError_t e) {
@@ -536,14 +759,73 @@ static cm_status cuda_st(cudaError_t e) {
     return CM_EDEVICE;
 }
 
-// Enqueue the RSH extractions; scratch holds rsh_scratch(n, l) bytes.
+template <int W, bool WIDE>
+static cudaError_t launch_groups(cm_ctx *ctx, const RshGroups &g, const uint64_t *x, uint64_t n, uint32_t l,
+                                 const uint64_t *seeds, uint64_t m, uint64_t *z, const Modulus &md, uint8_t *sc,
+                                 cudaStream_t st) {
+    constexpr int WT = WIDE ? W + 1 : W;
+    const int smem = 16 * WT * kRshThreads * (int)sizeof(uint64_t);
+    const uint64_t s = (n + l - 1) / l;
+    uint64_t *X = reinterpret_cast<uint64_t *>(sc), *V = reinterpret_cast<uint64_t *>(sc + g.v_off),
+             *R = reinterpret_cast<uint64_t *>(sc + g.r_off);
+    uint32_t *G = reinterpret_cast<uint32_t *>(sc + g.g_off);
+    cudaError_t e;
+    if ((e = smem_attr_once<k_rsh_powers<W, WIDE>>(smem)) != cudaSuccess) return e;
+    if ((e = smem_attr_once<k_rsh_join<W, WIDE>>(smem)) != cudaSuccess) return e;
+    const uint64_t cb = (s + 255) / 256, cap = (uint64_t)ctx->nsm * 8;
+    const unsigned grid = (unsigned)(((m + 63) / 64 * 64 + kRshThreads - 1) / kRshThreads);
+    {
+        ProfScope ps(ctx, "k_rsh_matrix", st);
+        k_rsh_chunks<W><<<(unsigned)(cb < cap ? cb : cap), 256, 0, st>>>(x, n, l, s, X);
+        if ((e = cudaMemsetAsync(G, 0, 4 * g.gw * g.rows, st)) != cudaSuccess) return e;
+        k_rsh_matrix<<<(unsigned)(((uint64_t)g.B * g.J + 3) / 4), 128, 0, st>>>(
+            X, W, s, l, md.taps[0], md.taps[1], md.taps[2], (int)md.count, g.B, g.J, g.gw, G);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_ss_f4_pack(G, g.gw, g.K, g.rows, sc + g.t_off, ctx->nsm, st)) != cudaSuccess) return e;
+    }
+    {
+        ProfScope ps(ctx, "k_rsh_powers", st);
+        k_rsh_powers<W, WIDE><<<grid, kRshThreads, smem, st>>>(seeds, l, m, md.taps[0], md.taps[1], md.taps[2],
+                                                               (int)md.count, g.B, g.wx, V);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    {
+        ProfScope ps(ctx, "k_ss_f4", st);
+        if ((e = launch_ss_f4(sc + g.t_off, g.K, g.rows, V, m, R, ctx->d_status, ctx->nsm, st)) != cudaSuccess) return e;
+    }
+    ProfScope ps(ctx, "k_rsh_join", st);
+    k_rsh_join<W, WIDE><<<grid, kRshThreads, smem, st>>>(R, g.wz, seeds, l, m, md.taps[0], md.taps[1], md.taps[2],
+                                                         (int)md.count, g.B, g.J, reinterpret_cast<uint32_t *>(z));
+    return cudaGetLastError();
+}
+
+template <int W>
+static cudaError_t launch_groups_w(cm_ctx *ctx, const RshGroups &g, const uint64_t *x, uint64_t n, uint32_t l,
+                                   const uint64_t *seeds, uint64_t m, uint64_t *z, const Modulus &md, uint8_t *sc,
+                                   cudaStream_t st) {
+    return l + 3 > 64u * W ? launch_groups<W, true>(ctx, g, x, n, l, seeds, m, z, md, sc, st)
+                           : launch_groups<W, false>(ctx, g, x, n, l, seeds, m, z, md, sc, st);
+}
+
+// Enqueue the RSH extractions; scratch holds rsh_scratch(n, l, m, budget) bytes
+// for the budget given here.
 static cm_status enqueue_rsh(cm_ctx *ctx, const uint64_t *x, uint64_t n, uint32_t l, const uint64_t *seeds,
-                             uint64_t m, uint64_t *z, uint8_t *scratch, cudaStream_t st) {
+                             uint64_t m, uint64_t *z, uint8_t *scratch, uint64_t budget, cudaStream_t st) {
     Modulus md;
     if (!find_modulus(l, &md) || !taps_ok(l, md)) return CM_EINVAL;
     const int W = (int)((l + 63) / 64);
     uint64_t *X = reinterpret_cast<uint64_t *>(scratch);
     cudaError_t e;
+    const RshGroups g = rsh_groups(n, l, m, budget);
+    if (g.on) {
+        switch (W) {
+            case 1: e = launch_groups_w<1>(ctx, g, x, n, l, seeds, m, z, md, scratch, st); break;
+            case 2: e = launch_groups_w<2>(ctx, g, x, n, l, seeds, m, z, md, scratch, st); break;
+            case 3: e = launch_groups_w<3>(ctx, g, x, n, l, seeds, m, z, md, scratch, st); break;
+            default: e = launch_groups_w<4>(ctx, g, x, n, l, seeds, m, z, md, scratch, st); break;
+        }
+        return cuda_st(e);
+    }
     ProfScope ps(ctx, "k_rsh", st);
     switch (W) {
         case 1: e = launch_rsh_w<1>(x, n, l, seeds, m, z, X, md, ctx->nsm, st); break;
@@ -581,7 +863,7 @@ extern "C" cm_status cm_rsh_modulus(uint32_t l, uint32_t taps[3], uint32_t *coun
 extern "C" cm_status cm_trevisan_rsh(cm_ctx *ctx, const uint64_t *x, uint64_t n, uint32_t l, const uint64_t *seeds,
                                      uint64_t m, uint64_t *z, cm_stream stream) {
     if (!ctx || !rsh_args_ok(x, n, l, seeds, m, z)) return CM_EINVAL;
-    const uint64_t need = rsh_scratch(n, l);
+    const uint64_t need = rsh_scratch(n, l, m, ctx->budget);
     if (need > ctx->budget) return CM_ENOMEM;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return CM_EDEVICE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -590,7 +872,7 @@ extern "C" cm_status cm_trevisan_rsh(cm_ctx *ctx, const uint64_t *x, uint64_t n,
         cudaGetLastError();
         return CM_ENOMEM;
     }
-    cm_status s = enqueue_rsh(ctx, x, n, l, seeds, m, z, static_cast<uint8_t *>(sc), st);
+    cm_status s = enqueue_rsh(ctx, x, n, l, seeds, m, z, static_cast<uint8_t *>(sc), ctx->budget, st);
     if (cudaFreeAsync(sc, st) != cudaSuccess && s == CM_OK) s = CM_EDEVICE;
     return s;
 }
@@ -600,7 +882,9 @@ extern "C" cm_status cm_trevisan(cm_ctx *ctx, const uint64_t *x, uint64_t n, con
                                  cm_stream stream) {
     if (!ctx || !y || !sets || d == 0 || !rsh_args_ok(x, n, l, sets, m, z) || t < 2 * l) return CM_EINVAL;
     const uint64_t sb = (2ull * l * m + 63) / 64 * 8;
-    const uint64_t soff = (rsh_scratch(n, l) + 255) & ~255ull;
+    if (sb > ctx->budget) return CM_ENOMEM;
+    const uint64_t room = ctx->budget - sb >= 256 ? ctx->budget - sb - 255 : 0;
+    const uint64_t soff = (rsh_scratch(n, l, m, room) + 255) & ~255ull;
     const uint64_t need = soff + sb;
     if (need > ctx->budget) return CM_ENOMEM;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return CM_EDEVICE;
@@ -618,7 +902,7 @@ extern "C" cm_status cm_trevisan(cm_ctx *ctx, const uint64_t *x, uint64_t n, con
         k_gather_seeds<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(y, d, sets, t, l, m, seeds);
         s = cuda_st(cudaGetLastError());
     }
-    if (s == CM_OK) s = enqueue_rsh(ctx, x, n, l, seeds, m, z, b, st);
+    if (s == CM_OK) s = enqueue_rsh(ctx, x, n, l, seeds, m, z, b, room, st);
     if (cudaFreeAsync(sc, st) != cudaSuccess && s == CM_OK) s = CM_EDEVICE;
     return s;
 }

@@ -180,12 +180,12 @@ __device__ __forceinline__ bool constant_input(const OutOp &o, bool tell) {
 // column 0 the stages are continued on the row's other end:
 //   kConvA     bits shifted past the row's end (hi) return as hi X to the start
 //              of their row and as hi to the next one;
-//   kConvBInv  the transpose: the words before column 0 are X end + (row above's
-//              end) of the input's end words;
-//   kConvB     its inverse: those words are found from the converted end, and
-//              their own inverse image starts the stripe.
+//   kConvBInv  the words before column 0 are X end + (row above's end);
+//   kConvB     its inverse: they are the row above's end alone.
 // A CTA has 512 rows of stripes (2^r rows each); the whole-row stages that
-// follow (kConvBInv: precede) run in shared memory.
+// follow (kConvBInv: precede) run in shared memory, and from r = 4 on the first
+// four levels of the transform with them: their twiddles are the same for every
+// length and column, so they are one fixed map of 16 rows (first_levels).
 constexpr int kRowsThreads = 512;
 constexpr int kRowsSmem = 4 * 512 * (32 + 16);
 
@@ -237,7 +237,93 @@ __device__ __forceinline__ void row_shifts(uint32_t (&x)[32], uint32_t *xch, uin
     }
 }
 
-// The words before column 0 from the end words e[row][16].
+// Row i of multiplication by C in GF(2^4): the input bits output bit i sums.
+template <uint32_t C>
+struct Rows4 {
+    uint32_t r[4];
+    constexpr Rows4() : r{} {
+        for (int j = 0; j < 4; ++j)
+            for (int i = 0; i < 4; ++i) r[i] |= ((gmul(1u << j, C, 2) >> i) & 1u) << j;
+    }
+};
+
+// f * C in GF(2^4), bit-sliced.
+template <uint32_t C>
+__device__ __forceinline__ void times4(const uint32_t (&f)[4], uint32_t (&o)[4]) {
+    constexpr Rows4<C> M{};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        o[i] = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if ((M.r[i] >> j) & 1u) o[i] ^= f[j];
+    }
+}
+
+// Levels lg - 1 .. lg - 4 on 16 words whose number's bits 3 .. 0 are those index
+// bits.  KIND 0: a, 1: b, 2: b's inverse.  Levels lg - 1, lg - 2 and lg - 4 are
+// missing ones (components x_0, x_1, x_2); the twiddles are beta_1 .. beta_4 with
+// the point bit of level lg - 3 (build_pass computes the same for the other
+// lengths' tables).
+template <int KIND>
+__device__ __forceinline__ void first_levels(uint32_t (&x)[16]) {
+    auto missing1 = [&]() {
+        if (KIND == 0) return;  // u = 0
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] ^= x[i + 8];
+    };
+    auto missing2 = [&]() {
+        if (KIND == 0) return;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            x[i] ^= x[i + 4];
+            x[i + 8] ^= x[i + 12];
+        }
+    };
+    auto level3 = [&]() {
+#pragma unroll
+        for (int b0 = 0; b0 < 2; ++b0) {
+            uint32_t f[4], o[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const int at = b0 + 8 * (w & 1) + 4 * (w >> 1);
+                f[w] = KIND == 2 ? x[at] ^ x[at + 2] : x[at + 2];
+            }
+            times4<KIND == 0 ? 0xBu : 0xAu>(f, o);
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const int at = b0 + 8 * (w & 1) + 4 * (w >> 1);
+                x[at] ^= o[w];
+                x[at + 2] = KIND == 2 ? f[w] : x[at] ^ f[w];
+            }
+        }
+    };
+    auto missing4 = [&]() {
+#pragma unroll
+        for (int b1 = 0; b1 < 2; ++b1) {
+            uint32_t f[4], o[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) f[w] = x[2 * b1 + 8 * (w & 1) + 4 * (w >> 1) + 1];
+            if (b1) times4<KIND == 0 ? 0xEu : 0xFu>(f, o);
+            else times4<KIND == 0 ? 0xCu : 0xDu>(f, o);
+#pragma unroll
+            for (int w = 0; w < 4; ++w) x[2 * b1 + 8 * (w & 1) + 4 * (w >> 1)] ^= o[w];
+        }
+    };
+    if (KIND == 2) {
+        missing4();
+        level3();
+        missing2();
+        missing1();
+    } else {
+        missing1();
+        missing2();
+        level3();
+        missing4();
+    }
+}
+
+// X e_row + e_(row - 1), word c (e_row at e + row * ld).
 __device__ __forceinline__ uint32_t row_before(const uint32_t *e, uint32_t row, uint32_t c, uint32_t ld) {
     uint32_t v = e[row * ld + c] << 1;
     if (c) v |= e[row * ld + c - 1] >> 31;
@@ -320,7 +406,7 @@ template <int RC, bool INV>
 __global__ void __launch_bounds__(kRowsThreads, 2) k_gf_rows(const __grid_constant__ Ops q, int lg,
                                                           const __grid_constant__ Stages st, uint32_t *__restrict__ data) {
     extern __shared__ __align__(16) uint32_t sm[];
-    uint32_t *xch = sm, *side = sm + 512 * 32;  // side: 2^r x 16 words about column 0
+    uint32_t *xch = sm, *side = sm + 512 * 32;  // side: 2^r x 16 words past the row's end
     constexpr int B0 = RC - 5;                  // first round's lowest row bit
     const int r = lg - 16, S = 9 - r;           // 2^S stripes a CTA (128 in all)
     const uint32_t R = 1u << r, groups = S < 7 ? 128u >> S : 1u;
@@ -332,37 +418,26 @@ __global__ void __launch_bounds__(kRowsThreads, 2) k_gf_rows(const __grid_consta
     if (!INV) {
         const InOp in = in_op(q, op);
         const Lin lin = lin_of(in, is_b, lg);
-        // phase 0: the row's end (its last words, then zeros a's shifts run into);
-        // phase 1: b's words before column 0; phase 2: the stripes
-        for (int phase = first ? 0 : 2; phase < 3; ++phase) {
-            if (phase == 1 && !is_b) continue;
+        // phase 0 (a's first stripe): the row's last words, then zeros its shifts
+        // run into; phase 1: the stripes
+        for (int phase = first && !is_b ? 0 : 1; phase < 2; ++phase) {
             __syncthreads();
             for (int i0 = 0; i0 < 32; i0 += 8) {
                 uint32_t v[8];
-                if (phase != 1)
-                    in_words<8>(in, lin, is_b, lg, [&](int i) -> uint32_t {
-                        const uint32_t u = row_unit<B0>(warp, i0 + i), row = u & (R - 1u), stripe = (grp << S) + (u >> r);
-                        uint32_t col = ~0u;
-                        if (phase == 2) {
-                            if (16 * stripe + lane >= 16 && stripe < 128) col = 16 * stripe + lane - 16;
-                        } else if (u < R && (is_b || lane < 16)) {
-                            col = (is_b ? 2016u : 2032u) + lane;
-                        }
-                        return col == ~0u ? col : row * 2048u + col;
-                    }, v);
+                in_words<8>(in, lin, is_b, lg, [&](int i) -> uint32_t {
+                    const uint32_t u = row_unit<B0>(warp, i0 + i), row = u & (R - 1u), stripe = (grp << S) + (u >> r);
+                    const uint32_t at = row * 2048u + 16 * stripe + lane - 16;  // b: on into the row above
+                    if (phase == 0) return u < R && lane < 16 ? row * 2048u + 2032u + lane : ~0u;
+                    return stripe < 128 && (16 * stripe + lane >= 16 || (is_b && row)) ? at : ~0u;
+                }, v);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const uint32_t u = row_unit<B0>(warp, i0 + i), row = u & (R - 1u);
-                    if (phase == 1) v[i] = u < R && lane >= 16 ? row_before(side, row, lane - 16, 16) : 0u;
-                    if (phase == 2 && is_b && first && u < R && lane < 16) v[i] = side[row * 16 + lane];
-                    xch[u * 32 + lane] = v[i];
-                }
+                for (int i = 0; i < 8; ++i) xch[row_unit<B0>(warp, i0 + i) * 32 + lane] = v[i];
             }
             __syncwarp();
 #pragma unroll
             for (int i = 0; i < 32; ++i) x[i] = xch[row_unit<B0>(warp, i) * 32 + lane];
             row_shifts<RC>(x, xch, warp, lane, r);
-            if (phase == 2) break;
+            if (phase == 1) break;
             __syncthreads();
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
@@ -380,17 +455,41 @@ __global__ void __launch_bounds__(kRowsThreads, 2) k_gf_rows(const __grid_consta
             for (uint32_t u = threadIdx.x >> 4; u < R; u += 32) sm[u * 16 + c] ^= row_before(side, u, c, 16);
         if (is_b) row_whole_stages<kConvB, 16, RC>(sm, st);
         else row_whole_stages<kConvA, 16, RC>(sm, st);
-        for (uint32_t u = threadIdx.x >> 4; u < 512; u += 32) {
-            const uint32_t row = u & (R - 1u), stripe = (grp << S) + (u >> r);
-            if (stripe < 128) arr[(uint64_t)row * 2048u + stripe * 16u + c] = sm[u * 16 + c];
+        if (r >= 4) {
+            const uint32_t g = threadIdx.x >> 4, row = g & (R / 16 - 1u), sl = g >> (r - 4), stripe = (grp << S) + sl;
+            uint32_t y[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) y[k] = sm[(sl * R + row + k * (R / 16)) * 16 + c];
+            if (is_b) first_levels<1>(y);
+            else first_levels<0>(y);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) arr[(uint64_t)(row + k * (R / 16)) * 2048u + stripe * 16u + c] = y[k];
+        } else {
+            for (uint32_t u = threadIdx.x >> 4; u < 512; u += 32) {
+                const uint32_t row = u & (R - 1u), stripe = (grp << S) + (u >> r);
+                if (stripe < 128) arr[(uint64_t)row * 2048u + stripe * 16u + c] = sm[u * 16 + c];
+            }
         }
     } else {
         const OutOp out = out_op(q, op);
         const bool bad = constant_input(out, first && threadIdx.x == 0);
+        if (r >= 4) {
+#pragma unroll
+            for (uint32_t g = warp; g < 32; g += 16) {
+                const uint32_t row = g & (R / 16 - 1u), sl = g >> (r - 4), col = (16u * ((grp << S) + sl) + lane - 16u) & 2047u;
+                uint32_t y[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) y[k] = arr[(uint64_t)(row + k * (R / 16)) * 2048u + col];
+                first_levels<2>(y);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) sm[(sl * R + row + k * (R / 16)) * 32 + lane] = y[k];
+            }
+        } else {
 #pragma unroll 8
-        for (uint32_t u = warp; u < 512; u += 16) {
-            const uint32_t row = u & (R - 1u), stripe = ((grp << S) + (u >> r)) & 127u;
-            sm[u * 32 + lane] = arr[(uint64_t)row * 2048u + ((16u * stripe + lane - 16u) & 2047u)];
+            for (uint32_t u = warp; u < 512; u += 16) {
+                const uint32_t row = u & (R - 1u), stripe = ((grp << S) + (u >> r)) & 127u;
+                sm[u * 32 + lane] = arr[(uint64_t)row * 2048u + ((16u * stripe + lane - 16u) & 2047u)];
+            }
         }
         row_whole_stages<kConvBInv, 32, RC>(sm, st);
 #pragma unroll
@@ -417,66 +516,257 @@ __global__ void __launch_bounds__(kRowsThreads, 2) k_gf_rows(const __grid_consta
 }
 
 // ---------------------------------------------------------------------------
-// Conversion of rows of 2^rb bits to 256-bit units: one CTA a row, one thread a
-// unit.  In place; for lg <= 16 the row is the whole operand, read from the
-// inputs or written to z.
-template <int KIND>
-__device__ void unit_stages(uint32_t (&x)[8], uint32_t *snap, uint32_t nu, int r, const Stages &st) {
-    const uint32_t t = threadIdx.x;
-    auto publish = [&]() {
-        __syncthreads();
+// Conversion of rows of 2^(8 + UB) bits to 256-bit units (UB = 8, or 7 for
+// transforms of 2^15): the same stages as across rows, units for rows and 8
+// words for columns.  16 threads have a unit's 8 words and the 8 words before
+// (kConvB, kConvBInv) or past (kConvA) it, 32 units in registers; the whole-unit
+// stages are the shifts of the upper four unit bits in shared memory, then four
+// bits' conversion in registers, twice.  Bound by instruction issue (about 55 a
+// word; stages between barriers on a unit a thread took 150).  In place; for
+// lg <= 16 the row is the whole operand, read from the inputs or written to z.
+constexpr int kUnitsThreads = 256;
+
+// Conversion of the 4 index bits of 16 registers.
+template <int KIND, int TOP, int SH>
+__device__ __forceinline__ void conv4_stage(uint32_t (&x)[16]) {
+    constexpr int H = 1 << TOP, S = 1 << SH;
+    auto wrap = [&]() {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) snap[i * nu + t] = x[i];
-        __syncthreads();
+        for (int b = 0; b < 16; b += 2 * H)
+#pragma unroll
+            for (int v = 0; v < S; ++v) {
+                const int o = b + (KIND == kConvA ? H : 0);
+                x[o + v] ^= x[o + H - S + v];
+            }
     };
-    auto whole = [&](int q) {
-        publish();
-        whole_stage<KIND>(t, st.top[q], st.sh[q], [&](uint32_t d) { unit_xor(x, snap, nu, t + d); });
-    };
-    if (KIND != kConvBInv) {
-        for (int j = r - 1; j >= 0; --j) {
-            publish();
-            bit_stage_n<KIND>(j, x, snap, nu, t);
-        }
-        for (int q = 0; q < st.n; ++q) whole(q);
+    if (KIND != kConvBInv) wrap();
+#pragma unroll
+    for (int b = 0; b < 16; b += 2 * H)
+#pragma unroll
+        for (int v = S; v < H; ++v) x[b + v] ^= x[b + H + v - S];
+    if (KIND == kConvBInv) wrap();
+}
+
+template <int KIND>
+__device__ __forceinline__ void conv4(uint32_t (&x)[16]) {
+    if (KIND == kConvBInv) {
+        conv4_stage<KIND, 1, 0>(x);
+        conv4_stage<KIND, 3, 2>(x);
+        conv4_stage<KIND, 2, 0>(x);
+        conv4_stage<KIND, 3, 1>(x);
     } else {
-        for (int q = st.n - 1; q >= 0; --q) whole(q);
-        for (int j = 0; j < r; ++j) {
-            publish();
-            bit_stage_n<KIND>(j, x, snap, nu, t);
-        }
+        conv4_stage<KIND, 3, 1>(x);
+        conv4_stage<KIND, 2, 0>(x);
+        conv4_stage<KIND, 3, 2>(x);
+        conv4_stage<KIND, 1, 0>(x);
     }
 }
 
-template <bool INV>
-__global__ void __launch_bounds__(256) k_gf_units(const __grid_constant__ Ops q, int lg,
-                                                  const __grid_constant__ Stages st, uint32_t *__restrict__ data) {
-    __shared__ uint32_t snap[2048];
-    const int rb = lg < 16 ? lg : 16;
-    const uint32_t nu = 1u << (rb - 8);  // blockDim.x
-    const uint64_t w0 = ((uint64_t)blockIdx.x << (rb - 5)) + 8 * threadIdx.x;
-    const uint32_t op = (uint32_t)(((uint64_t)blockIdx.x << rb) >> lg);
-    const bool is_b = op >= q.na;
-    uint32_t x[8];
-    if (!INV && lg <= 16) {
-        const InOp in = in_op(q, op);
-        in_words<8>(in, lin_of(in, is_b, lg), is_b, lg, [&](int i) -> uint32_t { return 8 * threadIdx.x + i; }, x);
+// Conversion of 3 index bits (the upper ones when UB = 7) of 8 registers, every
+// second of 16.
+template <int KIND>
+__device__ __forceinline__ void conv3(uint32_t (&x)[8]) {
+    // stages (2, 0), then (1, 0) of the lower two bits
+    auto st = [&](int H, int S) {
+        if (KIND != kConvBInv)
+            for (int b = 0; b < 8; b += 2 * H)
+                for (int v = 0; v < S; ++v) x[b + (KIND == kConvA ? H : 0) + v] ^= x[b + (KIND == kConvA ? H : 0) + H - S + v];
+        for (int b = 0; b < 8; b += 2 * H)
+            for (int v = S; v < H; ++v) x[b + v] ^= x[b + H + v - S];
+        if (KIND == kConvBInv)
+            for (int b = 0; b < 8; b += 2 * H)
+                for (int v = 0; v < S; ++v) x[b + v] ^= x[b + H - S + v];
+    };
+    if (KIND == kConvBInv) {
+        st(2, 1);
+        st(4, 1);
     } else {
-        const uint4 u = *reinterpret_cast<const uint4 *>(data + w0), v = *reinterpret_cast<const uint4 *>(data + w0 + 4);
-        x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
-        x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
+        st(4, 1);
+        st(2, 1);
     }
-    if (INV) unit_stages<kConvBInv>(x, snap, nu, rb - 8, st);
-    else if (is_b) unit_stages<kConvB>(x, snap, nu, rb - 8, st);
-    else unit_stages<kConvA>(x, snap, nu, rb - 8, st);
-    if (INV && lg <= 16) {
-        const OutOp out = out_op(q, op);
-        const bool bad = constant_input(out, threadIdx.x == 0);
+}
+
+// Shift stages HI - 1 .. LO of the unit bits B .. B + 4 in registers.
+template <int B, int HI, int LO>
+__device__ __forceinline__ void unit_shift_stages(uint32_t (&x)[32], uint32_t c16) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) out_word(out, bad, lg, 8 * threadIdx.x + i, x[i]);
+    for (int j = HI - 1; j >= LO; --j) {
+        const int s = 1 << j, bit = 1 << (j - B);
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (!(i & bit)) {
+                const uint32_t y = x[i | bit];
+                if (s < 32) {
+                    uint32_t p = __shfl_up_sync(0xFFFFFFFFu, y, 1, 16);
+                    if (c16 == 0) p = 0;
+                    x[i] ^= __funnelshift_l(p, y, s);
+                } else {
+                    const uint32_t p = __shfl_up_sync(0xFFFFFFFFu, y, s >> 5, 16);
+                    x[i] ^= c16 >= (uint32_t)(s >> 5) ? p : 0u;
+                }
+            }
+    }
+}
+
+// Whole-unit stages on S[unit * 8 + word].  tid: of the row's 2^(UB - 1) threads.
+template <int KIND, int UB>
+__device__ __forceinline__ void unit_whole_stages(uint32_t *S, uint32_t tid) {
+    constexpr uint32_t TPR = 1u << (UB - 1), NU = 1u << UB;
+    const uint32_t c = tid & 7u, g = tid >> 3;
+    auto shifts = [&](int top, int sh) {  // of the upper bits, by the lower four
+        const uint32_t H = 1u << top, s = 1u << sh;
+        auto bulk = [&]() {
+            __syncthreads();
+#pragma unroll
+            for (uint32_t i = 0; i < NU / 2; i += TPR / 8) {
+                const uint32_t u = i + g, v = u & (H - 1u), t = v | ((u ^ v) << 1);
+                if (v >= s) S[t * 8 + c] ^= S[(t + H - s) * 8 + c];
+            }
+        };
+        auto wrap = [&]() {
+            __syncthreads();
+            for (uint32_t u = g; u < (NU >> (top + 1)) * s; u += TPR / 8) {
+                const uint32_t t = ((u >> sh) << (top + 1)) + (KIND == kConvA ? H : 0u) + (u & (s - 1u));
+                S[t * 8 + c] ^= S[(t + H - s) * 8 + c];
+            }
+        };
+        if (KIND != kConvBInv) wrap();
+        bulk();
+        if (KIND == kConvBInv) wrap();
+    };
+    auto upper = [&]() {  // conversion of the upper UB - 4 bits
+        __syncthreads();
+        if (UB == 8) {
+            uint32_t x[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) x[i] = S[(16 * i + g) * 8 + c];
+            conv4<KIND>(x);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) S[(16 * i + g) * 8 + c] = x[i];
+        } else {
+            for (uint32_t k = g; k < 16; k += TPR / 8) {
+                uint32_t x[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) x[i] = S[(16 * i + k) * 8 + c];
+                conv3<KIND>(x);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) S[(16 * i + k) * 8 + c] = x[i];
+            }
+        }
+    };
+    auto lower = [&]() {  // of the lower four
+        __syncthreads();
+        for (uint32_t h = g; h < NU / 16; h += TPR / 8) {
+            uint32_t x[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) x[i] = S[(16 * h + i) * 8 + c];
+            conv4<KIND>(x);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) S[(16 * h + i) * 8 + c] = x[i];
+        }
+    };
+    if (KIND == kConvBInv) {
+        lower();
+        upper();
+#pragma unroll
+        for (int j = 0; j < UB - 4; ++j) shifts(4 + j, j);
     } else {
-        *reinterpret_cast<uint4 *>(data + w0) = make_uint4(x[0], x[1], x[2], x[3]);
-        *reinterpret_cast<uint4 *>(data + w0 + 4) = make_uint4(x[4], x[5], x[6], x[7]);
+#pragma unroll
+        for (int j = UB - 5; j >= 0; --j) shifts(4 + j, j);
+        upper();
+        lower();
+    }
+    __syncthreads();
+}
+
+// The shift stages of a row in S through the exchange buffer E[unit * 16 + c16].
+template <int KIND, int UB>
+__device__ __forceinline__ void unit_shifts(uint32_t *S, uint32_t *E, uint32_t tid, uint32_t (&x)[32]) {
+    const uint32_t c16 = tid & 15u, tu = tid >> 4;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        const uint32_t u = tu | (uint32_t)i << (UB - 5), at = u * 8 + c16;
+        if (KIND == kConvA) x[i] = c16 < 8 ? S[at] : 0u;
+        else if (KIND == kConvB) x[i] = at >= 8 ? S[at - 8] : 0u;
+        else x[i] = c16 >= 8 ? S[at - 8] : row_before(S, u, c16, 8);
+    }
+    unit_shift_stages<UB - 5, UB, UB - 5>(x, c16);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) E[(tu | (uint32_t)i << (UB - 5)) * 16 + c16] = x[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 32; ++i) x[i] = E[((uint32_t)i | tu << 5) * 16 + c16];
+    unit_shift_stages<0, UB - 5, 0>(x, c16);
+}
+
+// KIND is the same in a CTA: kConvA and kConvB rows (ra and rb of them) have CTAs
+// of their own.
+template <int KIND, int UB>
+__device__ __forceinline__ void units_row(const Ops &q, int lg, uint32_t row, bool in_range, uint32_t *S, uint32_t *E,
+                                          uint32_t tid, uint32_t *__restrict__ data) {
+    constexpr uint32_t TPR = 1u << (UB - 1), NW = 8u << UB;
+    uint32_t *arr = data + (uint64_t)row * NW;
+    const uint32_t op = (uint32_t)(((uint64_t)row << (UB + 8)) >> lg);
+    const uint32_t c16 = tid & 15u, tu = tid >> 4;
+    uint32_t x[32];
+    if (in_range) {
+        if (KIND != kConvBInv && lg <= 16) {
+            const InOp in = in_op(q, op);
+            const Lin lin = lin_of(in, KIND == kConvB, lg);
+            for (uint32_t i = 0; i < NW / TPR; i += 8) {
+                uint32_t v[8];
+                in_words<8>(in, lin, KIND == kConvB, lg, [&](int k) -> uint32_t { return (i + k) * TPR + tid; }, v);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) S[(i + k) * TPR + tid] = v[k];
+            }
+        } else {
+#pragma unroll
+            for (uint32_t i = tid; i < NW / 4; i += TPR) reinterpret_cast<uint4 *>(S)[i] = reinterpret_cast<const uint4 *>(arr)[i];
+        }
+    }
+    __syncthreads();
+    if (KIND == kConvBInv) unit_whole_stages<KIND, UB>(S, tid);
+    unit_shifts<KIND, UB>(S, E, tid, x);
+    if (KIND == kConvA) {
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) E[((uint32_t)i | tu << 5) * 16 + c16] = x[i];
+        __syncthreads();
+        for (uint32_t w = tid; w < NW; w += TPR) {
+            const uint32_t u = w >> 3, c = w & 7u;
+            S[w] = E[u * 16 + c] ^ row_before(E + 8, u, c, 16);
+        }
+    } else {  // all of S has been read
+        if (c16 >= 8)
+#pragma unroll
+            for (int i = 0; i < 32; ++i) S[((uint32_t)i | tu << 5) * 8 + c16 - 8] = x[i];
+    }
+    if (KIND != kConvBInv) unit_whole_stages<KIND, UB>(S, tid);
+    else __syncthreads();
+    if (!in_range) return;
+    if (KIND == kConvBInv && lg <= 16) {
+        const OutOp out = out_op(q, op);
+        const bool bad = constant_input(out, tid == 0);
+        for (uint32_t w = tid; w < NW; w += TPR) out_word(out, bad, lg, w, S[w]);
+    } else {
+#pragma unroll
+        for (uint32_t i = tid; i < NW / 4; i += TPR) reinterpret_cast<uint4 *>(arr)[i] = reinterpret_cast<const uint4 *>(S)[i];
+    }
+}
+
+template <bool INV, int UB>
+__global__ void __launch_bounds__(kUnitsThreads, 4) k_gf_units(const __grid_constant__ Ops q, int lg, uint32_t ra,
+                                                               uint32_t rb, uint32_t *__restrict__ data) {
+    constexpr uint32_t TPR = 1u << (UB - 1), NW = 8u << UB, RPC = kUnitsThreads / TPR;
+    extern __shared__ __align__(16) uint32_t sm[];
+    const uint32_t mine = threadIdx.x / TPR, tid = threadIdx.x % TPR, ca = (ra + RPC - 1) / RPC;
+    uint32_t *S = sm + mine * 3 * NW, *E = S + NW;
+    if (INV || blockIdx.x >= ca) {
+        const uint32_t k = (INV ? blockIdx.x : blockIdx.x - ca) * RPC + mine;
+        units_row<INV ? kConvBInv : kConvB, UB>(q, lg, INV ? k : ra + k, k < (INV ? ra : rb), S, E, tid, data);
+    } else {
+        const uint32_t k = blockIdx.x * RPC + mine;
+        units_row<kConvA, UB>(q, lg, k, k < ra, S, E, tid, data);
     }
 }
 
@@ -787,14 +1077,23 @@ cudaError_t rows_launch(cm_ctx *c, bool inv, const Ops &q, int lg, uint32_t ops,
     }
 }
 
-cudaError_t units_launch(cm_ctx *c, bool inv, const Ops &q, int lg, uint32_t ops, uint32_t *data, cudaStream_t st) {
-    const int rb = lg < 16 ? lg : 16;
-    const Stages s = stages_of(rb - 8);
-    const uint32_t grid = ops << (lg - rb), nt = 1u << (rb - 8);
-    Scope ps(c, inv ? "k_gf_units_inv" : "k_gf_units", st);
-    if (inv) k_gf_units<true><<<grid, nt, 0, st>>>(q, lg, s, data);
-    else k_gf_units<false><<<grid, nt, 0, st>>>(q, lg, s, data);
+template <int UB>
+cudaError_t units_launch_ub(bool inv, const Ops &q, int lg, uint32_t na, uint32_t nb, uint32_t *data, cudaStream_t st) {
+    constexpr uint32_t RPC = kUnitsThreads >> (UB - 1);
+    constexpr int smem = (int)(RPC * 3 * (8u << UB) * 4);
+    cudaError_t e = inv ? smem_attr_once<k_gf_units<true, UB>>(smem) : smem_attr_once<k_gf_units<false, UB>>(smem);
+    if (e != cudaSuccess) return e;
+    const uint32_t ra = na << (lg - 8 - UB), rb = nb << (lg - 8 - UB), grid = (ra + RPC - 1) / RPC + (rb + RPC - 1) / RPC;
+    if (inv) k_gf_units<true, UB><<<grid, kUnitsThreads, smem, st>>>(q, lg, ra, rb, data);
+    else k_gf_units<false, UB><<<grid, kUnitsThreads, smem, st>>>(q, lg, ra, rb, data);
     return cudaGetLastError();
+}
+
+// Forward: na arrays of a, nb of b; inverse: na arrays.
+cudaError_t units_launch(cm_ctx *c, bool inv, const Ops &q, int lg, uint32_t na, uint32_t nb, uint32_t *data,
+                         cudaStream_t st) {
+    Scope ps(c, inv ? "k_gf_units_inv" : "k_gf_units", st);
+    return lg == 15 ? units_launch_ub<7>(inv, q, lg, na, nb, data, st) : units_launch_ub<8>(inv, q, lg, na, nb, data, st);
 }
 
 template <int NB, int FMAX>
@@ -850,7 +1149,7 @@ cudaError_t launch_product(cm_ctx *c, int nsm, const Product &p, const Ops &q, c
     uint32_t *B = data + ((uint64_t)q.na << (p.lg - 5));
     cudaError_t e = cudaSuccess;
     if (s.colr && (e = rows_launch(c, false, q, p.lg, ops, data, st)) != cudaSuccess) return e;
-    if ((e = units_launch(c, false, q, p.lg, ops, data, st)) != cudaSuccess) return e;
+    if ((e = units_launch(c, false, q, p.lg, q.na, q.nb, data, st)) != cudaSuccess) return e;
     if (s.two) {
         Scope ps(c, "k_gf_cols", st);
         k_gf_cols<false><<<ops << (p.lg - 18), kColsThreads, 0, st>>>(p.lg, q.na, col, data);
@@ -883,7 +1182,7 @@ cudaError_t launch_product(cm_ctx *c, int nsm, const Product &p, const Ops &q, c
         k_gf_cols<true><<<q.nz << (p.lg - 18), kColsThreads, 0, st>>>(p.lg, 0, col, out);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if ((e = units_launch(c, true, q, p.lg, q.nz, out, st)) != cudaSuccess) return e;
+    if ((e = units_launch(c, true, q, p.lg, q.nz, 0, out, st)) != cudaSuccess) return e;
     if (s.colr) e = rows_launch(c, true, q, p.lg, q.nz, out, st);
     return e;
 }

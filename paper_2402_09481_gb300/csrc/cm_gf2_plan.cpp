@@ -181,7 +181,8 @@ void build_passes(int lg, Pass *mid, Pass *col) {
         const int rows = lg - s.lo;
         for (int i = 5; i < 5 + 13 - rows; ++i) cin.push_back(i);
         for (int i = s.lo; i < lg; ++i) cin.push_back(i);
-        build_pass(lg, 13, 9, 4, cin, lg - 1, s.lo, beta, col);
+        // from 2^20 on the row conversion does the first four levels (first_levels)
+        build_pass(lg, 13, 9, 4, cin, lg >= 20 ? lg - 5 : lg - 1, s.lo, beta, col);
     }
 }
 

@@ -131,117 +131,12 @@ CM_HD void conv8(uint32_t (&x)[8]) {
     }
 }
 
-// ---------------------------------------------------------------------------
-// Conversion of a row of 2^(8 + r) bits, r <= 8, above the 256-bit units: each
-// thread keeps one unit (8 words) in registers and reads others from a snapshot
-// (word i of unit t at snap[i * nu + t]).
-
 // Conversion stages above the first ones of a length: (block bit, shift bit)
-// pairs in units, in order for kConvA / kConvB.
+// pairs in rows, in order for kConvA / kConvB.
 struct Stages {
     int n;
     uint8_t top[16], sh[16];
 };
-
-CM_HD void unit_xor(uint32_t (&x)[8], const uint32_t *snap, uint32_t nu, uint32_t t) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] ^= snap[i * nu + t];
-}
-
-// x ^= the low S bits' worth of y's top S bits (y: 256 bits at unit t).
-template <int S>
-CM_HD void xor_top(uint32_t (&x)[8], const uint32_t *snap, uint32_t nu, uint32_t t) {
-    if constexpr (S < 32) x[0] ^= snap[7 * nu + t] >> (32 - S);
-    else {
-#pragma unroll
-        for (int i = 0; i < S / 32; ++i) x[i] ^= snap[(8 - S / 32 + i) * nu + t];
-    }
-}
-
-template <int S>
-CM_HD void xor_shl(uint32_t (&x)[8], const uint32_t (&y)[8]) {
-    if constexpr (S < 32) {
-#pragma unroll
-        for (int i = 7; i > 0; --i) x[i] ^= (y[i] << S) | (y[i - 1] >> (32 - S));
-        x[0] ^= y[0] << S;
-    } else {
-#pragma unroll
-        for (int i = S / 32; i < 8; ++i) x[i] ^= y[i - S / 32];
-    }
-}
-
-// Stage J: blocks of 2^(J+1) units, shift 2^J bits (< 256).
-template <int J, int KIND>
-CM_HD void bit_stage(uint32_t (&x)[8], const uint32_t *snap, uint32_t nu, uint32_t t) {
-    constexpr uint32_t H = 1u << J;
-    constexpr int S = 1 << J;
-    const uint32_t off = t & (H - 1u);
-    if (t & H) {
-        if (KIND == kConvA && off == 0) xor_top<S>(x, snap, nu, t + H - 1);
-        return;
-    }
-    uint32_t y[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) y[i] = snap[i * nu + t + H];
-    if (KIND == kConvA && off == 0) xor_top<S>(y, snap, nu, t + 2 * H - 1);
-    if (KIND == kConvB && off == 0) xor_top<S>(x, snap, nu, t + H - 1);
-    xor_shl<S>(x, y);
-    if (off) xor_top<S>(x, snap, nu, t + H - 1);
-    if (KIND == kConvBInv && off == 0) {  // the lower half's last unit as this stage leaves it
-        uint32_t l[8];
-        if (H == 1) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) l[i] = x[i];
-        } else {
-            uint32_t u[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                l[i] = snap[i * nu + t + H - 1];
-                u[i] = snap[i * nu + t + 2 * H - 1];
-            }
-            xor_shl<S>(l, u);
-        }
-        if constexpr (S < 32) x[0] ^= l[7] >> (32 - S);
-        else {
-#pragma unroll
-            for (int i = 0; i < S / 32; ++i) x[i] ^= l[8 - S / 32 + i];
-        }
-    }
-}
-
-template <int KIND>
-CM_HD void bit_stage_n(int j, uint32_t (&x)[8], const uint32_t *snap, uint32_t nu, uint32_t t) {
-    switch (j) {
-        case 0: bit_stage<0, KIND>(x, snap, nu, t); break;
-        case 1: bit_stage<1, KIND>(x, snap, nu, t); break;
-        case 2: bit_stage<2, KIND>(x, snap, nu, t); break;
-        case 3: bit_stage<3, KIND>(x, snap, nu, t); break;
-        case 4: bit_stage<4, KIND>(x, snap, nu, t); break;
-        case 5: bit_stage<5, KIND>(x, snap, nu, t); break;
-        case 6: bit_stage<6, KIND>(x, snap, nu, t); break;
-        default: bit_stage<7, KIND>(x, snap, nu, t);
-    }
-}
-
-// Stage (top, sh) in units: calls take(d) for the distance d of every unit (or
-// row) whose old value is added to unit t.
-template <int KIND, class F>
-CM_HD void whole_stage(uint32_t t, uint32_t top, uint32_t sh, F take) {
-    const uint32_t H = 1u << top, s = 1u << sh, v = t & (H - 1u);
-    if (t & H) {
-        if (KIND == kConvA && v < s) take(H - s);
-        return;
-    }
-    if (KIND == kConvA) {
-        if (v >= s) {
-            take(H - s);
-            if (v < 2 * s) take(2 * H - 2 * s);
-        }
-    } else {
-        take(H - s);
-        if (KIND == kConvBInv && v < s) take(2 * H - 2 * s);
-    }
-}
 
 // ---------------------------------------------------------------------------
 // Levels.

@@ -785,7 +785,7 @@ __device__ __forceinline__ void load_pass(Pass *P, const Pass *__restrict__ g) {
 constexpr int kColsThreads = 256;
 
 template <bool INV>
-__global__ void __launch_bounds__(kColsThreads) k_gf_cols(int lg, uint32_t na, const Pass *__restrict__ table,
+__global__ void __launch_bounds__(kColsThreads, 3) k_gf_cols(int lg, uint32_t na, const Pass *__restrict__ table,
                                                           uint32_t *__restrict__ data) {
     __shared__ __align__(16) uint32_t sm[8192];
     __shared__ Pass P;
@@ -901,7 +901,8 @@ __device__ void inverse_levels(uint32_t *sm, const Pass &P, const uint32_t *base
 // (a tile's own time counts); else one operand after the other on half as many
 // threads, so that three CTAs of an SM fill each other's gaps.
 template <int NB, int FMAX, bool PAR>
-__global__ void __launch_bounds__((PAR ? 2 : 1) * MidShape<NB, FMAX>::HALF) k_gf_mid(int lg, const Pass *__restrict__ table,
+__global__ void __launch_bounds__((PAR ? 2 : 1) * MidShape<NB, FMAX>::HALF, PAR ? 1 : 384 / MidShape<NB, FMAX>::HALF)
+k_gf_mid(int lg, const Pass *__restrict__ table,
                                                                          const uint32_t *__restrict__ A,
                                                                          uint32_t *__restrict__ B) {
     using S = MidShape<NB, FMAX>;

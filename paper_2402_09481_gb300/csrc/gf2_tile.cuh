@@ -181,33 +181,36 @@ template <int NFREE, int F, bool INV>
 CM_HD void level_unit(uint32_t *sm, const Lev &v, uint32_t base, bool lanes, uint32_t u) {
     const uint32_t a = unit_addr<NFREE>(u, v.p, F);
     uint32_t *s0 = sm + phys(a), *s1 = sm + phys(a | (1u << v.p));
-    uint32_t x1[1 << F], t[1 << F], o[1 << F];
+    uint32_t x0[1 << F], x1[1 << F], t[1 << F], o[1 << F];
     spread<F>(v, twiddle(v, base, a), lanes, t);
-    if (v.missing) {
+    // every load of a unit comes before its first store: the two halves' addresses
+    // are unrelated to the compiler, which would otherwise chain them
+    if (v.missing || !INV) {
 #pragma unroll
         for (int j = 0; j < (1 << F); ++j) x1[j] = s1[j << NFREE];
         mul<F>(x1, t, o);
 #pragma unroll
-        for (int j = 0; j < (1 << F); ++j) s0[j << NFREE] ^= o[j];
-    } else if (!INV) {
+        for (int j = 0; j < (1 << F); ++j) x0[j] = s0[j << NFREE] ^ o[j];
 #pragma unroll
-        for (int j = 0; j < (1 << F); ++j) x1[j] = s1[j << NFREE];
-        mul<F>(x1, t, o);
+        for (int j = 0; j < (1 << F); ++j) s0[j << NFREE] = x0[j];
+        if (!v.missing) {
 #pragma unroll
-        for (int j = 0; j < (1 << F); ++j) {
-            const uint32_t y = s0[j << NFREE] ^ o[j];
-            s0[j << NFREE] = y;
-            s1[j << NFREE] = y ^ x1[j];
+            for (int j = 0; j < (1 << F); ++j) s1[j << NFREE] = x0[j] ^ x1[j];
         }
     } else {
 #pragma unroll
         for (int j = 0; j < (1 << F); ++j) {
-            x1[j] = s0[j << NFREE] ^ s1[j << NFREE];
-            s1[j << NFREE] = x1[j];
+            x0[j] = s0[j << NFREE];
+            x1[j] = s1[j << NFREE];
         }
+#pragma unroll
+        for (int j = 0; j < (1 << F); ++j) x1[j] ^= x0[j];
         mul<F>(x1, t, o);
 #pragma unroll
-        for (int j = 0; j < (1 << F); ++j) s0[j << NFREE] ^= o[j];
+        for (int j = 0; j < (1 << F); ++j) {
+            s0[j << NFREE] = x0[j] ^ o[j];
+            s1[j << NFREE] = x1[j];
+        }
     }
 }
 

@@ -720,6 +720,13 @@ void gf_shape(int kind, uint64_t n, uint64_t m, gf::Product *p, gf::Ops *q) {
 // 1812 / 10659: below 2^24 too few tiles to fill the GPU.
 // Products of up to 2^13 terms run densely in one launch (cm_gf2_dense.cu).
 constexpr int kGfMinLg = 24;
+// Products of 2^17 .. 2^22 terms run densely on the tensor cores (cm_gf2_tc.cu)
+// while their longest chain of stages beats the transforms.  Measured, us a call,
+// integer transforms / dense (K x m: stages): 100000 x 50000: 3, 43 / 25; 300007 x
+// 150001: 24, 47 / 31.5; 349525 x 174762: 36, 47 / 39; 30000 x 2000000: 40, 66 / 35;
+// 2000000 x 20000: 52, 66 / 53; 450000 x 400000: 84, 50 / 101.
+constexpr int kTcMinLg = 17, kTcMaxLg = 22;
+constexpr uint64_t kTcMaxStages = 40;
 
 bool gf_allowed(const cm_ctx *ctx) {
     const PlanOptions &o = ctx->popt;
@@ -731,6 +738,19 @@ cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64
     r->n = n;
     r->m = m;
     const uint64_t terms = (kind == CM_CIRCULANT ? n + 1 : n) + m - 1;
+    if (gf_allowed(ctx) && n - 1 < kMaxBits && m - 1 < kMaxBits && terms > 1ull << kTcMinLg &&
+        terms <= 1ull << kTcMaxLg) {
+        r->shape = gf::tc_shape(terms - m + 1, m, ctx->nsm);
+        if (r->shape.stages <= kTcMaxStages && valid_args(kind, n, m)) {
+            gf_shape(kind, n, m, &r->prod, &r->ops);
+            gf_maps(kind, n, m, &r->ops);
+            r->tmp_off = (4 * r->shape.a_words + 255) & ~255ull;  // b's bits
+            r->pre_off = r->tmp_off + ((4 * r->shape.b_words + 255) & ~255ull);
+            r->need = r->pre_off + kFlagBytes;
+            r->tc = r->need <= budget;
+            if (r->tc) return CM_OK;
+        }
+    }
     if (gf_allowed(ctx) && n - 1 < kMaxBits && m - 1 < kMaxBits &&
         (terms <= 1ull << gf::kDenseMaxLg || terms > 1ull << (kGfMinLg - 1)) && valid_args(kind, n, m)) {
         if (terms <= 1ull << gf::kDenseMaxLg) {
@@ -760,6 +780,24 @@ cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t
         return cuda_status(gf::launch_dense(r.ops.a0.map, r.ops.b0.map, (uint32_t)(r.kind == CM_CIRCULANT ? r.n + 1 : r.n),
                                             (uint32_t)r.m, r.kind == CM_DODIS, z, ctx->d_status,
                                             sc ? reinterpret_cast<uint32_t *>(sc + r.pre_off) : nullptr, st));
+    }
+    if (r.tc) {
+        uint32_t *a = reinterpret_cast<uint32_t *>(sc), *b = reinterpret_cast<uint32_t *>(sc + r.tmp_off), *pre = nullptr;
+        r.ops.a0.map.src = x;
+        r.ops.b0.map.src = y;
+        if (r.kind == CM_DODIS) {
+            pre = reinterpret_cast<uint32_t *>(sc + r.pre_off);
+            cm_status s = enqueue_precondition(ctx, x, r.n, pre, st);
+            if (s != CM_OK) return s;
+        }
+        {
+            ProfScope ps(ctx, "k_gf_tc_prep", st);
+            cudaError_t e = gf::launch_tc_prep(r.ops, r.shape, a, b, z, r.m, st);
+            if (e != cudaSuccess) return cuda_status(e);
+        }
+        ProfScope ps(ctx, "k_gf_tc", st);
+        return cuda_status(gf::launch_tc(r.shape, a, b, z, r.m, pre, ctx->d_status,
+                                         gf::may_depend(st) && !ctx->prof_on, st));
     }
     if (!r.gf) return enqueue_blocks(ctx, r.bl, x, y, z, sc, r.tmp_off, r.pre_off, st);
     r.ops.a0.map.src = x;

@@ -1020,6 +1020,25 @@ __global__ void __launch_bounds__(256) k_gf_sum(int lg, uint32_t na, uint32_t ni
     store_tile<13>(sm, P, out + ((uint64_t)win << (lg - 5)) + tile_base(P, tile), threadIdx.x, 256);
 }
 
+// The operands of a dense product as plain bits: a_t at bit 256 + t, b_k at bit k,
+// zeros around; z cleared.
+__global__ void __launch_bounds__(256) k_gf_tc_prep(const __grid_constant__ Ops q, int lg, uint32_t aw, uint32_t bw,
+                                                    uint32_t zw, uint32_t *__restrict__ a, uint32_t *__restrict__ b,
+                                                    uint32_t *__restrict__ z) {
+    const uint32_t i = blockIdx.x * 256 + threadIdx.x, nw = 1u << (lg - 5);
+    uint32_t v[1];
+    let_next_start();
+    if (i < aw) {
+        in_words<1>(q.a0, lin_of(q.a0, false, lg), false, lg, [&](int) -> uint32_t { return i - 8 < nw ? i - 8 : ~0u; }, v);
+        a[i] = v[0];
+    }
+    if (i < bw) {
+        in_words<1>(q.b0, lin_of(q.b0, true, lg), true, lg, [&](int) -> uint32_t { return i < nw ? nw - 1 - i : ~0u; }, v);
+        b[i] = __brev(v[0]);
+    }
+    if (i < zw) z[i] = 0;
+}
+
 __global__ void __launch_bounds__(256) k_gf_same(const SameOp *__restrict__ ops) {
     const SameOp o = ops[blockIdx.x];
     const uint64_t words = (o.n + 63) >> 6;
@@ -1137,6 +1156,18 @@ uint32_t product_launches(const Product &p, const Ops &q) {
 
 cudaError_t launch_same(const SameOp *ops, uint32_t count, cudaStream_t st) {
     k_gf_same<<<dim3(count, 8), 256, 0, st>>>(ops);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tc_prep(const Ops &q, const TcShape &s, uint32_t *a, uint32_t *b, uint64_t *z, uint64_t m,
+                           cudaStream_t st) {
+    const uint64_t zw = 2 * ((m + 63) / 64);
+    uint64_t n = s.a_words > s.b_words ? s.a_words : s.b_words;
+    if (zw > n) n = zw;
+    int lg = 5;
+    while ((1ull << lg) < 32 * n) ++lg;
+    k_gf_tc_prep<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(q, lg, (uint32_t)s.a_words, (uint32_t)s.b_words, (uint32_t)zw, a,
+                                                              b, reinterpret_cast<uint32_t *>(z));
     return cudaGetLastError();
 }
 

@@ -12,6 +12,35 @@ struct cm_ctx;
 namespace cm {
 namespace gf {
 
+// The tensor-core product starts as a programmatic dependent of the launch that
+// lays out its operands: barriers, tensor memory and scales are ready when those
+// are.  (Launching the transforms' kernels this way measured slower, 199 -> 216 us
+// at 2^25: a kernel's early CTAs crowd the SMs that happen to be free.)
+#ifdef __CUDACC__
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class K, class... A>
+cudaError_t launch_after(bool dependent, K kern, uint32_t grid, uint32_t block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+// Dependent launches may be used on st (not under stream capture, where the
+// graphs of a batch keep plain edges).
+inline bool may_depend(cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+}
+#endif
+
 // One operand block: bit j of its array is map(base + j) for j < lim (a), or
 // map(base + 2^lg - 1 - j) (b, reversed; lim unused).
 struct InOp {
@@ -72,6 +101,18 @@ uint32_t product_launches(const Product &p, const Ops &ops);
 constexpr int kDenseMaxLg = 13;
 cudaError_t launch_dense(const BitMap &a, const BitMap &b, uint32_t K, uint32_t m, bool check, uint64_t *z,
                          uint32_t *status, uint32_t *pre, cudaStream_t st);
+
+// Dense product on the tensor cores (cm_gf2_tc.cu): the shape of K terms and m
+// outputs (stages: the longest CTA chain's, the time's measure), the operands as
+// plain bits (a after 256 zero bits; b in order) with z cleared, the product.
+struct TcShape {
+    uint64_t rows, chunks, splits, per, a_words, b_words, stages;
+};
+TcShape tc_shape(uint64_t K, uint64_t m, int nsm);
+cudaError_t launch_tc_prep(const Ops &q, const TcShape &s, uint32_t *a, uint32_t *b, uint64_t *z, uint64_t m,
+                           cudaStream_t st);
+cudaError_t launch_tc(const TcShape &s, const uint32_t *a, const uint32_t *b, uint64_t *z, uint64_t m,
+                      const uint32_t *pre, uint32_t *status, bool dependent, cudaStream_t st);
 
 // Host image of the device tables.
 constexpr int kTables = 2 * (kMaxLg - kMinLg + 1);

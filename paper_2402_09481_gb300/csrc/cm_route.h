@@ -10,7 +10,8 @@
 namespace cm {
 
 struct Route {
-    bool gf = false, dense = false;
+    bool gf = false, dense = false, tc = false;
+    gf::TcShape shape;
     gf::Product prod;
     gf::Ops ops;  // pointers filled in by enqueue_route
     int kind;

@@ -30,76 +30,19 @@
 
 #include "cm_internal.h"
 #include "cm_ss_f4.h"
+#include "tc05.cuh"
 
 namespace cm {
+
+using namespace tc;
 
 namespace {
 
 constexpr int kStages = 3, kChunk = 256;              // K elements a stage: rows of 128 bytes
-constexpr int kRows = 224;                            // outputs a CTA
 constexpr int kInBytes = 256 * 128, kTileBytes = kRows * 128;
 constexpr int kStageBytes = kInBytes + kTileBytes;
 constexpr int kSmem = kStages * kStageBytes + 1024;   // 1 KB to align
-constexpr uint32_t kScaleCol = 2 * kRows;             // tensor memory columns of scales
 constexpr int kF4Threads = 14 * 32;
-constexpr uint64_t kWaitNs = 2000000000ull;
-
-__device__ __forceinline__ uint32_t saddr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ uint64_t now_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ bool try_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok;
-}
-
-// False when the wait ran out (here or, through `dead`, in another warp).
-__device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity, volatile uint32_t *dead) {
-    if (try_wait(bar, parity)) return true;
-    const uint64_t t0 = now_ns();
-    while (!try_wait(bar, parity)) {
-        if (*dead) return false;
-        if (now_ns() - t0 > kWaitNs) {
-            *dead = 1;
-            return false;
-        }
-    }
-    return true;
-}
-
-__device__ __forceinline__ void arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-// Shared-memory operand descriptor: K-major rows of 128 bytes, 128-byte
-// swizzle, 1024 bytes between groups of 8 rows.
-__device__ __forceinline__ uint64_t operand(uint32_t addr) {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
-}
-
-// e2m1 x e2m1 -> f32, ue8m0 scales, M = 128, N = 224, both operands K-major.
-constexpr uint32_t kInstr = (1u << 7) | (1u << 10) | ((uint32_t)(kRows >> 3) << 17) | (1u << 23) | ((128u >> 4) << 24);
-
-__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t scale, bool add) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%5], [%5], p;\n}" ::"r"(d),
-        "l"(a), "l"(b), "r"(kInstr), "r"((uint32_t)add), "r"(scale)
-        : "memory");
-}
-
-__device__ __forceinline__ void commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
 
 __global__ void __launch_bounds__(kF4Threads, 1) k_ss_f4(const uint8_t *__restrict__ T, uint32_t chunks, uint32_t pblocks,
                                                        const uint64_t *__restrict__ X, uint64_t n, uint64_t wx,
@@ -132,15 +75,7 @@ __global__ void __launch_bounds__(kF4Threads, 1) k_ss_f4(const uint8_t *__restri
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_at;
-    if (warp < 4) {  // every scale 1.0 (127), whatever row and block it is read for
-#pragma unroll 1
-        for (uint32_t c = 0; c < 64; c += 8)
-            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(
-                             tmem + ((warp * 32u) << 16) + kScaleCol + c),
-                         "r"(0x7F7F7F7Fu)
-                         : "memory");
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    }
+    if (warp < 4) set_scales(tmem, warp);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -174,8 +109,7 @@ __global__ void __launch_bounds__(kF4Threads, 1) k_ss_f4(const uint8_t *__restri
                     for (int h = 0; h < 2; ++h) {
                         const uint32_t b = (uint32_t)(w[i] >> (32 * h));
                         *reinterpret_cast<uint4 *>(dst + i * 1024 + (((2 * q + h) ^ (r0 & 7u)) << 4)) =
-                            make_uint4(b & 0x11111111u, (b >> 1) & 0x11111111u, (b >> 2) & 0x11111111u,
-                                       (b >> 3) & 0x11111111u);
+                            nibbles(b);
                     }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 arrive(full + 8 * s);
@@ -232,22 +166,7 @@ __global__ void __launch_bounds__(kF4Threads, 1) k_ss_f4(const uint8_t *__restri
                 uint32_t word[7];
 #pragma unroll
                 for (int q = 0; q < 7; ++q) {
-                    uint32_t v[32];
-                    const uint32_t at = tmem + ((warp * 32u) << 16) + kRows * h + 32 * q;
-                    asm volatile(
-                        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-                          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-                          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-                        : "r"(at));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    uint32_t o = 0;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        o = __funnelshift_r(o, __float_as_uint(__uint_as_float(v[j]) + 2097152.0f), 1);
-                    word[q] = o;
+                    word[q] = parities(tmem + ((warp * 32u) << 16) + kRows * h + 32 * q);
                 }
                 if (c < count) {
                     uint32_t *row = reinterpret_cast<uint32_t *>(Z + c * wz);
@@ -304,8 +223,7 @@ __global__ void __launch_bounds__(256) k_ss_f4_rows(const uint32_t *__restrict__
             if (cnt < 32) w &= (1u << cnt) - 1u;
         }
         uint8_t *row = T + blk * kTileBytes + r * 128;
-        *reinterpret_cast<uint4 *>(row + ((g ^ (r & 7u)) << 4)) =
-            make_uint4(w & 0x11111111u, (w >> 1) & 0x11111111u, (w >> 2) & 0x11111111u, (w >> 3) & 0x11111111u);
+        *reinterpret_cast<uint4 *>(row + ((g ^ (r & 7u)) << 4)) = nibbles(w);
     }
 }
 
@@ -317,8 +235,7 @@ __global__ void __launch_bounds__(256) k_ss_f4_pack(const uint32_t *__restrict__
         const uint32_t r = (uint32_t)(rr - blk * kRows);
         const uint64_t i = kRows * p + r, j = 8 * k + g;
         const uint32_t w = i < m && j < gw ? __ldg(G + i * gw + j) : 0u;
-        *reinterpret_cast<uint4 *>(T + blk * kTileBytes + r * 128 + ((g ^ (r & 7u)) << 4)) =
-            make_uint4(w & 0x11111111u, (w >> 1) & 0x11111111u, (w >> 2) & 0x11111111u, (w >> 3) & 0x11111111u);
+        *reinterpret_cast<uint4 *>(T + blk * kTileBytes + r * 128 + ((g ^ (r & 7u)) << 4)) = nibbles(w);
     }
 }
 

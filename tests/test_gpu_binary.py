@@ -173,3 +173,47 @@ def test_dense_form_matches(cm_ctx, q30, kind, n, m):
             assert cm_ctx.device_status()[0] == native.CM_EPRECOND
             assert cm_ctx.extract_host(D, torch.from_numpy(c.view(np.int64)), n, y.cpu(), m, zh) == native.CM_EPRECOND
             cm_ctx.device_status()
+
+
+TENSOR = [(T, 2 ** 17, 2), (T, 3, 2 ** 17 - 1), (T, 300007, 150001), (T, 131000, 224 * 256), (T, 131000, 224 * 256 + 1),
+          (T, 256 * 600 - 223, 223), (T, 256 * 600 - 222, 225), (C, 200000, 100001), (C, 140000, 77), (D, 150000, 149000),
+          (D, 262000, 65)]
+
+
+@pytest.mark.parametrize("kind,n,m", TENSOR)
+def test_tensor_core_form_matches(cm_ctx, q30, kind, n, m):
+    # dense products on the tensor cores: edges of its 256-window, 224-output and
+    # 256-term tiles, against the integer transforms and the oracle
+    n, m = resolve(kind, n, m)
+    xw, yw = inputs.bernoulli_half(51 + n % 97, n), inputs.bernoulli_half(52 + m % 89, ybits(kind, n, m))
+    if kind == D:
+        xw[0] = (xw[0] | np.uint64(1)) & ~np.uint64(2)
+    x, y = to_dev(xw), to_dev(yw)
+    cm_ctx.profile_enable(True)
+    cm_ctx.profile_read(reset=True)
+    z = run(cm_ctx, kind, n, m, x, y)
+    prof = cm_ctx.profile_read(reset=True)
+    cm_ctx.profile_enable(False)
+    assert prof["k_gf_tc"][0] == 1
+    assert torch.equal(z, run(q30, kind, n, m, x, y))
+    assert cm_ctx.device_status() == (native.CM_OK, 0)
+    zw = from_dev(z)
+    rows = np.unique(np.random.default_rng(m).integers(0, m, 8))
+    got = ((zw[rows >> 6] >> (rows & 63).astype(np.uint64)) & np.uint64(1)).astype(np.uint8)
+    fn = {T: lambda: oracle.toeplitz_rows(xw, n, yw, m, rows), C: lambda: oracle.circulant_rows(xw, n, yw, m, rows),
+          D: lambda: oracle.dodis_rows(xw, yw, n, m, rows)}[kind]
+    assert (got == fn()).all()
+    if kind == D:
+        for fill in (0, 1):
+            c = to_dev(ex.pack_bits(np.full(n, fill, dtype=np.uint8)))
+            assert not from_dev(run(cm_ctx, D, n, m, c, y)).any()
+            assert cm_ctx.device_status()[0] == native.CM_EPRECOND
+
+
+def test_tensor_core_form_largest_counts(cm_ctx):
+    # all ones: every count is n, in shares of up to 2^14 terms
+    for n, m in ((300_000, 1000), (300_001, 1000)):
+        x = torch.full((native.words(n),), -1, dtype=torch.int64, device="cuda")
+        y = torch.full((native.words(n + m - 1),), -1, dtype=torch.int64, device="cuda")
+        z = from_dev(run(cm_ctx, T, n, m, x, y))
+        assert int(sum(bin(int(w)).count("1") for w in z)) == (m if n & 1 else 0)

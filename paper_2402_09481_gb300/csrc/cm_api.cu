@@ -984,6 +984,24 @@ static void build_tables25(std::vector<uint32_t> &h) {
         }
 }
 
+// The tables' host images: constants, computed by the process's first context
+// (about 2 ms) and kept for the others (3 MB).
+struct HostTables {
+    std::vector<uint64_t> gl;
+    std::vector<uint32_t> f30, f25;
+    std::vector<gf::Pass> gf;
+    HostTables() : gf(gf::kTables) {
+        build_tables(gl);
+        build_tables30(f30);
+        build_tables25(f25);
+        gf::build_tables(gf.data());
+    }
+};
+static const HostTables &host_tables() {
+    static const HostTables t;
+    return t;
+}
+
 }  // namespace cm
 
 using namespace cm;
@@ -1020,11 +1038,10 @@ extern "C" cm_status cm_create(cm_ctx **out, int device, const cm_options *opt) 
     uint64_t thr = UINT64_MAX;
     cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &thr);
 
-    std::vector<uint64_t> h;
-    build_tables(h);
-    std::vector<uint32_t> h30, h25;
-    build_tables30(h30);
-    build_tables25(h25);
+    const HostTables &ht = host_tables();
+    const std::vector<uint64_t> &h = ht.gl;
+    const std::vector<uint32_t> &h30 = ht.f30, &h25 = ht.f25;
+    const std::vector<gf::Pass> &hg = ht.gf;
     if (cudaMalloc(&c->d_tables, h.size() * sizeof(uint64_t)) != cudaSuccess ||
         cudaMalloc(&c->d_tables30, h30.size() * sizeof(uint32_t)) != cudaSuccess ||
         cudaMalloc(&c->d_tables25, h25.size() * sizeof(uint32_t)) != cudaSuccess ||
@@ -1049,8 +1066,6 @@ extern "C" cm_status cm_create(cm_ctx **out, int device, const cm_options *opt) 
     c->rt30.big_lo_inv = c->rt30.big_hi_fwd + 32768;
     c->rt30.big_hi_inv = c->rt30.big_lo_inv + 32768;
     c->rt30.bits16 = c->rt30.big_hi_inv + 32768;
-    std::vector<gf::Pass> hg(gf::kTables);
-    gf::build_tables(hg.data());
     cudaMemcpy(c->d_gf, hg.data(), hg.size() * sizeof(gf::Pass), cudaMemcpyHostToDevice);
     cudaMemset(c->d_status, 0, 64);
     c->rt.small = c->d_tables;

@@ -330,22 +330,39 @@ def plan_params(kind: int, model: int, adversary: int, n_raw: int, k1: float, lo
                 k1=float(p.k1), k2=float(p.k2), m=int(p.m))
 
 
-def _stream_handle(stream) -> int:
+_torch = None       # torch and what a call needs of it, looked up once
+_word_types = ()
+_raw_stream = None
+
+
+def _load_torch():
+    global _torch, _word_types, _raw_stream
     import torch
+    _word_types = (torch.int64, torch.uint64)
+    # the current stream's handle without a Stream object (about 2 us of a 10 us call)
+    get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    _raw_stream = (lambda: get(dev())) if get and dev else (lambda: torch.cuda.current_stream().cuda_stream)
+    _torch = torch
+
+
+def _stream_handle(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        if _torch is None:
+            _load_torch()
+        return _raw_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
 
 
 def _dev_words(t, nbits: int, name: str):
-    import torch
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+    if _torch is None:
+        _load_torch()
+    if not isinstance(t, _torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor of 64-bit words")
-    if t.dtype not in (torch.int64, torch.uint64) or not t.is_contiguous():
+    if t.dtype not in _word_types or not t.is_contiguous():
         raise TypeError(f"{name} must be a contiguous int64/uint64 tensor")
-    if t.numel() < words(nbits):
+    if t.numel() < (nbits + 63) // 64:
         raise ValueError(f"{name} holds {t.numel()} words, needs {words(nbits)} for {nbits} bits")
     return t.data_ptr()
 
@@ -380,18 +397,16 @@ class Context:
             pass
 
     def _out(self, z, m, like):
-        import torch
         if z is None:
-            z = torch.empty(words(m), dtype=torch.int64, device=like.device)
-        _dev_words(z, m, "z")
-        return z
+            z = _torch.empty(words(m), dtype=_torch.int64, device=like.device)
+        return z, _dev_words(z, m, "z")
 
     def toeplitz(self, x, n: int, y, m: int, z=None, stream=None):
         """z = toep(y) x over GF(2): x has n bits, y has n + m - 1 bits."""
         px = _dev_words(x, n, "x")
         py = _dev_words(y, n + m - 1, "y")
-        z = self._out(z, m, x)
-        _check(self._L.cm_toeplitz(self._h, px, n, py, m, z.data_ptr(), _stream_handle(stream)),
+        z, pz = self._out(z, m, x)
+        _check(self._L.cm_toeplitz(self._h, px, n, py, m, pz, _stream_handle(stream)),
                "cm_toeplitz")
         return z
 
@@ -399,8 +414,8 @@ class Context:
         """Circulant(x, y): x has n bits, y has n + 1 bits (n + 1 prime in N_A)."""
         px = _dev_words(x, n, "x")
         py = _dev_words(y, n + 1, "y")
-        z = self._out(z, m, x)
-        _check(self._L.cm_circulant(self._h, px, n, py, m, z.data_ptr(), _stream_handle(stream)),
+        z, pz = self._out(z, m, x)
+        _check(self._L.cm_circulant(self._h, px, n, py, m, pz, _stream_handle(stream)),
                "cm_circulant")
         return z
 
@@ -408,8 +423,8 @@ class Context:
         """Dodis et al.(x, y): both n bits, n prime in N_A."""
         px = _dev_words(x, n, "x")
         py = _dev_words(y, n, "y")
-        z = self._out(z, m, x)
-        _check(self._L.cm_dodis(self._h, px, py, n, m, z.data_ptr(), _stream_handle(stream)),
+        z, pz = self._out(z, m, x)
+        _check(self._L.cm_dodis(self._h, px, py, n, m, pz, _stream_handle(stream)),
                "cm_dodis")
         return z
 
@@ -420,8 +435,8 @@ class Context:
         ybits = {TOEPLITZ: n1 + m1 - 1, CIRCULANT: n1 + 1, DODIS: n1}.get(kind1, 0)
         px = _dev_words(x, n1, "x")
         py = _dev_words(y, ybits, "y")
-        z = self._out(z, m1 + m2, x)
-        _check(self._L.cm_compose(self._h, kind1, px, n1, py, m1, kind2, n2, m2, z.data_ptr(),
+        z, pz = self._out(z, m1 + m2, x)
+        _check(self._L.cm_compose(self._h, kind1, px, n1, py, m1, kind2, n2, m2, pz,
                                   _stream_handle(stream)), "cm_compose")
         return z
 
@@ -457,8 +472,8 @@ class Context:
         """m RSH one-bit extractions of x; one-bit seed i = bits 2 l i .. 2 l i + 2l - 1 of seeds."""
         _dev_words(x, n, "x")
         _dev_words(seeds, 2 * l * m, "seeds")
-        z = self._out(z, m, x)
-        _check(self._L.cm_trevisan_rsh(self._h, x.data_ptr(), n, l, seeds.data_ptr(), m, z.data_ptr(),
+        z, pz = self._out(z, m, x)
+        _check(self._L.cm_trevisan_rsh(self._h, x.data_ptr(), n, l, seeds.data_ptr(), m, pz,
                                        _stream_handle(stream)), "cm_trevisan_rsh")
         return z
 
@@ -468,9 +483,9 @@ class Context:
         _dev_words(y, d, "y")
         if sets.device.type != "cuda" or sets.numel() < m * t or sets.element_size() != 4:
             raise ValueError("sets: a CUDA tensor of m * t 32-bit indices")
-        z = self._out(z, m, x)
+        z, pz = self._out(z, m, x)
         _check(self._L.cm_trevisan(self._h, x.data_ptr(), n, y.data_ptr(), d, sets.data_ptr(), t, m, l,
-                                   z.data_ptr(), _stream_handle(stream)), "cm_trevisan")
+                                   pz, _stream_handle(stream)), "cm_trevisan")
         return z
 
     def von_neumann_host(self, x, n: int, z, stream=None) -> tuple[int, int]:

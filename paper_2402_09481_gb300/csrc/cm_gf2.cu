@@ -984,6 +984,11 @@ __global__ void __launch_bounds__(128) k_gf_fwd(int lg, uint32_t na, const Pass 
 
 // ... and a window's sum of products with the inverse: window w adds a's block
 // i times b's block i + w over i < nin.  One thread a point word (32 elements).
+__device__ __forceinline__ void load32(uint32_t (&v)[32], const uint32_t *p) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __ldg(p + (j << 8));
+}
+
 __global__ void __launch_bounds__(256) k_gf_sum(int lg, uint32_t na, uint32_t nin, const Pass *__restrict__ table,
                                                 const uint32_t *__restrict__ hat, uint32_t *__restrict__ out) {
     __shared__ __align__(16) uint32_t sm[8192];
@@ -1002,11 +1007,8 @@ __global__ void __launch_bounds__(256) k_gf_sum(int lg, uint32_t na, uint32_t ni
     for (int j = 0; j < 32; ++j) acc[j] = 0;
     for (uint32_t i = 0; i < nin; ++i) {
         uint32_t a[32], b[32], o[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            a[j] = __ldg(ha + (j << 8));
-            b[j] = __ldg(hb + (j << 8));
-        }
+        load32(a, ha);
+        load32(b, hb);
         mul<5>(a, b, o);
 #pragma unroll
         for (int j = 0; j < 32; ++j) acc[j] ^= o[j];
@@ -1018,6 +1020,75 @@ __global__ void __launch_bounds__(256) k_gf_sum(int lg, uint32_t na, uint32_t ni
     __syncthreads();
     inverse_levels<13, 5>(sm, P, base, 256);
     store_tile<13>(sm, P, out + ((uint64_t)win << (lg - 5)) + tile_base(P, tile), threadIdx.x, 256);
+}
+
+// Two windows at a time: a_0, a_1 (blocks i, i + 1) and B_0, B_1, B_2 (blocks
+// i + w ..) give w and w + 1 with three products for four,
+//   a_0 B_0 + a_1 B_1 = a_0 (B_0 + B_1) + (a_0 + a_1) B_1,
+//   a_0 B_1 + a_1 B_2 = a_1 (B_1 + B_2) + (a_0 + a_1) B_1,
+// and both inverses run together, one on each half of the threads.
+__global__ void __launch_bounds__(256) k_gf_sum2(int lg, uint32_t na, uint32_t nb, uint32_t nin, uint32_t nz,
+                                                 const Pass *__restrict__ table, const uint32_t *__restrict__ hat,
+                                                 uint32_t *__restrict__ out) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    __shared__ Pass P;
+    __shared__ uint32_t base[kMaxLev];
+    const uint32_t tile = blockIdx.x & ((1u << (lg - 18)) - 1u), win = 2 * (blockIdx.x >> (lg - 18));
+    load_pass(&P, table);
+    __syncthreads();
+    if (threadIdx.x < P.nlev)
+        base[threadIdx.x] = ext_twiddle(P.lev[threadIdx.x], P.lev[threadIdx.x].base[1], tile);
+    const uint32_t at = phys(threadIdx.x);
+    const uint32_t *h0 = hat + ((uint64_t)tile << 13) + at;
+    auto block = [&](uint32_t k) { return h0 + ((uint64_t)k << (lg - 5)); };
+    uint32_t w0[32], w1[32], a[32], b[32], o[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) w0[j] = w1[j] = 0;
+#pragma unroll 1
+    for (uint32_t i = 0; i < nin; i += 2) {
+        const bool odd = i + 1 == nin;  // no a_1
+        const uint32_t last = nb - 1, k0 = i + win, k1 = k0 + 1 < last ? k0 + 1 : last, k2 = k0 + 2 < last ? k0 + 2 : last;
+        const uint32_t *a0 = block(i), *a1 = block(i + 1), *b0 = block(na + k0), *b1 = block(na + k1), *b2 = block(na + k2);
+#pragma unroll 1
+        for (int t = 0; t < (odd ? 2 : 3); ++t) {
+            // t = 0: (a_0 + a_1) B_1 to both; 1: a_0 (B_0 + B_1) to w; 2: a_1 (B_1 + B_2) to w + 1
+            load32(a, t == 2 ? a1 : a0);
+            if (t == 0 && !odd) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) a[j] ^= __ldg(a1 + (j << 8));
+            }
+            load32(b, b1);
+            if (t) {
+                const uint32_t *bx = t == 1 ? b0 : b2;
+#pragma unroll
+                for (int j = 0; j < 32; ++j) b[j] ^= __ldg(bx + (j << 8));
+            }
+            mul<5>(a, b, o);
+            const uint32_t m0 = t == 2 ? 0u : ~0u, m1 = t == 1 ? 0u : ~0u;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                w0[j] ^= o[j] & m0;
+                w1[j] ^= o[j] & m1;
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        sm[at + (j << 8)] = w0[j];
+        sm[8192 + at + (j << 8)] = w1[j];
+    }
+    __syncthreads();
+    const uint32_t h = threadIdx.x >> 7, tid = threadIdx.x & 127u;
+    uint32_t *mine = sm + 8192 * h;
+    for (int l = (int)P.nlev - 1; l >= 0; --l) {
+        level<13, 8, 5, true>(mine, P.lev[l], base[l], l >= (int)P.npre, tid, 128);
+        __syncthreads();
+        if (l == (int)P.npre) {
+            transpose_bits<13>(mine, P, tid >> 5, 4);
+            __syncthreads();
+        }
+    }
+    if (win + h < nz) store_tile<13>(mine, P, out + ((uint64_t)(win + h) << (lg - 5)) + tile_base(P, tile), tid, 128);
 }
 
 // The operands of a dense product as plain bits: a_t at bit 256 + t, b_k at bit k,
@@ -1197,7 +1268,12 @@ cudaError_t launch_product(cm_ctx *c, int nsm, const Product &p, const Ops &q, c
         }
         out = data;  // the operands' arrays are free again: na + nb >= nz of them
         Scope ps(c, "k_gf_sum", st);
-        k_gf_sum<<<q.nz << (p.lg - 18), 256, 0, st>>>(p.lg, q.na, p.nin, mid, hat, out);
+        if (q.nz > 1) {
+            if ((e = smem_attr_once<k_gf_sum2>(65536)) != cudaSuccess) return e;
+            k_gf_sum2<<<(q.nz + 1) / 2 << (p.lg - 18), 256, 65536, st>>>(p.lg, q.na, q.nb, p.nin, q.nz, mid, hat, out);
+        } else {
+            k_gf_sum<<<1 << (p.lg - 18), 256, 0, st>>>(p.lg, q.na, p.nin, mid, hat, out);
+        }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     } else {
         Scope ps(c, "k_gf_mid", st);

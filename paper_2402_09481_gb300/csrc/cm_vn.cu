@@ -16,7 +16,8 @@
 //   k_vn_write  re-reads each tile, compresses every word with a 64 KiB
 //               shared-memory table (one byte per 16-bit chunk: the outputs of
 //               those 8 pairs, in order), packs the bits into a shared staging
-//               buffer aligned to the tile's global output offset, and writes
+//               buffer aligned to the tile's global output offset (32-bit words:
+//               0.414 -> 0.389 ms at 6.5e9 bits against 64-bit atomics), and writes
 //               the words it alone owns with plain coalesced stores and the
 //               shared ones with atomic ORs into the zeroed words.
 //
@@ -285,25 +286,29 @@ k_vn_write(const uint64_t *__restrict__ x, uint64_t words, uint64_t lastmask, ui
             }
             __syncthreads();
 
-            // ---- pack; staging word i is output word (O >> 6) + i ----
+            // ---- pack into 32-bit words; staging word i is the 32 output bits from
+            // bit 64 (O >> 6) + 32 i.  A thread's bits are one run: the words it
+            // fills alone are stored, its first and last are ORed in (32-bit shared
+            // atomics are native, 64-bit ones a compare-and-swap loop).
             const uint32_t start = s0 + wsum[32 + warp] + (inc - total);
+            uint32_t *st32 = reinterpret_cast<uint32_t *>(stage);
+            uint32_t pos = start & 31, k = start >> 5;
             uint64_t acc = 0;
-            uint32_t pos = start & 63, k = start >> 6;
+            bool shared_word = pos != 0;
 #pragma unroll
             for (int i = 0; i < kVnWpt; ++i) {
-                const uint32_t c = oc[i], v = ov[i];
-                if (c == 0) continue;
-                acc |= (uint64_t)v << pos;
-                if (pos + c >= 64) {  // pos >= 32 here
-                    atomicOr(reinterpret_cast<unsigned long long *>(stage + k), (unsigned long long)acc);
+                acc |= (uint64_t)ov[i] << pos;  // pos <= 31, 32 bits at most
+                pos += oc[i];
+                if (pos >= 32) {
+                    if (shared_word) atomicOr(st32 + k, (uint32_t)acc);
+                    else st32[k] = (uint32_t)acc;
+                    shared_word = false;
                     ++k;
-                    acc = (uint64_t)v >> (64 - pos);
-                    pos = pos + c - 64;
-                } else {
-                    pos += c;
+                    acc >>= 32;
+                    pos -= 32;
                 }
             }
-            if (pos) atomicOr(reinterpret_cast<unsigned long long *>(stage + k), (unsigned long long)acc);
+            if (pos) atomicOr(st32 + k, (uint32_t)acc);
         }
         // the next tile's words load while this one is written out
         uint64_t nxt[kVnWpt];

@@ -34,6 +34,7 @@
 
 #include "cm.h"
 #include "cm_batch_internal.h"
+#include "cm_route.h"
 #include "cm_ctx.h"
 #include "cm_internal.h"
 
@@ -122,6 +123,7 @@ struct Slot {
     size_t foot = 0;
     uint64_t wave = 0;
     Buf insts, items, ctrl, flags;  // flags: [0] status word, then 2 words per request
+    Buf gf;                         // operand, window and input lists of the wave's groups
     std::vector<std::pair<SeedKey, bool>> seeds;  // cache entries used (true: created by this wave)
 };
 
@@ -256,6 +258,28 @@ struct Wave {
     std::vector<SeedEntry *> make;  // per request: a new entry whose buffer the launch allocates
 };
 
+// Requests of one transform length that run as binary polynomials in a group of
+// launches (cm_gf2.cu); off: their arrays in the wave's scratch.
+struct WaveGroup {
+    int lg;
+    std::vector<uint32_t> idx;
+    size_t off = 0;
+};
+
+// Groups are for transforms of 2^18 .. 2^25 with at least 2^22 elements in all: a
+// group takes 130 to 190 us whatever it holds up to there, the work list and the
+// single calls about 35 us per 2^20 elements.
+constexpr int kGroupMinLg = 18;
+constexpr uint64_t kGroupMinElements = 1ull << 22;
+
+// log2 of the transform that holds the request's K + m - 1 terms.
+int request_lg(const cm_desc &d) {
+    const uint64_t terms = (d.kind == CM_CIRCULANT ? d.n + 1 : d.n) + d.m - 1;
+    int lg = 0;
+    while (lg < 40 && (1ull << lg) < terms) ++lg;
+    return lg;
+}
+
 // Waves that may pass a queued request whose scratch does not fit; after
 // that, nothing behind it is admitted until it fits.
 constexpr uint32_t kMaxPassed = 16;
@@ -386,7 +410,8 @@ bool admit_wave(cm_server *S, Slot &sl, Wave &w) {
 // touches only the slot, the wave's copies and the seed entries it created,
 // which no other thread reads).
 cm_status enqueue_wave(cm_server *S, Slot &sl, Wave &w, uint8_t *scratch, const std::vector<size_t> &off,
-                       const std::vector<uint32_t> &wl, const std::vector<uint32_t> &solo) {
+                       const std::vector<uint32_t> &wl, const std::vector<uint32_t> &solo,
+                       const std::vector<WaveGroup> &groups, Route *lone) {
     cm_ctx *ctx = S->ctx;
     const uint32_t n = (uint32_t)w.r.size();
     std::vector<cm_desc> descs(n);
@@ -397,7 +422,14 @@ cm_status enqueue_wave(cm_server *S, Slot &sl, Wave &w, uint8_t *scratch, const 
     }
     // flags: status word, pad, then a pair per work-list instance (index k) and
     // one per single-call request (index wl.size() + i)
-    const size_t flag_words = 2 + 2 * ((size_t)n + n);
+    // then the groups' Dodis et al. requests
+    size_t grouped = 0, group_dodis = 0;
+    for (const WaveGroup &g : groups)
+        for (uint32_t i : g.idx) {
+            ++grouped;
+            group_dodis += w.r[i].d.kind == CM_DODIS;
+        }
+    const size_t group_pair = 2 * (size_t)n, flag_words = 2 + 2 * (group_pair + group_dodis);
     if (!sl.flags.ensure(flag_words * 4)) return CM_ENOMEM;
     uint32_t *dflags = static_cast<uint32_t *>(sl.flags.dev);
     std::vector<void *> bext(wl.size(), nullptr);
@@ -439,6 +471,66 @@ cm_status enqueue_wave(cm_server *S, Slot &sl, Wave &w, uint8_t *scratch, const 
                            sl.st) != cudaSuccess)
             return CM_EDEVICE;
     }
+    if (grouped) {
+        const size_t out_at = r256(2 * grouped * sizeof(gf::InOp)), same_at = r256(out_at + grouped * sizeof(gf::OutOp)),
+                     bytes = same_at + group_dodis * sizeof(gf::SameOp) + 8;
+        if (!sl.gf.ensure(bytes)) return CM_ENOMEM;
+        uint8_t *h = static_cast<uint8_t *>(sl.gf.host), *d = static_cast<uint8_t *>(sl.gf.dev);
+        gf::InOp *hin = reinterpret_cast<gf::InOp *>(h);
+        gf::OutOp *hout = reinterpret_cast<gf::OutOp *>(h + out_at);
+        gf::SameOp *hsame = reinterpret_cast<gf::SameOp *>(h + same_at);
+        std::vector<gf::Ops> ops(groups.size());
+        size_t ni = 0, no = 0, ns = 0;
+        for (size_t k = 0; k < groups.size(); ++k) {
+            const uint32_t cnt = (uint32_t)groups[k].idx.size();
+            memset(&ops[k], 0, sizeof(ops[k]));
+            ops[k].in = reinterpret_cast<gf::InOp *>(d) + ni;
+            ops[k].out = reinterpret_cast<gf::OutOp *>(d + out_at) + no;
+            ops[k].na = ops[k].nb = ops[k].nz = cnt;
+            for (uint32_t c = 0; c < cnt; ++c) {
+                const uint32_t i = groups[k].idx[c];
+                const cm_desc &q = w.r[i].d;
+                gf::Ops one;
+                gf::Product p;
+                gf_shape(q.kind, q.n, q.m, &p, &one);
+                gf_maps(q.kind, q.n, q.m, &one);
+                one.a0.map.src = q.x;
+                one.b0.map.src = q.y;
+                hin[ni + c] = one.a0;
+                hin[ni + cnt + c] = one.b0;
+                uint32_t *pre = nullptr;
+                if (q.kind == CM_DODIS) {
+                    sl.pre_index[i] = (int)(group_pair + ns);
+                    pre = dflags + 2 + 2 * (group_pair + ns);
+                    hsame[ns++] = gf::SameOp{q.x, q.n, pre};
+                }
+                hout[no + c] = gf::OutOp{q.z, q.m, pre, dflags};
+            }
+            ni += 2 * cnt;
+            no += cnt;
+        }
+        if (cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, sl.st) != cudaSuccess) return CM_EDEVICE;
+        if (ns) {
+            ProfScope ps(ctx, "k_gf_same", sl.st);
+            if (cudaMemsetAsync(dflags + 2 + 2 * group_pair, 0, 8 * ns, sl.st) != cudaSuccess ||
+                gf::launch_same(reinterpret_cast<gf::SameOp *>(d + same_at), (uint32_t)ns, sl.st) != cudaSuccess)
+                return CM_EDEVICE;
+        }
+        for (size_t k = 0; k < groups.size(); ++k)
+            if (gf::launch_product(ctx, ctx->nsm, gf::Product{groups[k].lg, 1}, ops[k], ctx->d_gf, scratch + groups[k].off,
+                                   sl.st) != cudaSuccess)
+                return CM_EDEVICE;
+    }
+    if (lone) {  // a wave of one: the single call
+        const WaveReq &r = w.r[0];
+        cm_status s = enqueue_route(ctx, *lone, r.d.x, r.d.y, r.d.z, scratch, sl.st);
+        if (s != CM_OK) return s;
+        if (r.d.kind == CM_DODIS) {
+            sl.pre_index[0] = 0;
+            if (cudaMemcpyAsync(dflags + 2, scratch + lone->pre_off, 8, cudaMemcpyDeviceToDevice, sl.st) != cudaSuccess)
+                return CM_EDEVICE;
+        }
+    }
     for (uint32_t i : solo) {
         const WaveReq &r = w.r[i];
         uint8_t *sc = scratch + off[i];
@@ -464,10 +556,39 @@ cm_status launch_wave(cm_server *S, Slot &sl, Wave &w) {
     const uint32_t n = (uint32_t)w.r.size();
     std::vector<size_t> off(n, 0);
     std::vector<uint32_t> wl, solo;
+    std::vector<WaveGroup> groups;
+    std::vector<uint8_t> grouped(n, 0);
+    Route route, *lone = nullptr;
     size_t total = 0;
+    if (gf_allowed(S->ctx) && n > 1) {
+        std::vector<uint32_t> by_lg[gf::kMaxLg + 1];
+        for (uint32_t i = 0; i < n; ++i) {
+            const int lg = request_lg(w.r[i].d);
+            if (lg >= kGroupMinLg && lg <= gf::kMaxLg && !w.bext[i] && !w.make[i]) by_lg[lg].push_back(i);
+        }
+        for (int lg = gf::kMaxLg; lg >= kGroupMinLg; --lg) {
+            if ((uint64_t)by_lg[lg].size() << lg < kGroupMinElements) continue;
+            WaveGroup g;
+            g.lg = lg;
+            g.idx = by_lg[lg];
+            g.off = total;
+            total += r256(2 * g.idx.size() << (lg - 3));  // a quarter byte a bit: within the requests' footprints
+            for (uint32_t i : g.idx) grouped[i] = 1;
+            groups.push_back(g);
+        }
+    } else if (n == 1 && request_lg(w.r[0].d) <= gf::kMaxLg && !w.bext[0] && !w.make[0]) {
+        const cm_desc &d = w.r[0].d;
+        if (make_route(S->ctx, d.kind, d.n, d.m, sl.foot, &route) == CM_OK && (route.dense || route.tc || route.gf)) {
+            if (route.dense) route.need = 256;  // its flags
+            lone = &route;
+            grouped[0] = 1;
+            total = r256(route.need);
+        }
+    }
     for (uint32_t i = 0; i < n; ++i) {
         const WaveReq &r = w.r[i];
         off[i] = total;
+        if (grouped[i]) continue;
         if (!r.solo) {
             wl.push_back(i);
             total += worklist_scratch_bytes(r.p);
@@ -482,7 +603,7 @@ cm_status launch_wave(cm_server *S, Slot &sl, Wave &w) {
         cudaGetLastError();
         return CM_ENOMEM;
     }
-    cm_status s = enqueue_wave(S, sl, w, static_cast<uint8_t *>(scratch), off, wl, solo);
+    cm_status s = enqueue_wave(S, sl, w, static_cast<uint8_t *>(scratch), off, wl, solo, groups, lone);
     if (scratch) cudaFreeAsync(scratch, sl.st);
     if (s == CM_OK && cudaEventRecord(sl.ev, sl.st) != cudaSuccess) s = CM_EDEVICE;
     return s;
@@ -543,6 +664,7 @@ void server_release(cm_server *S) {
         sl.items.release();
         sl.ctrl.release();
         sl.flags.release();
+        sl.gf.release();
         if (sl.ev) cudaEventDestroy(sl.ev);
     }
     for (Slot &sl : S->slots)

@@ -73,11 +73,12 @@ def seed_bits(kind, n, m):
 # Any other kernel is keyed on every unit but those of the stand-alone
 # extractors (Von Neumann, Trevisan, shared seed).  Each unit counts with the
 # headers it includes (transitively).
-OWN_UNITS = {"k_vn": ("cm_vn.cu",), "k_rsh": ("cm_trevisan.cu",), "k_ss": ("cm_shared_seed.cu",),
+OWN_UNITS = {"k_vn": ("cm_vn.cu",), "k_rsh": ("cm_trevisan.cu",), "k_ss_f4": ("cm_ss_f4.cu",), "k_ss": ("cm_shared_seed.cu",),
              "k_pass_fwd_bits_f25": ("cm_pass25.cu", "cm_api.cu"), "k_middle_f25": ("cm_pass25.cu", "cm_api.cu"),
              "k_pass_inv_parity_f25": ("cm_pass25.cu", "cm_api.cu"),
              "k_pack_tail": ("cm_launch_misc.cu", "cm_api.cu"), "k_cluster_f25": ("cm_cluster25.cu", "cm_api.cu"),
-             "k_batch": ("cm_batch.cu", "cm_api.cu")}
+             "k_batch": ("cm_batch.cu", "cm_api.cu"), "k_gf_tc": ("cm_gf2_tc.cu", "cm_api.cu"),
+             "k_gf": ("cm_gf2.cu", "cm_gf2_plan.cpp", "cm_api.cu")}
 _INCLUDE = re.compile(r'^\s*#\s*include\s+"([^"]+)"', re.M)
 
 
@@ -604,23 +605,12 @@ def run_batched_a(args, world, rank, local, emit=True):
     assert torch.equal(zp, zd), "batched output differs from the per-call output"
     plain_value = world * out_bits / (statistics.median(plain_ms) * 1e-3) / 1e9
 
-    # roofline of the work-list kernel (the only kernel of a step), in the
-    # path's HBM model: 48 L bytes per instance with 8-byte
-    # elements (on-chip instances, L <= 2^13: the bits only) + the bit I/O; the
-    # work list runs 4-byte elements, so it moves about half of that.  k_batch
-    # runs the instances of the work list (L <= 2^21); the longer ones run the
-    # single-call kernels in the same graph and count in the step's figure only
-    Ls = np.array([native.plan_query(native.TOEPLITZ, int(n), int(m), plan_mode=native.PLAN_SINGLE)
-                   ["transform_length"] for n, m in zip(ns, ms)])
-    onlist = Ls <= (1 << 21)
-    if int((~onlist).sum()) != int(info["solo_instances"]):
-        raise RuntimeError("work-list split differs from the batch's own")
-    big = (Ls > (1 << 13)) & onlist
-    bits = (ns + (ns + ms - 1) + ms) / 8
-    io = float(bits[onlist].sum())
-    alg = float(48 * Ls[big].sum()) + io
-    act = float(24 * Ls[big].sum()) + io
-    alg_step = float(48 * Ls[Ls > (1 << 13)].sum() + bits.sum())
+    # the step against its bound: instances of 2^15 .. 2^25 run as binary
+    # polynomials (their products' ALU-pipe instructions), the shorter ones on the
+    # work list (not counted)
+    Ls = np.array([1 << (int(n) + int(m) - 2).bit_length() for n, m in zip(ns, ms)])
+    ops = sum(binary_ops(*binary_shape(0, int(n), int(m))) for n, m in zip(ns, ms) if int(n) + int(n // 2) > 1 << 14)
+    io = float(((ns + (ns + ms - 1) + ms) / 8).sum())
     peak, peak_src = measured_peaks()
     ctx.profile_enable(True)
     ctx.profile_read(reset=True)
@@ -628,20 +618,15 @@ def run_batched_a(args, world, rank, local, emit=True):
         b.launch()
     prof = ctx.profile_read(reset=True)
     ctx.profile_enable(False)
-    kb = prof.get("k_batch", (1, ms_per_step))
-    per_launch = kb[1] / kb[0]
-    achieved = alg / (per_launch * 1e-3) / 1e9
-    roof = {"bound": "hbm", "kernel": "k_batch", "achieved": achieved, "peak": peak, "unit": "GB/s",
-            "frac": achieved / peak, "peak_source": f"{peak_src} HBM copy bandwidth (MEASURED_PEAKS.json)",
-            "traffic": ncu_traffic("k_batch", "batched_a") if count == 4096 else None,  # the figure is for 4096
-            "model": "48 L bytes per work-list instance with 2^13 < L <= 2^21 (8-byte elements) + their bit I/O",
-            "algorithmic_bytes_per_launch": alg, "avg_launch_ms": per_launch,
-            "work_list_instances": int(onlist.sum()), "single_call_instances": int((~onlist).sum()),
-            "actual_element_bytes": {"bytes_per_launch": act, "achieved": act / (per_launch * 1e-3) / 1e9,
-                                     "frac": act / (per_launch * 1e-3) / 1e9 / peak},
-            "step": {"bytes": alg_step, "achieved": alg_step / (ms_per_step * 1e-3) / 1e9,
-                     "frac": alg_step / (ms_per_step * 1e-3) / 1e9 / peak,
-                     "model": "48 L bytes per instance with L > 2^13 + all bit I/O, over the whole step"}}
+    dom = max(prof, key=lambda k: prof[k][1])
+    rate = 152 * 64 * 2070e6
+    roof = {"bound": "alu", "kernel": dom, "achieved": ops / (ms_per_step * 1e-3) / 1e12, "peak": rate / 1e12,
+            "unit": "T ALU instructions/s (lanes), whole step", "frac": ops / (ms_per_step * 1e-3) / rate,
+            "peak_source": "152 SMs x 64 ALU lanes x 2070 MHz", "avg_launch_ms": prof[dom][1] / prof[dom][0],
+            "traffic": ncu_traffic(dom, "batched_a") if count == 4096 else None,
+            "hbm": {"bytes": io, "achieved": io / (ms_per_step * 1e-3) / 1e9, "peak": peak,
+                    "peak_source": f"{peak_src} HBM copy bandwidth (MEASURED_PEAKS.json)"},
+            "long_instances": int(info["solo_instances"])}
 
     # end to end: host inputs (pinned) -> device, batch, outputs -> host
     xp = torch.from_numpy(xh.view(np.int64)).pin_memory()
@@ -1146,8 +1131,8 @@ def run_trevisan(args, world, rank, local):
         step()
     prof = ctx.profile_read(reset=True)
     ctx.profile_enable(False)
-    c_, t_ = prof["k_rsh"]
-    per_launch = t_ / c_
+    grouped = "k_rsh_join" in prof  # the chunks' matrix on the tensor cores
+    per_launch = sum(t for _, t in prof.values()) / args.steps
     s = -(-n // l)
     # schoolbook GF(2) work: (s - 1) products of l-bit polynomials (l^2 bit
     # AND-XORs each) per output; one LOP3 does 32 of them on one lane
@@ -1155,11 +1140,16 @@ def run_trevisan(args, world, rank, local):
     clk = (sampler.summary(tw0, tw1) or {}).get("sm_mhz") or 2070.0
     peak = NUM_SMS * ALU_LANES_PER_SM * clk * 1e6 * 32 / 1e9
     ach = macs / (per_launch * 1e-3) / 1e9
-    roof = {"bound": "alu", "kernel": "k_rsh", "achieved": ach, "peak": peak, "unit": "G GF(2) bit-MACs/s",
+    if grouped:
+        per_launch = prof["k_ss_f4"][1] / prof["k_ss_f4"][0]
+        ach, peak = macs / (per_launch * 1e-3) / 1e9, 13.5e15 / 2 / 1e9
+    roof = {"bound": "tensor" if grouped else "alu", "kernel": "k_ss_f4" if grouped else "k_rsh", "achieved": ach,
+            "peak": peak, "unit": "G GF(2) bit-MACs/s",
             "frac": ach / peak,
-            "peak_source": f"{NUM_SMS} SMs x {ALU_LANES_PER_SM} ALU lanes x {clk:.0f} MHz measured x 32 "
+            "peak_source": "nominal dense fp4 multiply-adds" if grouped else
+                           f"{NUM_SMS} SMs x {ALU_LANES_PER_SM} ALU lanes x {clk:.0f} MHz measured x 32 "
                            "(one LOP3 = 32 AND + 32 XOR)",
-            "traffic": ncu_traffic("k_rsh", "trevisan"), "avg_launch_ms": per_launch,
+            "traffic": ncu_traffic("k_ss_f4" if grouped else "k_rsh", "trevisan"), "avg_launch_ms": per_launch,
             "gf2_bit_macs_per_launch": macs}
     # end to end: input and seeds from pinned host memory, output back
     xh = torch.from_numpy(xw.view(np.int64)).pin_memory()
@@ -1446,6 +1436,57 @@ def run_served(args, world, rank, local, emit=True):
     return line
 
 
+# LOP3-pipe instructions of one bit-sliced product of 2^f components (32
+# elements): Karatsuba at every step of the tower, three-input XORs merged.
+BINARY_MUL = (1, 5, 23, 84, 290, 966)
+
+
+def binary_shape(kind, n, m):
+    """(lg, na, nb, nz, nin) of the binary-polynomial form of one call: the
+    transforms of 2^lg bits (blocks of a and b, output windows, products a window
+    sums)."""
+    K, N = (n + 1 if kind == 1 else n), 1 << 25
+    if K + m - 1 <= N:
+        return max(15, (K + m - 2).bit_length()), 1, 1, 1, 1
+    if m <= N // 2:
+        a, zs = N - m + 1, m
+    elif K <= N // 2:
+        a, zs = K, (N - K + 1) & ~63
+    else:
+        a, zs = N // 2, N // 2
+    na, nz = -(-K // a), -(-m // zs)
+    return 25, na, na + nz - 1, nz, na
+
+
+def binary_ops(lg, na, nb, nz, nin):
+    """ALU-pipe instructions (lanes) of the form: per level a product per pair of
+    elements and two XORs a word, na + nb forward and nz inverse transforms, and the
+    pointwise products (three for four of a pair of windows); basis conversions,
+    addresses and the twiddles' bits are not counted."""
+    words = 1 << (lg - 5)
+    missing = {lg - (1 << j) for j in range(5)}
+    per = 0.0
+    for i in range(lg):
+        f = sum(lg - (1 << j) > i for j in range(5))
+        per += words / (2 << f) * (BINARY_MUL[f] + (1 if i in missing else 2) * (1 << f))
+    f = 5 if lg >= 16 else 4
+    point = words / (1 << f) * BINARY_MUL[f] * nin * nz * (0.75 if nz > 1 else 1.0)
+    return per * (na + nb + nz) + point
+
+
+def binary_roofline(kind, n, sb, m, ms_per_step, sm_mhz, peak_hbm):
+    """The binary form's bound: its ALU-pipe instructions (64 lanes an SM) against
+    the step, beside the time of its bits at the measured HBM bandwidth."""
+    shape = binary_shape(kind, n, m)
+    ops, rate = binary_ops(*shape), 152 * 64 * sm_mhz * 1e6
+    io = (n + sb + m) / 8
+    t_alu, t_hbm = ops / rate * 1e3, io / (peak_hbm * 1e9) * 1e3
+    return {"definition": "max(bits in and out at the measured HBM bandwidth, ALU-pipe instructions of the "
+                          "transforms' products at 64 lanes an SM) / measured step",
+            "frac": max(t_alu, t_hbm) / ms_per_step, "t_alu_ms": t_alu, "t_hbm_ms": t_hbm, "alu_ops": ops,
+            "transform_lg": shape[0], "a_blocks": shape[1], "b_blocks": shape[2], "windows": shape[3]}
+
+
 def roofline_of(prof, products, m, peak, peak_src, workload):
     """The dominant kernel's roofline: algorithmic bytes per launch (the scope's
     48 L model, with the path's own element size beside it) over its average
@@ -1595,6 +1636,20 @@ def run_single(args, world, rank, local, dist):
     roof, kernels = roofline_of(prof, products, m, peak, peak_src, args.workload)
     rates = {f: native.modmul_rate(local, f) for f in (native.FIELD_GOLDILOCKS, native.FIELD_Q30, native.FIELD_Q25)}
     path_roof = path_roofline_of(products, n, sb, m, ms_per_step, peak, rates)
+    binary = any(k.startswith("k_gf") for k in prof)
+    if binary:  # the call ran as binary polynomials or densely: other kernels, other model
+        launches = round(sum(c for c, _ in prof.values()) / args.steps)
+        dom = max(prof, key=lambda k: prof[k][1])
+        path_roof = None
+        roof = {"bound": "latency", "kernel": dom, "avg_launch_ms": prof[dom][1] / prof[dom][0]}
+        if "k_gf_rows" in prof or "k_gf_units" in prof:
+            mhz = (sampler.summary(t_wall0, t_wall1) or {}).get("sm_mhz") or 2070.0
+            path_roof = binary_roofline(kind, n, sb, m, ms_per_step, mhz, peak)
+            rate = 152 * 64 * mhz * 1e6
+            roof = {"bound": "alu", "kernel": dom, "achieved": path_roof["alu_ops"] / (ms_per_step * 1e-3) / 1e12,
+                    "peak": rate / 1e12, "unit": "T ALU instructions/s (lanes), whole step", "frac": path_roof["frac"],
+                    "peak_source": "152 SMs x 64 ALU lanes x measured SM clock", "traffic": ncu_traffic(dom, args.workload),
+                    "avg_launch_ms": prof[dom][1] / prof[dom][0]}
 
     # the Dodis et al. workload as its configuration states it: one Goldilocks
     # transform of length 2^31 (single-transform plan); same bits
@@ -1669,9 +1724,11 @@ def run_single(args, world, rank, local, dist):
         "metric": "extracted output Gbit/s", "value": value, "unit": "Gbit/s",
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "u64" if pf == FIELD_GL else "u32", "data": "synthetic",
+        "vs_baseline": None, "dtype": "u32 (bit-sliced GF(2))" if binary else "u64" if pf == FIELD_GL else "u32",
+        "data": "synthetic",
         "config": {"workload": wl["name"], "n": n, "m": m, "seed_bits": sb,
-                   "plan": {"products": plan["products"], "windows": plan["windows"],
+                   "form": "binary polynomials / dense over GF(2)" if binary else "integer transforms",
+                   "integer_plan" if binary else "plan": {"products": plan["products"], "windows": plan["windows"],
                             "transform_length": L, "field": FIELD_NAMES.get(pf, pf),
                             "tail_terms": plan["tail_terms"], "planner_estimate_ms": plan["est_ms"]},
                    "l2": "flushed between timed steps (256 MiB write)",
@@ -1696,8 +1753,7 @@ def dodis_extra(local, steps=5):
     from paper_2402_09481_gb300 import inputs, native
     n, m = 1073741789, 429496715
     ctx = native.Context(local)
-    plan = native.plan_query(2, n, m)
-    products = native.plan_products(2, n, m)
+    shape = binary_shape(2, n, m)
     nw = native.words(n)
     xu = torch.from_numpy(inputs.bernoulli_half(31, n).view(np.int64)).cuda()
     yd = torch.from_numpy(inputs.bernoulli_half(32, n).view(np.int64)).cuda()
@@ -1710,10 +1766,9 @@ def dodis_extra(local, steps=5):
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device="cuda")
     stream = torch.cuda.current_stream()
     peak, _ = measured_peaks()
-    rates = {f: native.modmul_rate(local, f) for f in (native.FIELD_GOLDILOCKS, native.FIELD_Q30, native.FIELD_Q25)}
     out = {"workload": "Dodis et al.: n = 1073741789 (largest N_A prime <= 2^30), m = floor(0.4 n)",
-           "plan": {"products": plan["products"], "transform_length": plan["transform_length"],
-                    "field": FIELD_NAMES.get(plan["field"], plan["field"])}}
+           "plan": {"form": "binary polynomials", "transform_length": 1 << shape[0], "a_blocks": shape[1],
+                    "b_blocks": shape[2], "windows": shape[3]}}
     for name, xd in (("bernoulli_half", xu), ("x_0p8_biased", xb)):
         for _ in range(2):
             ctx.dodis(xd, yd, n, m, zd)
@@ -1729,9 +1784,9 @@ def dodis_extra(local, steps=5):
         st, fl = ctx.device_status()
         assert st == native.CM_OK, native.STATUS.get(st)
         ms_ = statistics.median(ts)
-        pr = path_roofline_of(products, n, n, m, ms_, peak, rates)
+        pr = binary_roofline(2, n, n, m, ms_, 2070.0, peak)
         out[name] = {"ms_per_step": ms_, "value": m / (ms_ * 1e-3) / 1e9, "unit": "Gbit/s",
-                     "path_roofline_frac": pr["frac"], "frac_actual_element_bytes": pr["actual_element_bytes"]["frac"]}
+                     "path_roofline_frac": pr["frac"], "t_alu_ms": pr["t_alu_ms"], "t_hbm_ms": pr["t_hbm_ms"]}
     ctx.close()
     del xu, xb, yd, zd, flush
     torch.cuda.empty_cache()

@@ -44,11 +44,44 @@ struct CRows {
     }
 };
 
+// Three-input forms the compiler does not always find.
+CM_HD uint32_t xor3(uint32_t a, uint32_t b, uint32_t c) {
+#ifdef __CUDA_ARCH__
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0x96;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
+#else
+    return a ^ b ^ c;
+#endif
+}
+CM_HD uint32_t and_xor(uint32_t a, uint32_t b, uint32_t c) {  // (a & b) ^ c
+#ifdef __CUDA_ARCH__
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
+#else
+    return (a & b) ^ c;
+#endif
+}
+CM_HD uint32_t xor_and(uint32_t a, uint32_t b, uint32_t c) {  // (a ^ b) & c
+#ifdef __CUDA_ARCH__
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0x28;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
+#else
+    return (a ^ b) & c;
+#endif
+}
+
 // o = a b on 2^LW words each.
 template <int LW>
 CM_HD void mul(const uint32_t *a, const uint32_t *b, uint32_t *o) {
     if constexpr (LW == 0) {
         o[0] = a[0] & b[0];
+    } else if constexpr (LW == 1) {  // x_0^2 = x_0 + 1: five operations
+        const uint32_t p0 = a[0] & b[0], s = b[0] ^ b[1];
+        o[0] = and_xor(a[1], b[1], p0);
+        o[1] = xor_and(a[0], a[1], s) ^ p0;
     } else {
         constexpr int H = 1 << (LW - 1);
         constexpr CRows<LW - 1> C{};
@@ -64,11 +97,16 @@ CM_HD void mul(const uint32_t *a, const uint32_t *b, uint32_t *o) {
 #pragma unroll
         for (int i = 0; i < H; ++i) {
             o[H + i] = p1[i] ^ p0[i];
-            uint32_t v = p0[i];
+            uint32_t v = p0[i], w = 0;
+            bool half = false;  // w holds a term waiting for a second
 #pragma unroll
             for (int j = 0; j < H; ++j)
-                if ((C.r[i] >> j) & 1u) v ^= p2[j];
-            o[i] = v;
+                if ((C.r[i] >> j) & 1u) {
+                    if (half) v = xor3(v, w, p2[j]);
+                    w = p2[j];
+                    half = !half;
+                }
+            o[i] = half ? v ^ w : v;
         }
     }
 }

@@ -81,7 +81,7 @@ typedef struct {
      * 5 * 2^25 + 1; CM_FIELD_GOLDILOCKS takes Goldilocks throughout.  Results
      * are identical.  Under CM_FIELD_AUTO, with max_transform_lg,
      * max_sum_blocks and plan_mode at their defaults too, single calls with
-     * K + m - 1 > 2^23 and batch instances with K + m - 1 > 2^14 run as binary
+     * K + m - 1 > 2^23 (above 2^22: where the planner has one transform) and batch instances with K + m - 1 > 2^14 run as binary
      * polynomials (when that form's scratch fits the budget).  The work list of
      * batches and the server runs over 5 * 2^25 + 1. */
     uint32_t field;
@@ -400,8 +400,11 @@ typedef struct {
  * that does not fit yet is passed over by at most 16 waves, after which
  * nothing behind it starts until it fits).  A wave runs its requests with
  * transforms up to 2^21 as one work-list kernel (the cm_batch_create
- * machinery) and longer ones through the single-call planner, on the slot's
- * stream; a wave of one request runs the single-call kernels.  Waves on
+ * machinery) and longer ones through the integer single-call planner, on the
+ * slot's stream; with the context's options at their defaults (see
+ * cm_options.field) those of 2^18 .. 2^25, where one length has 2^22 elements or
+ * more, run as binary polynomials instead, one group of launches a length.  A
+ * wave of one request up to 2^25 runs what its single call runs.  Waves on
  * different streams overlap on the device; each stream has two slots, so the
  * next wave is enqueued behind the running one.  Express slots (high stream
  * priority) take only requests up to 2^21, so that short requests are not

@@ -715,11 +715,12 @@ void gf_shape(int kind, uint64_t n, uint64_t m, gf::Product *p, gf::Ops *q) {
 
 // Products longer than 2^23 take the binary form in a context with default
 // options (a context that names a field, a transform limit, a sum cap or single
-// transforms keeps the integer ones).  Measured, us a call, binary / integer:
-// 2^23 206 / 153, 2^24 216 / 307, 2^25 245 / 722, 2^26 517 / 2565, 2^28
-// 1812 / 10659: below 2^24 too few tiles to fill the GPU.
+// transforms keeps the integer ones), and those above 2^22 that the integer
+// planner would run as one transform of 2^23.  Measured, us a call, binary /
+// integer: 2^22 140 / 92, 2^23 148 / 153, 2^24 158 / 306, 2^25 198 / 719, 2^26
+// 414 / 2561, 2^28 1431 / 10650: below, too few tiles to fill the GPU.
 // Products of up to 2^13 terms run densely in one launch (cm_gf2_dense.cu).
-constexpr int kGfMinLg = 24;
+constexpr int kGfMinLg = 23;
 // Products of 2^17 .. 2^22 terms run densely on the tensor cores (cm_gf2_tc.cu)
 // while their longest chain of stages beats the transforms.  Measured, us a call,
 // integer transforms / dense (K x m: stages): 100000 x 50000: 3, 43 / 25; 300007 x
@@ -731,6 +732,13 @@ constexpr uint64_t kTcMaxStages = 40;
 bool gf_allowed(const cm_ctx *ctx) {
     const PlanOptions &o = ctx->popt;
     return o.fields == kFieldsAll && o.max_lg == 32 && !o.max_sum && !o.single;
+}
+
+// Whether the integer planner would run the product as one transform of 2^kGfMinLg.
+static bool one_transform(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t terms) {
+    std::vector<Block> bl;
+    return terms > 1ull << (kGfMinLg - 1) && make_blocks(kind, n, m, ctx->popt, &bl) && bl.size() == 1 &&
+           bl[0].p.lg == kGfMinLg;
 }
 
 cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t budget, Route *r) {
@@ -752,7 +760,8 @@ cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64
         }
     }
     if (gf_allowed(ctx) && n - 1 < kMaxBits && m - 1 < kMaxBits &&
-        (terms <= 1ull << gf::kDenseMaxLg || terms > 1ull << (kGfMinLg - 1)) && valid_args(kind, n, m)) {
+        (terms <= 1ull << gf::kDenseMaxLg || terms > 1ull << kGfMinLg || one_transform(ctx, kind, n, m, terms)) &&
+        valid_args(kind, n, m)) {
         if (terms <= 1ull << gf::kDenseMaxLg) {
             gf_maps(kind, n, m, &r->ops);
             r->dense = true;

@@ -35,7 +35,11 @@
 //   k_gf_units  conversion of each row down to units of 256 bits
 //   k_gf_cols   (k > 18) levels k-1 .. lo on tiles of 2^13 words, both operands
 //   k_gf_mid    256-bit conversions, levels lo-1 .. 0, product, and back
-// and the inverses of the first three on the product.  Levels are bit-sliced
+// and the inverses of the first three on the product.  One product of 2^25 bits,
+// us: rows 35.5 (inverse 20.7), units 18.5 (12), cols 23.5 (18.5), mid 84.5; the
+// call 198, two summed integer products of 2^24 before it 545.  Past 2^25 bits
+// k_gf_fwd and k_gf_sum / k_gf_sum2 stand in for k_gf_mid (2^28: 449 and 282 us
+// of 1431; integer transforms 10650).  Levels are bit-sliced
 // (gf2.cuh): a thread holds whole elements, one component a register, 32 of
 // them a word.
 #include <cuda_runtime.h>
@@ -781,7 +785,10 @@ __device__ __forceinline__ void load_pass(Pass *P, const Pass *__restrict__ g) {
 }
 
 // Levels lg - 1 .. lo: fields up to GF(2^16), twiddles that depend on the tile's
-// own bits only.  In place; grid: tiles of every array.
+// own bits only.  In place; grid: tiles of every array.  Two operands of 2^25: 23.5
+// us, most of it the loads' and stores' latency (four levels are left to it: the
+// first four, on single bits to GF(16), are constants and run with the row
+// conversion).
 constexpr int kColsThreads = 256;
 
 template <bool INV>
@@ -899,7 +906,10 @@ __device__ void inverse_levels(uint32_t *sm, const Pass &P, const uint32_t *base
 // transform in place of b's tile.  The ALU pipe bounds it; a thread holds one
 // unit of 2 x 32 words.  PAR: half the threads on each operand, for few tiles
 // (a tile's own time counts); else one operand after the other on half as many
-// threads, so that three CTAs of an SM fill each other's gaps.
+// threads, so that three CTAs of an SM fill each other's gaps.  2^25: 84.5 us (91
+// before a unit's loads came before its stores), half of the ALU rate: 128 tiles
+// have two warps a scheduler, the inverse one.  Both operands' units in one
+// thread, sharing the twiddle sums, took 120 for 91 (255 registers).
 template <int NB, int FMAX, bool PAR>
 __global__ void __launch_bounds__((PAR ? 2 : 1) * MidShape<NB, FMAX>::HALF, PAR ? 1 : 384 / MidShape<NB, FMAX>::HALF)
 k_gf_mid(int lg, const Pass *__restrict__ table,
@@ -954,7 +964,8 @@ k_gf_mid(int lg, const Pass *__restrict__ table,
     store_tile<NB>(sb, P, B + off, threadIdx.x, NT);
 }
 
-// Several blocks: the forward half alone, tile words to H in tile order ...
+// Several blocks: the forward half alone, tile words to H in tile order (449 us in
+// the 2^28 product; ALU pipe) ...
 __global__ void __launch_bounds__(128) k_gf_fwd(int lg, uint32_t na, const Pass *__restrict__ table,
                                                 const uint32_t *__restrict__ data, uint32_t *__restrict__ hat) {
     __shared__ __align__(16) uint32_t sm[8192];
@@ -1026,7 +1037,9 @@ __global__ void __launch_bounds__(256) k_gf_sum(int lg, uint32_t na, uint32_t ni
 // i + w ..) give w and w + 1 with three products for four,
 //   a_0 B_0 + a_1 B_1 = a_0 (B_0 + B_1) + (a_0 + a_1) B_1,
 //   a_0 B_1 + a_1 B_2 = a_1 (B_1 + B_2) + (a_0 + a_1) B_1,
-// and both inverses run together, one on each half of the threads.
+// and both inverses run together, one on each half of the threads.  ALU pipe; the
+// two-source extraction of 2^30 bits (64 + 89 blocks) 10.2 -> 9.2 ms against
+// k_gf_sum for each window.
 __global__ void __launch_bounds__(256) k_gf_sum2(int lg, uint32_t na, uint32_t nb, uint32_t nin, uint32_t nz,
                                                  const Pass *__restrict__ table, const uint32_t *__restrict__ hat,
                                                  uint32_t *__restrict__ out) {
@@ -1209,7 +1222,12 @@ void build_tables(Pass *t) {
     for (int lg = kMinLg; lg <= kMaxLg; ++lg) {
         Pass *p = t + 2 * (lg - kMinLg);
         memset(p, 0, 2 * sizeof(Pass));
-        build_passes(lg, p, p + 1);
+        build_passes(lg, false, p, p + 1);
+    }
+    for (int lg = kFewMinLg; lg <= kFewMaxLg; ++lg) {
+        Pass *p = t + kFewTables + 2 * (lg - kFewMinLg);
+        memset(p, 0, 2 * sizeof(Pass));
+        build_passes(lg, true, p, p + 1);
     }
 }
 
@@ -1244,9 +1262,16 @@ cudaError_t launch_tc_prep(const Ops &q, const TcShape &s, uint32_t *a, uint32_t
 
 cudaError_t launch_product(cm_ctx *c, int nsm, const Product &p, const Ops &q, const Pass *tables, void *scratch,
                            cudaStream_t st) {
-    const Shape s = shape_of(p.lg);
-    const Pass *mid = tables + 2 * (p.lg - kMinLg), *col = mid + 1;
     const bool sum = summed(p, q);
+    // Few operands: last-pass tiles of 2^12 words, one level more in the column
+    // passes, while one SM each holds them all: such a tile's pass is a chain of
+    // levels with one warp a scheduler, half as long in its forward half on half
+    // the words (one product of 2^24, us: k_gf_mid 84.0 -> 68.1, the column passes
+    // 31.9 -> 36.2, the call 167 -> 158).  Not for more: 4096 mixed instances,
+    // k_gf_mid 7.06 ms, 9.11 with these tiles.
+    const bool few = !sum && p.lg >= kFewMinLg && p.lg <= kFewMaxLg && (uint64_t)q.na << (p.lg - 17) <= (uint64_t)nsm;
+    const Shape s = shape_of(p.lg, few);
+    const Pass *mid = tables + (few ? kFewTables + 2 * (p.lg - kFewMinLg) : 2 * (p.lg - kMinLg)), *col = mid + 1;
     const uint32_t ops = q.na + q.nb;
     uint32_t *data = static_cast<uint32_t *>(scratch);
     uint32_t *B = data + ((uint64_t)q.na << (p.lg - 5));

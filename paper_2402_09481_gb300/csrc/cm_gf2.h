@@ -115,7 +115,8 @@ cudaError_t launch_tc(const TcShape &s, const uint32_t *a, const uint32_t *b, ui
                       const uint32_t *pre, uint32_t *status, bool dependent, cudaStream_t st);
 
 // Host image of the device tables.
-constexpr int kTables = 2 * (kMaxLg - kMinLg + 1);
+constexpr int kFewTables = 2 * (kMaxLg - kMinLg + 1);  // where the few-operand shapes' begin
+constexpr int kTables = kFewTables + 2 * (kFewMaxLg - kFewMinLg + 1);
 void build_tables(Pass *t);  // kTables entries
 
 }  // namespace gf

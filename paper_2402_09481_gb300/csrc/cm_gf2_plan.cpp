@@ -40,15 +40,15 @@ void cantor_basis(uint32_t beta[32]) {
     }
 }
 
-Shape shape_of(int lg) {
+Shape shape_of(int lg, bool few) {
     Shape s;
     s.lg = lg;
     s.fmax = lg < 16 ? 4 : 5;
     s.two = lg > 18;
-    s.nb = lg >= 18 ? 13 : lg - 5;
+    s.nb = few ? 12 : lg >= 18 ? 13 : lg - 5;
     s.nfree = s.nb - s.fmax;
     // components whose index bit is at least lo come with the tile from above it
-    s.lo = !s.two ? lg : (lg <= 21 ? 15 : 14);
+    s.lo = !s.two ? lg : few ? 13 : lg <= 21 ? 15 : 14;
     s.tiles = 1 << (lg - 5 - s.nb);
     s.colr = lg > 16 ? lg - 16 : 0;
     return s;
@@ -167,8 +167,8 @@ static void build_pass(int lg, int nb, int nfree, int fmax, const std::vector<in
     if (lo > 4) P->npre = P->nlev;
 }
 
-void build_passes(int lg, Pass *mid, Pass *col) {
-    const Shape s = shape_of(lg);
+void build_passes(int lg, bool few, Pass *mid, Pass *col) {
+    const Shape s = shape_of(lg, few);
     uint32_t beta[32];
     cantor_basis(beta);
     std::vector<int> in;

@@ -18,10 +18,11 @@ struct Shape {
     int tiles;      // tiles of the last pass (and of the column pass)
     int colr;       // index bits above 16 (rows of the first conversion), 0 if lg <= 16
 };
-Shape shape_of(int lg);
+// few: the smaller tiles for few operands (lg of kFewMinLg .. kFewMaxLg).
+Shape shape_of(int lg, bool few = false);
 
 // Fill the pass tables: mid always, col when two.
-void build_passes(int lg, Pass *mid, Pass *col);
+void build_passes(int lg, bool few, Pass *mid, Pass *col);
 
 }  // namespace gf
 }  // namespace cm

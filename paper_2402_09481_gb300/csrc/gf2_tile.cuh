@@ -12,6 +12,8 @@ enum ConvKind : int { kConvA = 0, kConvB = 1, kConvBInv = 2 };
 
 constexpr int kMinLg = 15;  // shortest and longest transform, log2 bits
 constexpr int kMaxLg = 25;
+// lengths with a second shape, last-pass tiles of 2^12 words, for few operands
+constexpr int kFewMinLg = 22, kFewMaxLg = 24;
 constexpr int kMaxLev = 18;  // levels of one pass
 
 // One level of a pass over tiles.  A tile word address has NB bits: NFREE

@@ -217,3 +217,37 @@ def test_tensor_core_form_largest_counts(cm_ctx):
         y = torch.full((native.words(n + m - 1),), -1, dtype=torch.int64, device="cuda")
         z = from_dev(run(cm_ctx, T, n, m, x, y))
         assert int(sum(bin(int(w)).count("1") for w in z)) == (m if n & 1 else 0)
+
+
+@pytest.mark.parametrize("kind,n,m", [(T, 2 ** 23 - 4_000_000, 4_000_001), (T, 4_900_007, 3_100_003),
+                                      (C, 6_000_000, 2_000_003), (D, 4_194_389, 2_000_003), (T, 5_000_000, 64)])
+def test_one_transform_of_2_23(cm_ctx, q30, kind, n, m):
+    # above 2^22: either form, the same bits; the first is a single transform of 2^23
+    n, m = resolve(kind, n, m)
+    xw = inputs.bernoulli_half(41 + n % 83, n)
+    if kind == D:
+        xw[0] = (xw[0] | np.uint64(1)) & ~np.uint64(2)
+    x, y = to_dev(xw), to_dev(inputs.bernoulli_half(42 + m % 79, ybits(kind, n, m)))
+    cm_ctx.profile_enable(True)
+    cm_ctx.profile_read(reset=True)
+    z = run(cm_ctx, kind, n, m, x, y)
+    prof = cm_ctx.profile_read(reset=True)
+    cm_ctx.profile_enable(False)
+    if m == 4_000_001:
+        assert any(k.startswith("k_gf_mid") for k in prof), prof
+    assert torch.equal(z, run(q30, kind, n, m, x, y))
+
+
+@pytest.mark.parametrize("lg,count", [(22, 1), (22, 4), (22, 5), (23, 2), (23, 3), (24, 1), (24, 2)])
+def test_batch_few_operands(cm_ctx, q30, lg, count):
+    # both tile shapes of the last pass, on each side of the line between them
+    items, want = [], []
+    for j in range(count):
+        m = 2 ** (lg - 2) + 3 * j + 1
+        n = 2 ** lg - m + 1 - j
+        x, y = to_dev(inputs.bernoulli_half(700 + j, n)), to_dev(inputs.bernoulli_half(800 + j, n + m - 1))
+        items.append((T, n, m, x, y, torch.full((native.words(m),), -1, dtype=torch.int64, device="cuda")))
+        want.append(run(q30, T, n, m, x, y))
+    cm_ctx.batch_extract(items)
+    for it, z in zip(items, want):
+        assert torch.equal(it[5], z)

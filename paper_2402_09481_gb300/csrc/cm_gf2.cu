@@ -786,9 +786,8 @@ __device__ __forceinline__ void load_pass(Pass *P, const Pass *__restrict__ g) {
 
 // Levels lg - 1 .. lo: fields up to GF(2^16), twiddles that depend on the tile's
 // own bits only.  In place; grid: tiles of every array.  Two operands of 2^25: 23.5
-// us, most of it the loads' and stores' latency (four levels are left to it: the
-// first four, on single bits to GF(16), are constants and run with the row
-// conversion).
+// us, most of it the loads' and stores' latency (seven levels; the first four, on
+// single bits to GF(16), have constant twiddles and run with the row conversion).
 constexpr int kColsThreads = 256;
 
 template <bool INV>
@@ -907,8 +906,9 @@ __device__ void inverse_levels(uint32_t *sm, const Pass &P, const uint32_t *base
 // unit of 2 x 32 words.  PAR: half the threads on each operand, for few tiles
 // (a tile's own time counts); else one operand after the other on half as many
 // threads, so that three CTAs of an SM fill each other's gaps.  2^25: 84.5 us (91
-// before a unit's loads came before its stores), half of the ALU rate: 128 tiles
-// have two warps a scheduler, the inverse one.  Both operands' units in one
+// before a unit's loads came before its stores), 46% of the ALU rate: 128 tiles
+// have two warps a scheduler, the inverse one, and the first stall is instruction
+// fetch (a product of GF(2^32) elements is about a thousand instructions in line).  Both operands' units in one
 // thread, sharing the twiddle sums, took 120 for 91 (255 registers).
 template <int NB, int FMAX, bool PAR>
 __global__ void __launch_bounds__((PAR ? 2 : 1) * MidShape<NB, FMAX>::HALF, PAR ? 1 : 384 / MidShape<NB, FMAX>::HALF)

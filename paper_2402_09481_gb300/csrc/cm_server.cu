@@ -8,8 +8,11 @@
 // the HBM budget still unclaimed by requests on the device; a request that
 // does not fit yet is passed over by at most a fixed number of waves, after
 // which nothing behind it starts until it fits.  A wave runs as one work-list
-// kernel on the slot's stream (requests with transforms longer than 2^21
-// follow on the same stream through the single-call kernels).  Waves on
+// kernel on the slot's stream; its requests with transforms of 2^18 .. 2^25 run
+// as binary polynomials, those of one length together in each launch, where a
+// length has 2^22 elements or more (48 requests up to 2^23 bits: 2.50 -> 1.43
+// ms); a lone request runs as its single call would, and requests with
+// transforms longer than 2^25 follow through the integer single-call kernels.  Waves on
 // different slots run concurrently, so requests that arrive while others are
 // on the GPU start as soon as a slot and memory free up.  Admission holds the
 // server lock; planning, upload and launch run outside it, so submissions

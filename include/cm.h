@@ -81,8 +81,9 @@ typedef struct {
      * 5 * 2^25 + 1; CM_FIELD_GOLDILOCKS takes Goldilocks throughout.  Results
      * are identical.  Under CM_FIELD_AUTO, with max_transform_lg,
      * max_sum_blocks and plan_mode at their defaults too, single calls with
-     * K + m - 1 > 2^23 (above 2^22: where the planner has one transform) and batch instances with K + m - 1 > 2^14 run as binary
-     * polynomials (when that form's scratch fits the budget).  The work list of
+     * K + m - 1 > 2^23 (above 2^22: where the planner has one transform) and batch
+     * instances with K + m - 1 > 2^14, where a length has enough of them, run as
+     * binary polynomials (when that form's scratch fits the budget).  The work list of
      * batches and the server runs over 5 * 2^25 + 1. */
     uint32_t field;
     /* Most input blocks whose transform-domain products are summed before one

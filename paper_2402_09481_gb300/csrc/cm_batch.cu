@@ -556,6 +556,13 @@ static double time_once(cm_batch *b, cudaStream_t st) {
     return ms;
 }
 
+// Elements (instances x length) from which a length's instances run as binary
+// polynomials.  A group is a chain of 3 (to 2^16), 5 (to 2^18) or 7 launches, about
+// 45, 75 and 145 us however few it holds; the work list takes 25 ps an element
+// (4.4e9 in 109 ms).  43 instances of 2^11 .. 2^18 bits: 248 us on the work list, 566
+// as five groups; 245 of 2^12 .. 2^15: 256, 224.
+static uint64_t group_min(int lg) { return lg <= 16 ? 1ull << 21 : lg <= 18 ? 1ull << 22 : 1ull << 23; }
+
 extern "C" cm_status cm_batch_create(cm_ctx *ctx, const cm_desc *descs, uint32_t count, uint32_t flags,
                                      cm_batch **out) {
     if (!ctx || !out || (count && !descs)) return CM_EINVAL;
@@ -569,10 +576,11 @@ extern "C" cm_status cm_batch_create(cm_ctx *ctx, const cm_desc *descs, uint32_t
     b->plans.resize(count);
     b->off_scratch.assign(count, 0);
     // Transforms of 2^15 .. 2^25 run as binary polynomials, every length's
-    // instances together, unless the context's options ask for the integer ones
-    // (the bounded waits that CM_BATCH_TEST_STALL runs out are the work list's).
+    // instances together where they are enough, unless the context's options ask
+    // for the integer ones (the bounded waits that CM_BATCH_TEST_STALL runs out are the work list's).
     const bool use_gf = gf_allowed(ctx) && !b->test_stall;
     std::vector<uint32_t> by_lg[gf::kMaxLg + 1];
+    uint64_t elems[gf::kMaxLg + 1] = {};
     size_t total = 0;
     for (uint32_t i = 0; i < count; ++i) {
         const cm_desc &d = descs[i];
@@ -580,9 +588,14 @@ extern "C" cm_status cm_batch_create(cm_ctx *ctx, const cm_desc *descs, uint32_t
             delete b;
             return CM_EINVAL;
         }
+        if (b->plans[i].lg <= gf::kMaxLg) elems[b->plans[i].lg] += b->plans[i].L;
+    }
+    for (uint32_t i = 0; i < count; ++i) {
+        const cm_desc &d = descs[i];
         b->off_scratch[i] = total;
         if (!on_worklist(b->plans[i])) ++b->long_instances;
-        if (use_gf && b->plans[i].lg >= gf::kMinLg && b->plans[i].lg <= gf::kMaxLg) {
+        if (use_gf && b->plans[i].lg >= gf::kMinLg && b->plans[i].lg <= gf::kMaxLg &&
+            elems[b->plans[i].lg] >= group_min(b->plans[i].lg)) {
             by_lg[b->plans[i].lg].push_back(i);
         } else if (on_worklist(b->plans[i])) {
             b->wl.push_back(i);
@@ -591,7 +604,7 @@ extern "C" cm_status cm_batch_create(cm_ctx *ctx, const cm_desc *descs, uint32_t
             // the single-call kernels, over the context's field set
             make_plan(d.kind, d.n, d.m, &b->plans[i], ctx->popt.fields, ctx->popt.tune);
             b->solo.push_back(i);
-            if (use_gf) {  // past 2^25
+            if (use_gf) {  // past 2^25, or a lone one of 2^22
                 Route r;
                 const cm_status rs = make_route(ctx, d.kind, d.n, d.m, ctx->budget, &r);
                 if (rs != CM_OK) {

@@ -251,3 +251,24 @@ def test_batch_few_operands(cm_ctx, q30, lg, count):
     cm_ctx.batch_extract(items)
     for it, z in zip(items, want):
         assert torch.equal(it[5], z)
+
+
+@pytest.mark.parametrize("lg,count", [(15, 63), (15, 64), (16, 32), (17, 31), (17, 32), (18, 16), (19, 15), (19, 16)])
+def test_batch_group_line(cm_ctx, q30, lg, count):
+    # the fewest instances of a length that run as a group, and one less
+    items, want = [], []
+    for j in range(count):
+        m = 2 ** (lg - 1) + 3 * j - 40
+        n = 2 ** lg - m + 1 - j
+        x, y = to_dev(inputs.bernoulli_half(900 + j, n)), to_dev(inputs.bernoulli_half(980 + j, n + m - 1))
+        items.append((T, n, m, x, y, torch.full((native.words(m),), -1, dtype=torch.int64, device="cuda")))
+        want.append(run(q30, T, n, m, x, y))
+    cm_ctx.profile_enable(True)
+    cm_ctx.profile_read(reset=True)
+    cm_ctx.batch_extract(items)
+    prof = cm_ctx.profile_read(reset=True)
+    cm_ctx.profile_enable(False)
+    line = 21 if lg <= 16 else 22 if lg <= 18 else 23
+    assert ("k_batch" in prof) == (count << lg < 1 << line), prof
+    for it, z in zip(items, want):
+        assert torch.equal(it[5], z)

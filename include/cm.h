@@ -204,10 +204,18 @@ cm_status cm_device_status(cm_ctx *ctx, cm_stream stream, uint32_t *flags);
  * gives full copy bandwidth; pageable works).  Word counts: x ceil(n/64);
  * y ceil((n+m-1)/64) for Toeplitz, ceil((n+1)/64) for Circulant, ceil(n/64)
  * for Dodis et al.; z ceil(m/64).  Device copies come from the context pool.
- * Returns CM_EPRECOND (z zero-filled) for a constant Dodis et al. x.
+ * Returns CM_EPRECOND (z zero-filled) for a constant Dodis et al. x and
+ * CM_ETIMEDOUT (z undefined) if a bounded device wait ran out.
  */
 cm_status cm_extract_host(cm_ctx *ctx, int kind, const uint64_t *x_host, uint64_t n,
                           const uint64_t *y_host, uint64_t m, uint64_t *z_host, cm_stream stream);
+
+/* Failure-path test: while on, calls that run densely on the tensor cores (see
+ * cm_options.field) leave out the signal their last bounded wait is for.  It runs
+ * out after 2 s: the outputs are undefined and CM_FLAG_TIMEOUT is reported, by
+ * cm_device_status for device-pointer calls, as CM_ETIMEDOUT by cm_extract_host
+ * and in a served request's result.  CM_EINVAL if ctx is NULL. */
+cm_status cm_test_stall(cm_ctx *ctx, int on);
 
 /*
  * Allocation-free Toeplitz extraction (the paper has no counterpart; this is a

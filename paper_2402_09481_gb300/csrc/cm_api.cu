@@ -780,7 +780,7 @@ cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64
 }
 
 cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t *y, uint64_t *z, void *scratch,
-                               cudaStream_t st) {
+                        cudaStream_t st, uint32_t *gave_up) {
     uint8_t *sc = static_cast<uint8_t *>(scratch);
     if (r.dense) {
         r.ops.a0.map.src = x;
@@ -806,6 +806,7 @@ cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t
         }
         ProfScope ps(ctx, "k_gf_tc", st);
         return cuda_status(gf::launch_tc(r.shape, a, b, z, r.m, pre, ctx->d_status,
+                                         gave_up ? gave_up : ctx->d_status, ctx->test_stall,
                                          gf::may_depend(st) && !ctx->prof_on, st));
     }
     if (!r.gf) return enqueue_blocks(ctx, r.bl, x, y, z, sc, r.tmp_off, r.pre_off, st);
@@ -1315,15 +1316,25 @@ extern "C" cm_status cm_extract_host(cm_ctx *ctx, int kind, const uint64_t *xh, 
     if (cudaMemcpyAsync(xd, xh, 8 * xw, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(yd, yh, 8 * yw, cudaMemcpyHostToDevice, st) != cudaSuccess)
         s = CM_EDEVICE;
-    uint32_t pre_h[2] = {1, 1};
-    if (s == CM_OK) s = enqueue_route(ctx, r, xd, yd, zd, b, st);
+    // the Dodis et al. flags and, behind them, the tensor-core form's timeout word
+    uint32_t flags_h[3] = {1, 1, 0};
+    uint32_t *flags_d = reinterpret_cast<uint32_t *>(b + r.pre_off);
+    if (s == CM_OK && r.tc && cudaMemsetAsync(flags_d, 0, sizeof(flags_h), st) != cudaSuccess) s = CM_EDEVICE;
+    if (s == CM_OK) s = enqueue_route(ctx, r, xd, yd, zd, b, st, r.tc ? flags_d + 2 : nullptr);
     if (s == CM_OK && cudaMemcpyAsync(zh, zd, 8 * zw, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         s = CM_EDEVICE;
-    if (s == CM_OK && kind == CM_DODIS &&
-        cudaMemcpyAsync(pre_h, b + r.pre_off, sizeof(pre_h), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+    if (s == CM_OK && (kind == CM_DODIS || r.tc) &&
+        cudaMemcpyAsync(flags_h, flags_d, (r.tc ? 3 : 2) * sizeof(uint32_t), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         s = CM_EDEVICE;
     cudaFreeAsync(buf, st);
     if (cudaStreamSynchronize(st) != cudaSuccess) return CM_EDEVICE;
-    if (s == CM_OK && kind == CM_DODIS && (pre_h[0] == 0 || pre_h[1] == 0)) s = CM_EPRECOND;
+    if (s == CM_OK && kind == CM_DODIS && (flags_h[0] == 0 || flags_h[1] == 0)) s = CM_EPRECOND;
+    if (s == CM_OK && (flags_h[2] & CM_FLAG_TIMEOUT)) s = CM_ETIMEDOUT;
     return s;
+}
+
+extern "C" cm_status cm_test_stall(cm_ctx *ctx, int on) {
+    if (!ctx) return CM_EINVAL;
+    ctx->test_stall = on != 0;
+    return CM_OK;
 }

@@ -32,6 +32,7 @@ struct cm_ctx {
     cm::RootTables25 rt25{};
     cm::gf::Pass *d_gf = nullptr;  // level tables of the binary-polynomial transforms
     cm_server *server = nullptr;
+    std::atomic<bool> test_stall{false};  // cm_test_stall
     // one-launch cluster kernel per length 2^14 .. 2^17: -1 not yet checked, 0 no, 1 yes
     std::atomic<int> cluster25[4] = {-1, -1, -1, -1};
 

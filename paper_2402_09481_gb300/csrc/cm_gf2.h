@@ -105,6 +105,8 @@ cudaError_t launch_dense(const BitMap &a, const BitMap &b, uint32_t K, uint32_t 
 // Dense product on the tensor cores (cm_gf2_tc.cu): the shape of K terms and m
 // outputs (stages: the longest CTA chain's, the time's measure), the operands as
 // plain bits (a after 256 zero bits; b in order) with z cleared, the product.
+// status: the Dodis et al. flag; gave_up: CM_FLAG_TIMEOUT when a bounded wait ran
+// out (z is then undefined); stall: make one run out.
 struct TcShape {
     uint64_t rows, chunks, splits, per, a_words, b_words, stages;
 };
@@ -112,7 +114,8 @@ TcShape tc_shape(uint64_t K, uint64_t m, int nsm);
 cudaError_t launch_tc_prep(const Ops &q, const TcShape &s, uint32_t *a, uint32_t *b, uint64_t *z, uint64_t m,
                            cudaStream_t st);
 cudaError_t launch_tc(const TcShape &s, const uint32_t *a, const uint32_t *b, uint64_t *z, uint64_t m,
-                      const uint32_t *pre, uint32_t *status, bool dependent, cudaStream_t st);
+                      const uint32_t *pre, uint32_t *status, uint32_t *gave_up, bool stall, bool dependent,
+                      cudaStream_t st);
 
 // Host image of the device tables.
 constexpr int kFewTables = 2 * (kMaxLg - kMinLg + 1);  // where the few-operand shapes' begin

@@ -16,7 +16,8 @@
 //   warp 19       MMAs; warps 0..3 parities and XORs
 // About 0.7 us a stage after 12 us of launches, set-up and parities: n = 300007,
 // m = 150001 31.5 us (integer transforms 47).
-// Every wait has a limit, after which the kernel records CM_FLAG_TIMEOUT and ends.
+// Every wait has a limit, after which the kernel records CM_FLAG_TIMEOUT at gave_up
+// and ends (stall, for tests: the accumulators' wait runs out).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -37,7 +38,8 @@ constexpr int kTcThreads = 20 * 32;
 
 __global__ void __launch_bounds__(kTcThreads, 1) k_gf_tc(const uint32_t *a, const uint32_t *b, uint32_t chunks, uint32_t rows, uint32_t splits, uint32_t per,
                                                          uint32_t *__restrict__ z, uint64_t m,
-                                                         const uint32_t *__restrict__ pre, uint32_t *status) {
+                                                         const uint32_t *__restrict__ pre, uint32_t *status,
+                                                         uint32_t *gave_up, bool stall) {
     extern __shared__ uint8_t raw[];
     __shared__ __align__(8) uint64_t bars[2 * kStages + 1];
     __shared__ uint32_t tmem_at;
@@ -129,7 +131,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gf_tc(const uint32_t *a, cons
             }
             commit(empty + 8 * s);
         }
-        if (ok) commit(done);
+        if (ok && !stall) commit(done);
     } else if (warp < 4 && n) {
         const bool bad = pre && (pre[0] == 0u || pre[1] == 0u);
         if (bad && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, kFlagPrecond);
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gf_tc(const uint32_t *a, cons
     if (dead) __nanosleep(1000000);  // MMAs still in flight end by themselves
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (threadIdx.x == 0 && dead) atomicOr(status, kFlagTimeout);
+    if (threadIdx.x == 0 && dead) atomicOr(gave_up, kFlagTimeout);
     if (warp == 19) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
@@ -180,13 +182,14 @@ TcShape tc_shape(uint64_t K, uint64_t m, int nsm) {
 }
 
 cudaError_t launch_tc(const TcShape &s, const uint32_t *a, const uint32_t *b, uint64_t *z, uint64_t m,
-                      const uint32_t *pre, uint32_t *status, bool dependent, cudaStream_t st) {
+                      const uint32_t *pre, uint32_t *status, uint32_t *gave_up, bool stall, bool dependent,
+                      cudaStream_t st) {
     cudaError_t e = smem_attr_once<k_gf_tc>(kSmem);
     if (e != cudaSuccess) return e;
     const uint64_t blocks = (s.rows + 255) / 256;
     return launch_after(dependent, k_gf_tc, (uint32_t)(blocks * s.splits), kTcThreads, kSmem, st, a, b, (uint32_t)s.chunks,
                         (uint32_t)s.rows, (uint32_t)s.splits, (uint32_t)s.per, reinterpret_cast<uint32_t *>(z), m, pre,
-                        status);
+                        status, gave_up, stall);
 }
 
 }  // namespace gf

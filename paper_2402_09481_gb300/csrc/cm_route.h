@@ -28,7 +28,9 @@ void gf_shape(int kind, uint64_t n, uint64_t m, gf::Product *p, gf::Ops *q);
 
 // CM_EINVAL for invalid arguments, CM_ENOMEM when no form fits `budget`.
 cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t budget, Route *r);
+// gave_up: where a bounded wait that runs out (tc) is recorded, for callers that
+// report it themselves; null: the context's status.
 cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t *y, uint64_t *z, void *scratch,
-                        cudaStream_t st);
+                        cudaStream_t st, uint32_t *gave_up = nullptr);
 
 }  // namespace cm

@@ -526,7 +526,7 @@ cm_status enqueue_wave(cm_server *S, Slot &sl, Wave &w, uint8_t *scratch, const 
     }
     if (lone) {  // a wave of one: the single call
         const WaveReq &r = w.r[0];
-        cm_status s = enqueue_route(ctx, *lone, r.d.x, r.d.y, r.d.z, scratch, sl.st);
+        cm_status s = enqueue_route(ctx, *lone, r.d.x, r.d.y, r.d.z, scratch, sl.st, dflags);
         if (s != CM_OK) return s;
         if (r.d.kind == CM_DODIS) {
             sl.pre_index[0] = 0;

@@ -42,6 +42,7 @@ PROTOTYPES = {
                            ctypes.POINTER(ctypes.c_int32)]),
     "cm_device_status": (_I, [_P, _P, ctypes.POINTER(_U32)]),
     "cm_extract_host": (_I, [_P, _I, _P, _U64, _P, _U64, _P, _P]),
+    "cm_test_stall": (_I, [_P, _I]),
     "cm_toeplitz_noalloc": (_I, [_P, _U64, _P, _U64, _P, _P]),
     "cm_field_selftest": (_I, [_I, _U64, _U64, ctypes.POINTER(_U64)]),
     "cm_batch_toeplitz_shared_seed": (_I, [_P, _P, _U64, _U64, _P, _U64, _P, _I, _P]),
@@ -604,6 +605,10 @@ class Context:
         st = ServerStats()
         _check(self._L.cm_server_get_stats(self._h, ctypes.byref(st)), "cm_server_get_stats")
         return {k: getattr(st, k) for k, _ in ServerStats._fields_ if k != "reserved"}
+
+    def test_stall(self, on: bool):
+        """Failure-path test switch (cm_test_stall)."""
+        _check(self._L.cm_test_stall(self._h, 1 if on else 0), "cm_test_stall")
 
     def device_status(self, stream=None) -> tuple[int, int]:
         f = ctypes.c_uint32(0)

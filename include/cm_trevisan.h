@@ -51,9 +51,9 @@ cm_status cm_rsh_modulus(uint32_t l, uint32_t taps[3], uint32_t *count);
  * 2 l i .. 2 l i + 2l - 1 of `seeds` (ceil(2 l m / 64) words).  2 <= l <= 256,
  * 1 <= m <= 2^32.  Scratch: ceil(n / l) chunks of ceil(l / 64) words, from
  * the context's pool; many outputs of long inputs (m >= 4096, at least 64
- * chunks, n l m >= 2^33) group the chunks where that fits the HBM budget, about
- * sqrt(n l) m / 4 + 5 n l / 8 bytes.  CM_EINVAL for bad arguments, CM_ENOMEM over
- * the HBM budget. */
+ * chunks, n l m >= 2^33) group the chunks where that fits the HBM budget and the
+ * free memory, about sqrt(n l) m / 4 + 5 n l / 8 bytes.  CM_EINVAL for bad
+ * arguments, CM_ENOMEM where the chunks alone do not fit. */
 cm_status cm_trevisan_rsh(cm_ctx *ctx, const uint64_t *x, uint64_t n, uint32_t l, const uint64_t *seeds,
                           uint64_t m, uint64_t *z, cm_stream stream);
 

@@ -748,9 +748,23 @@ static RshGroups rsh_groups(uint64_t n, uint32_t l, uint64_t m, uint64_t budget)
     return g;
 }
 
-static uint64_t rsh_scratch(uint64_t n, uint32_t l, uint64_t m, uint64_t budget) {
-    const RshGroups g = rsh_groups(n, l, m, budget);
-    return g.on ? g.bytes : rsh_chunk_bytes(n, l);
+// Scratch for the extractions (`own` bytes) with `extra` bytes behind it, from the
+// context's pool.  The grouped form's is sqrt(n l) m / 4 bytes and more, so the
+// plain form's (the chunks alone) is tried where the pool cannot give it, whatever
+// the budget says: the default budget is 80% of what was free when the context
+// was made.
+static cm_status rsh_alloc(cm_ctx *ctx, uint64_t n, uint32_t l, uint64_t m, uint64_t extra, cudaStream_t st,
+                           RshGroups *g, uint64_t *own, void **sc) {
+    if (extra > ctx->budget) return CM_ENOMEM;
+    *g = rsh_groups(n, l, m, ctx->budget - extra);
+    for (;;) {
+        *own = g->on ? g->bytes : rsh_chunk_bytes(n, l);  // multiples of 256
+        if (*own > ctx->budget - extra) return CM_ENOMEM;
+        if (cudaMallocFromPoolAsync(sc, *own + extra, ctx->pool, st) == cudaSuccess) return CM_OK;
+        cudaGetLastError();
+        if (!g->on) return CM_ENOMEM;
+        g->on = false;
+    }
 }
 
 static cm_status cuda_st(cudaError_t e) {
@@ -807,16 +821,14 @@ static cudaError_t launch_groups_w(cm_ctx *ctx, const RshGroups &g, const uint64
                            : launch_groups<W, false>(ctx, g, x, n, l, seeds, m, z, md, sc, st);
 }
 
-// Enqueue the RSH extractions; scratch holds rsh_scratch(n, l, m, budget) bytes
-// for the budget given here.
-static cm_status enqueue_rsh(cm_ctx *ctx, const uint64_t *x, uint64_t n, uint32_t l, const uint64_t *seeds,
-                             uint64_t m, uint64_t *z, uint8_t *scratch, uint64_t budget, cudaStream_t st) {
+// Enqueue the RSH extractions in the form g says; scratch as rsh_alloc gave it.
+static cm_status enqueue_rsh(cm_ctx *ctx, const RshGroups &g, const uint64_t *x, uint64_t n, uint32_t l,
+                             const uint64_t *seeds, uint64_t m, uint64_t *z, uint8_t *scratch, cudaStream_t st) {
     Modulus md;
     if (!find_modulus(l, &md) || !taps_ok(l, md)) return CM_EINVAL;
     const int W = (int)((l + 63) / 64);
     uint64_t *X = reinterpret_cast<uint64_t *>(scratch);
     cudaError_t e;
-    const RshGroups g = rsh_groups(n, l, m, budget);
     if (g.on) {
         switch (W) {
             case 1: e = launch_groups_w<1>(ctx, g, x, n, l, seeds, m, z, md, scratch, st); break;
@@ -863,16 +875,14 @@ extern "C" cm_status cm_rsh_modulus(uint32_t l, uint32_t taps[3], uint32_t *coun
 extern "C" cm_status cm_trevisan_rsh(cm_ctx *ctx, const uint64_t *x, uint64_t n, uint32_t l, const uint64_t *seeds,
                                      uint64_t m, uint64_t *z, cm_stream stream) {
     if (!ctx || !rsh_args_ok(x, n, l, seeds, m, z)) return CM_EINVAL;
-    const uint64_t need = rsh_scratch(n, l, m, ctx->budget);
-    if (need > ctx->budget) return CM_ENOMEM;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return CM_EDEVICE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     void *sc = nullptr;
-    if (cudaMallocFromPoolAsync(&sc, need, ctx->pool, st) != cudaSuccess) {
-        cudaGetLastError();
-        return CM_ENOMEM;
-    }
-    cm_status s = enqueue_rsh(ctx, x, n, l, seeds, m, z, static_cast<uint8_t *>(sc), ctx->budget, st);
+    RshGroups g;
+    uint64_t own;
+    cm_status s = rsh_alloc(ctx, n, l, m, 0, st, &g, &own, &sc);
+    if (s != CM_OK) return s;
+    s = enqueue_rsh(ctx, g, x, n, l, seeds, m, z, static_cast<uint8_t *>(sc), st);
     if (cudaFreeAsync(sc, st) != cudaSuccess && s == CM_OK) s = CM_EDEVICE;
     return s;
 }
@@ -882,27 +892,22 @@ extern "C" cm_status cm_trevisan(cm_ctx *ctx, const uint64_t *x, uint64_t n, con
                                  cm_stream stream) {
     if (!ctx || !y || !sets || d == 0 || !rsh_args_ok(x, n, l, sets, m, z) || t < 2 * l) return CM_EINVAL;
     const uint64_t sb = (2ull * l * m + 63) / 64 * 8;
-    if (sb > ctx->budget) return CM_ENOMEM;
-    const uint64_t room = ctx->budget - sb >= 256 ? ctx->budget - sb - 255 : 0;
-    const uint64_t soff = (rsh_scratch(n, l, m, room) + 255) & ~255ull;
-    const uint64_t need = soff + sb;
-    if (need > ctx->budget) return CM_ENOMEM;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return CM_EDEVICE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     void *sc = nullptr;
-    if (cudaMallocFromPoolAsync(&sc, need, ctx->pool, st) != cudaSuccess) {
-        cudaGetLastError();
-        return CM_ENOMEM;
-    }
+    RshGroups g;
+    uint64_t soff;
+    cm_status s = rsh_alloc(ctx, n, l, m, sb, st, &g, &soff, &sc);
+    if (s != CM_OK) return s;
     uint8_t *b = static_cast<uint8_t *>(sc);
     uint64_t *seeds = reinterpret_cast<uint64_t *>(b + soff);
-    cm_status s = cuda_st(cudaMemsetAsync(seeds, 0, sb, st));
+    s = cuda_st(cudaMemsetAsync(seeds, 0, sb, st));
     if (s == CM_OK) {
         ProfScope ps(ctx, "k_gather_seeds", st);
         k_gather_seeds<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(y, d, sets, t, l, m, seeds);
         s = cuda_st(cudaGetLastError());
     }
-    if (s == CM_OK) s = enqueue_rsh(ctx, x, n, l, seeds, m, z, b, room, st);
+    if (s == CM_OK) s = enqueue_rsh(ctx, g, x, n, l, seeds, m, z, b, st);
     if (cudaFreeAsync(sc, st) != cudaSuccess && s == CM_OK) s = CM_EDEVICE;
     return s;
 }

@@ -252,6 +252,7 @@ struct WaveReq {
     Plan p;
     std::vector<Block> blocks;
     uint64_t tmp_off = 0, pre_off = 0;
+    size_t foot = 0;    // what admission reserved for it
     bool solo = false;  // runs the single-call kernels (blocks) even where the work list could take it
 };
 struct Wave {
@@ -359,6 +360,7 @@ bool admit_wave(cm_server *S, Slot &sl, Wave &w) {
         w.r[i].blocks = r.blocks;
         w.r[i].tmp_off = r.tmp_off;
         w.r[i].pre_off = r.pre_off;
+        w.r[i].foot = r.foot;
         w.r[i].solo = !on_worklist(r.p);
         if (n == 1 && on_worklist(r.p) && !(r.flags & CM_REQ_SEED_CACHE)) {
             // a wave of one: the single call's kernels (one to a few launches)
@@ -566,8 +568,11 @@ cm_status launch_wave(cm_server *S, Slot &sl, Wave &w) {
     if (gf_allowed(S->ctx) && n > 1) {
         std::vector<uint32_t> by_lg[gf::kMaxLg + 1];
         for (uint32_t i = 0; i < n; ++i) {
+            // two arrays of 2^lg bits, within what admission reserved (the planner's
+            // blocks of a small budget can be smaller; such a request keeps them)
             const int lg = request_lg(w.r[i].d);
-            if (lg >= kGroupMinLg && lg <= gf::kMaxLg && !w.bext[i] && !w.make[i]) by_lg[lg].push_back(i);
+            if (lg >= kGroupMinLg && lg <= gf::kMaxLg && size_t(1) << (lg - 2) <= w.r[i].foot && !w.bext[i] && !w.make[i])
+                by_lg[lg].push_back(i);
         }
         for (int lg = gf::kMaxLg; lg >= kGroupMinLg; --lg) {
             if ((uint64_t)by_lg[lg].size() << lg < kGroupMinElements) continue;
@@ -575,7 +580,7 @@ cm_status launch_wave(cm_server *S, Slot &sl, Wave &w) {
             g.lg = lg;
             g.idx = by_lg[lg];
             g.off = total;
-            total += r256(2 * g.idx.size() << (lg - 3));  // a quarter byte a bit: within the requests' footprints
+            total += g.idx.size() << (lg - 2);
             for (uint32_t i : g.idx) grouped[i] = 1;
             groups.push_back(g);
         }

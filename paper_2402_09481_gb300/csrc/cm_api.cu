@@ -741,12 +741,12 @@ static bool one_transform(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, u
            bl[0].p.lg == kGfMinLg;
 }
 
-cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t budget, Route *r) {
+cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t budget, bool in_place, Route *r) {
     r->kind = kind;
     r->n = n;
     r->m = m;
     const uint64_t terms = (kind == CM_CIRCULANT ? n + 1 : n) + m - 1;
-    if (gf_allowed(ctx) && n - 1 < kMaxBits && m - 1 < kMaxBits && terms > 1ull << kTcMinLg &&
+    if (gf_allowed(ctx) && !in_place && n - 1 < kMaxBits && m - 1 < kMaxBits && terms > 1ull << kTcMinLg &&
         terms <= 1ull << kTcMaxLg) {
         r->shape = gf::tc_shape(terms - m + 1, m, ctx->nsm);
         if (r->shape.stages <= kTcMaxStages && valid_args(kind, n, m)) {
@@ -760,7 +760,8 @@ cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64
         }
     }
     if (gf_allowed(ctx) && n - 1 < kMaxBits && m - 1 < kMaxBits &&
-        (terms <= 1ull << gf::kDenseMaxLg || terms > 1ull << kGfMinLg || one_transform(ctx, kind, n, m, terms)) &&
+        ((terms <= 1ull << gf::kDenseMaxLg && !in_place) || terms > 1ull << kGfMinLg ||
+         one_transform(ctx, kind, n, m, terms)) &&
         valid_args(kind, n, m)) {
         if (terms <= 1ull << gf::kDenseMaxLg) {
             gf_maps(kind, n, m, &r->ops);
@@ -828,7 +829,7 @@ cm_status run_single(cm_ctx *ctx, int kind, const uint64_t *x, uint64_t n, const
                      uint64_t m, uint64_t *z, cudaStream_t st) {
     if (!ctx || !x || !y || !z) return CM_EINVAL;
     Route r;
-    cm_status s = make_route(ctx, kind, n, m, ctx->budget, &r);
+    cm_status s = make_route(ctx, kind, n, m, ctx->budget, in_place(kind, n, m, x, y, z), &r);
     if (s != CM_OK) return s;
     const uint64_t need = r.need;
     cudaError_t e = cudaSetDevice(ctx->device);
@@ -1298,7 +1299,7 @@ extern "C" cm_status cm_extract_host(cm_ctx *ctx, int kind, const uint64_t *xh, 
     const uint64_t io = 8 * (xw + yw + zw) + 4 * 256 + 255;
     if (io > ctx->budget) return CM_ENOMEM;
     Route r;
-    cm_status s = make_route(ctx, kind, n, m, ctx->budget - io, &r);
+    cm_status s = make_route(ctx, kind, n, m, ctx->budget - io, false, &r);
     if (s != CM_OK) return s;
     if (r.dense) r.need = kFlagBytes;  // Dodis et al. flags, read back below
     const uint64_t sbr = (r.need + 255) & ~255ull;

@@ -606,7 +606,7 @@ extern "C" cm_status cm_batch_create(cm_ctx *ctx, const cm_desc *descs, uint32_t
             b->solo.push_back(i);
             if (use_gf) {  // past 2^25, or a lone one of 2^22
                 Route r;
-                const cm_status rs = make_route(ctx, d.kind, d.n, d.m, ctx->budget, &r);
+                const cm_status rs = make_route(ctx, d.kind, d.n, d.m, ctx->budget, in_place(d.kind, d.n, d.m, d.x, d.y, d.z), &r);
                 if (rs != CM_OK) {
                     delete b;
                     return rs;

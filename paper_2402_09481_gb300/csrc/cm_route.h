@@ -26,8 +26,20 @@ bool gf_allowed(const cm_ctx *ctx);
 void gf_maps(int kind, uint64_t n, uint64_t m, gf::Ops *q);
 void gf_shape(int kind, uint64_t n, uint64_t m, gf::Product *p, gf::Ops *q);
 
+// z's words overlap an operand's.  The dense forms' CTAs read the operands while
+// others write z; the transforms' launches have read them before the last one
+// writes, so such calls keep to those.
+inline bool in_place(int kind, uint64_t n, uint64_t m, const uint64_t *x, const uint64_t *y, const uint64_t *z) {
+    const uint64_t yb = kind == CM_TOEPLITZ ? n + m - 1 : kind == CM_CIRCULANT ? n + 1 : n;
+    auto meets = [&](const uint64_t *p, uint64_t bits) {
+        const uintptr_t a = (uintptr_t)p, b = (uintptr_t)z;
+        return a < b + 8 * ((m + 63) / 64) && b < a + 8 * ((bits + 63) / 64);
+    };
+    return meets(x, n) || meets(y, yb);
+}
+
 // CM_EINVAL for invalid arguments, CM_ENOMEM when no form fits `budget`.
-cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t budget, Route *r);
+cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64_t budget, bool in_place, Route *r);
 // gave_up: where a bounded wait that runs out (tc) is recorded, for callers that
 // report it themselves; null: the context's status.
 cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t *y, uint64_t *z, void *scratch,

@@ -586,7 +586,8 @@ cm_status launch_wave(cm_server *S, Slot &sl, Wave &w) {
         }
     } else if (n == 1 && request_lg(w.r[0].d) <= gf::kMaxLg && !w.bext[0] && !w.make[0]) {
         const cm_desc &d = w.r[0].d;
-        if (make_route(S->ctx, d.kind, d.n, d.m, sl.foot, &route) == CM_OK && (route.dense || route.tc || route.gf)) {
+        if (make_route(S->ctx, d.kind, d.n, d.m, sl.foot, in_place(d.kind, d.n, d.m, d.x, d.y, d.z), &route) == CM_OK &&
+            (route.dense || route.tc || route.gf)) {
             if (route.dense) route.need = 256;  // its flags
             lone = &route;
             grouped[0] = 1;

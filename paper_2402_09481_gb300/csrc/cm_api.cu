@@ -789,7 +789,8 @@ cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t
         ProfScope ps(ctx, "k_gf_dense", st);
         return cuda_status(gf::launch_dense(r.ops.a0.map, r.ops.b0.map, (uint32_t)(r.kind == CM_CIRCULANT ? r.n + 1 : r.n),
                                             (uint32_t)r.m, r.kind == CM_DODIS, z, ctx->d_status,
-                                            sc ? reinterpret_cast<uint32_t *>(sc + r.pre_off) : nullptr, st));
+                                            sc && r.kind == CM_DODIS ? reinterpret_cast<uint32_t *>(sc + r.pre_off) : nullptr,
+                                            st));
     }
     if (r.tc) {
         uint32_t *a = reinterpret_cast<uint32_t *>(sc), *b = reinterpret_cast<uint32_t *>(sc + r.tmp_off), *pre = nullptr;
@@ -1296,13 +1297,14 @@ extern "C" cm_status cm_extract_host(cm_ctx *ctx, int kind, const uint64_t *xh, 
     if (!valid_args(kind, n, m)) return CM_EINVAL;
     const uint64_t ybits = kind == CM_TOEPLITZ ? n + m - 1 : (kind == CM_CIRCULANT ? n + 1 : n);
     const uint64_t xw = words_of(n), yw = words_of(ybits), zw = words_of(m);
-    const uint64_t io = 8 * (xw + yw + zw) + 4 * 256 + 255;
+    const uint64_t io = 8 * (xw + yw + zw) + 3 * 256;
     if (io > ctx->budget) return CM_ENOMEM;
     Route r;
-    cm_status s = make_route(ctx, kind, n, m, ctx->budget - io, false, &r);
+    cm_status s = make_route(ctx, kind, n, m, (ctx->budget - io) & ~255ull, false, &r);
     if (s != CM_OK) return s;
-    if (r.dense) r.need = kFlagBytes;  // Dodis et al. flags, read back below
+    if (r.dense) r.need = flag_bytes(kind);  // read back below
     const uint64_t sbr = (r.need + 255) & ~255ull;
+    if (sbr + io > ctx->budget) return CM_ENOMEM;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return CM_EDEVICE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     void *buf = nullptr;

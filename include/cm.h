@@ -276,6 +276,8 @@ typedef struct {
 
 typedef struct cm_batch cm_batch;
 
+/* solo_instances: those with L > 2^21, too long for the work list, whether they run
+ * one by one or in a group; kernel_launches: of one execution. */
 typedef struct {
     uint32_t instances, work_items, solo_instances, tile_lg, grid, graph;
     uint64_t scratch_bytes, kernel_launches, output_bits, transform_elements;

@@ -1168,6 +1168,12 @@ static uint32_t blocks_launches(const std::vector<Block> &bl) {
     return c;
 }
 
+uint32_t cm::route_launches(const Route &r) {
+    if (r.dense) return 1;
+    if (!r.tc && !r.gf) return blocks_launches(r.bl);
+    return (r.tc ? 2 : gf::product_launches(r.prod, r.ops)) + (r.kind == CM_DODIS ? 1 : 0);  // the precondition's
+}
+
 // The plan of (kind, n, m) under opt (NULL: defaults); false if invalid.
 static bool query(int kind, uint64_t n, uint64_t m, const cm_options *opt, cm_plan_info *info) {
     memset(info, 0, sizeof(*info));

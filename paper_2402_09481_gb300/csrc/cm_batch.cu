@@ -460,8 +460,7 @@ static cm_status batch_enqueue(cm_batch *b, cudaStream_t st) {
             Route &r = b->routes[i];
             cm_status s = enqueue_route(ctx, r, d.x, d.y, d.z, sc + b->off_scratch[di], st);
             if (s != CM_OK) return s;
-            b->kernel_launches += r.gf ? gf::product_launches(r.prod, r.ops) + (d.kind == CM_DODIS)
-                                       : b->plans[di].launches;
+            b->kernel_launches += route_launches(r);
             continue;
         }
         cm_status s = enqueue_extract(ctx, b->plans[di], d.x, d.y, d.z, sc + b->off_scratch[di], st);

@@ -45,4 +45,7 @@ cm_status make_route(const cm_ctx *ctx, int kind, uint64_t n, uint64_t m, uint64
 cm_status enqueue_route(cm_ctx *ctx, Route &r, const uint64_t *x, const uint64_t *y, uint64_t *z, void *scratch,
                         cudaStream_t st, uint32_t *gave_up = nullptr);
 
+// Kernel launches of a route.
+uint32_t route_launches(const Route &r);
+
 }  // namespace cm

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gf_tc(const uint32_t *a, cons
         for (uint32_t k = 0; k < n; ++k) {
             if (k + 1 < n) load(k + 1, nx);
             const uint32_t s = k % kStages, ph = (k / kStages) & 1u;
-            if (!wait(empty + 8 * s, ph ^ 1u, &dead)) break;
+            if (!wait_warp(empty + 8 * s, ph ^ 1u, &dead)) break;
             uint8_t *dst = base + s * kStageBytes + (shifts ? kInBytes : 0) + r0 * 128;
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_gf_tc(const uint32_t *a, cons
     } else if (warp < 4 && n) {
         const bool bad = pre && (pre[0] == 0u || pre[1] == 0u);
         if (bad && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(status, kFlagPrecond);
-        if (wait(done, 0, &dead)) {
+        if (wait_warp(done, 0, &dead)) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
             for (int h = 0; h < 2; ++h) {

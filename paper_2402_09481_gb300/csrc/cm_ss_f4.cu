@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kF4Threads, 1) k_ss_f4(const uint8_t *__restri
     } else if (warp < 4) {
         uint32_t acc = 0;
         for (uint64_t u = blockIdx.x; u < units; u += gridDim.x, ++acc) {
-            if (!wait(accfull, acc & 1u, &dead)) break;
+            if (!wait_warp(accfull, acc & 1u, &dead)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t pb = u % pblocks;
 #pragma unroll 1

@@ -44,6 +44,12 @@ __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity, volatile uin
     return true;
 }
 
+// The same for a warp whose lanes go on together (__syncwarp, tcgen05.ld): one answer
+// for all, so that where a wait runs out no lane stays behind in a loop the others left.
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t *dead) {
+    return __all_sync(0xFFFFFFFFu, wait(bar, parity, dead));
+}
+
 __device__ __forceinline__ void arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }

@@ -619,10 +619,12 @@ def run_batched_a(args, world, rank, local, emit=True):
     prof = ctx.profile_read(reset=True)
     ctx.profile_enable(False)
     dom = max(prof, key=lambda k: prof[k][1])
-    rate = 152 * 64 * 2070e6
+    sm_mhz = (sampler.summary(tw0, tw1) or {}).get("sm_mhz") or 2070.0
+    rate = 152 * 64 * sm_mhz * 1e6
     roof = {"bound": "alu", "kernel": dom, "achieved": ops / (ms_per_step * 1e-3) / 1e12, "peak": rate / 1e12,
             "unit": "T ALU instructions/s (lanes), whole step", "frac": ops / (ms_per_step * 1e-3) / rate,
-            "peak_source": "152 SMs x 64 ALU lanes x 2070 MHz", "avg_launch_ms": prof[dom][1] / prof[dom][0],
+            "peak_source": f"152 SMs x 64 ALU lanes x {sm_mhz:.0f} MHz (sampled)",
+            "avg_launch_ms": prof[dom][1] / prof[dom][0],
             "traffic": ncu_traffic(dom, "batched_a") if count == 4096 else None,
             "hbm": {"bytes": io, "achieved": io / (ms_per_step * 1e-3) / 1e9, "peak": peak,
                     "peak_source": f"{peak_src} HBM copy bandwidth (MEASURED_PEAKS.json)"},
@@ -1743,7 +1745,7 @@ def run_single(args, world, rank, local, dist):
     }
 
 
-def dodis_extra(local, steps=5):
+def dodis_extra(local, sm_mhz, steps=5):
     """The Dodis et al. workload (n = 1073741789, m = floor(0.4 n)), Bernoulli(1/2)
     sources and a second run with x 0.8-biased (drawn on the device: timing
     only; the tests check this run's bits against the oracle)."""
@@ -1784,7 +1786,7 @@ def dodis_extra(local, steps=5):
         st, fl = ctx.device_status()
         assert st == native.CM_OK, native.STATUS.get(st)
         ms_ = statistics.median(ts)
-        pr = binary_roofline(2, n, n, m, ms_, 2070.0, peak)
+        pr = binary_roofline(2, n, n, m, ms_, sm_mhz, peak)
         out[name] = {"ms_per_step": ms_, "value": m / (ms_ * 1e-3) / 1e9, "unit": "Gbit/s",
                      "path_roofline_frac": pr["frac"], "t_alu_ms": pr["t_alu_ms"], "t_hbm_ms": pr["t_hbm_ms"]}
     ctx.close()
@@ -1848,7 +1850,7 @@ def main():
     if (line is not None and world == 1 and args.workload == "circulant" and args.field == "auto"
             and not args.no_extras):
         t0 = time.time()
-        line["dodis"] = dodis_extra(local)
+        line["dodis"] = dodis_extra(local, (line.get("clocks") or {}).get("sm_mhz") or 2070.0)
         sub = argparse.Namespace(**vars(args))
         sub.steps, sub.warmup, sub.no_cpu_baseline = 3, 3, True
         ba = run_batched_a(sub, 1, 0, local, emit=False)

@@ -10,9 +10,10 @@
  * product's length) is exact: q = 5 * 2^25 + 1 with lazy reduction for
  * transforms up to 2^25, the paper's own q = 3 * 2^30 + 1 (Section
  * "Performance") up to 2^30, and Goldilocks p = 2^64 - 2^32 + 1 up to 2^32.
- * Long single calls and batches of a context with default options work on the
- * bits themselves instead: the same product over GF(2), by additive transforms
- * of binary polynomials.  The choice changes speed, never a result bit.
+ * A context with default options works on the bits themselves at most lengths
+ * instead: the same product over GF(2), by additive transforms of binary
+ * polynomials where it is long, densely where it is short or the tensor cores hold
+ * it (cm_options.field).  The choice changes speed, never a result bit.
  *
  * Conventions shared by every entry point
  * ---------------------------------------
@@ -80,11 +81,14 @@ typedef struct {
      * smaller fields to one longer transform); CM_FIELD_Q30 skips the field of
      * 5 * 2^25 + 1; CM_FIELD_GOLDILOCKS takes Goldilocks throughout.  Results
      * are identical.  Under CM_FIELD_AUTO, with max_transform_lg,
-     * max_sum_blocks and plan_mode at their defaults too, single calls with
-     * K + m - 1 > 2^23 (above 2^22: where the planner has one transform) and batch
-     * instances with K + m - 1 > 2^14, where a length has enough of them, run as
-     * binary polynomials (when that form's scratch fits the budget).  The work list of
-     * batches and the server runs over 5 * 2^25 + 1. */
+     * max_sum_blocks and plan_mode at their defaults too, single calls run by
+     * their number of terms T = K + m - 1: T <= 2^13 densely in one launch;
+     * 2^17 < T <= 2^22 densely on the tensor cores while no multiprocessor's
+     * share is longer than 40 stages of 256 terms; T > 2^23 (above 2^22: where
+     * the planner has one transform of 2^23) as binary polynomials; the others,
+     * those whose scratch does not fit the budget, and those whose z lies over x
+     * or y at the dense lengths, by integer transforms.  Batches: cm_batch_create.
+     * The work list of batches and the server runs over 5 * 2^25 + 1. */
     uint32_t field;
     /* Most input blocks whose transform-domain products are summed before one
      * inverse transform; 0 = as many as keep every count below the field's
@@ -287,14 +291,16 @@ typedef struct {
  * Plan a batch of `count` extractions of any mix of kinds (the paper has no
  * batched form; each instance computes exactly what its single call computes).
  * Instances with 2^14 < L <= 2^25 run as binary polynomials, the instances of
- * one length together in each launch, when the context's options leave the
- * form to the library (cm_options.field).  Shorter ones (all up to 2^21 in
- * other contexts and under CM_BATCH_TEST_STALL) run in ONE persistent kernel
- * launch that walks a work list: an instance with L <= 2^13 is one item, a
+ * one length together in each launch, where the batch holds at least 2^21 (L up
+ * to 2^16), 2^22 (2^18) or 2^23 elements of that length and the context's options
+ * leave the form to the library (cm_options.field).  The others up to 2^21 (all of
+ * them in other contexts and under CM_BATCH_TEST_STALL) run in ONE persistent
+ * kernel launch that walks a work list: an instance with L <= 2^13 is one item, a
  * larger one is split into forward column-pass tiles, fused middle rows,
  * inverse tiles with parity, and pack chunks, each item starting once the
  * items it depends on are done (bounded waits; CM_FLAG_TIMEOUT if one runs
- * out).  Longer instances run the single calls' kernels after it.
+ * out).  Longer instances outside the groups run the single calls' kernels after
+ * it, one by one.
  * Scratch for every instance is allocated here (cudaMalloc, held until
  * cm_batch_destroy); CM_ENOMEM if it exceeds the context budget.  With
  * CM_BATCH_AUTOTUNE the candidate column-pass tiles (2^14 and 2^13 elements)
@@ -414,7 +420,8 @@ typedef struct {
  * machinery) and longer ones through the integer single-call planner, on the
  * slot's stream; with the context's options at their defaults (see
  * cm_options.field) those of 2^18 .. 2^25, where one length has 2^22 elements or
- * more, run as binary polynomials instead, one group of launches a length.  A
+ * more, run as binary polynomials instead, one group of launches a length, as far
+ * as the scratch they were admitted with holds them.  A
  * wave of one request up to 2^25 runs what its single call runs.  Waves on
  * different streams overlap on the device; each stream has two slots, so the
  * next wave is enqueued behind the running one.  Express slots (high stream
@@ -501,9 +508,10 @@ uint64_t cm_prev_na_prime(uint64_t n);
 
 /* How the integer transforms run (kind, n, m) under the given options (the
  * planner described at cm_toeplitz).  The server plans every request this way;
- * single calls and batches do where they do not take the binary form (see
- * cm_options.field), whose scratch is smaller: a quarter byte per transform
- * bit, half a byte where blocks are summed. */
+ * single calls and batches do where they take none of the other forms (see
+ * cm_options.field), whose scratch is smaller: binary polynomials a quarter byte
+ * per transform bit, half a byte where blocks are summed; the tensor-core form
+ * both operands' bits; the one-launch form none. */
 typedef struct {
     uint64_t transform_length; /* the longest product's transform length L */
     uint64_t products;         /* middle products: input blocks x output windows */

@@ -724,7 +724,7 @@ constexpr int kGfMinLg = 23;
 // Products of 2^17 .. 2^22 terms run densely on the tensor cores (cm_gf2_tc.cu)
 // while their longest chain of stages beats the transforms.  Measured, us a call,
 // integer transforms / dense (K x m: stages): 100000 x 50000: 3, 43 / 25; 300007 x
-// 150001: 24, 47 / 31.5; 349525 x 174762: 36, 47 / 39; 30000 x 2000000: 40, 66 / 35;
+// 150001: 24, 47 / 29.4; 349525 x 174762: 36, 47 / 39; 30000 x 2000000: 40, 66 / 35;
 // 2000000 x 20000: 52, 66 / 53; 450000 x 400000: 84, 50 / 101.
 constexpr int kTcMinLg = 17, kTcMaxLg = 22;
 constexpr uint64_t kTcMaxStages = 40;

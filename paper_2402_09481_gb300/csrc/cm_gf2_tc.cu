@@ -1,5 +1,6 @@
-// One extraction of 2^17 .. about 2^19.5 terms as a dense product on the 5th-
-// generation tensor cores.
+// One extraction as a dense product on the 5th-generation tensor cores: 2^17 .. 2^22
+// terms, while the longest chain of stages leaves it ahead of the transforms (to about
+// 2^19.2 terms where K and m are alike, further for a short or a narrow product).
 //
 // z_(224 c + i) = sum_u b_(u + 224 c) a_(u - i), i < 224: a product of two bit
 // matrices, rows of windows of b 224 apart and rows of shifts of a, whose outputs
@@ -15,7 +16,7 @@
 //   warps 12..18  a's shifts (224 rows): funnel shifts
 //   warp 19       MMAs; warps 0..3 parities and XORs
 // About 0.7 us a stage after 12 us of launches, set-up and parities: n = 300007,
-// m = 150001 31.5 us (integer transforms 47).
+// m = 150001 29.4 us (integer transforms 47).
 // Every wait has a limit, after which the kernel records CM_FLAG_TIMEOUT at gave_up
 // and ends (stall, for tests: the accumulators' wait runs out).
 #include <cuda_runtime.h>

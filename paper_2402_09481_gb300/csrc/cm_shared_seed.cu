@@ -349,7 +349,10 @@ k_ss_bmma(const uint32_t *__restrict__ T, uint32_t rows_pad, uint32_t words_pad,
 // CM_ENGINE_AUTO takes the tcgen05 engine for this many bit products or more.
 // Measured, us a call, CUDA cores / tcgen05 (n x m x count): 4096 x 2048 x 65536
 // 1309 / 232, 8000 x 6000 x 300 169 / 44, 4096 x 2048 x 300 59 / 28, 1000 x 300 x
-// 4096 (2^30.2) 22.3 / 16.6; below, either is launch latency.
+// 4096 (2^30.2) 22.3 / 16.6; below, either is launch latency.  So it is however few
+// the inputs or the rows: 16384 x 65536 x 1 (a 512 MB matrix) 2708 / 270 and x 64
+// 2753 / 283, 4096 x 4096 x 64 76 / 35, 1024 x 1024 x 1024 31.8 / 24.2, 4096 x 64 x
+// 16384 42.9 / 32.2; over 208 shapes from 2^30 to 2^37 the ratio was 0.07 to 0.76.
 constexpr double kSsF4Min = 1073741824.0;
 
 std::mutex g_engine_mu;

@@ -1,6 +1,6 @@
 """Trevisan's one-bit step where the grouped form's scratch fits the context's budget
 but not the memory that is free when the call is made: the plain form runs.  In a
-process of its own: the driver would serve the call from what other contexts'
+process of its own: CUDA would serve the call from what other contexts'
 pools hold unused in this one."""
 
 import os
